@@ -49,7 +49,7 @@ __host__ __device__ __forceinline__ T proj_threshold(T delta) {
 }
 
 template <typename T, int DIM>
-__device__ __forceinline__ PtK<T> make_ptk(const Phys<T>& P, T h) {
+__host__ __device__ __forceinline__ PtK<T> make_ptk(const Phys<T>& P, T h) {
   PtK<T> K;
   const T ih = T(1) / h;
   K.ih2 = ih * ih;

@@ -25,6 +25,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <atomic>
 #include <cmath>
 #include <new>
 
@@ -33,6 +34,7 @@
 #include "fm_stepper.cuh"
 #include "fm_zmarch.cuh"
 #include "fm_coop.cuh"
+#include "fm_cluster.cuh"
 
 namespace fm {
 
@@ -924,9 +926,10 @@ struct Solver {
 
   // One V-cycle from level l down; *out_in_r: on return the correction of
   // level l is in its r buffer (1) or in e (0).
-  // The V-cycle of the small levels S (each of at most SMALL_N points) in
-  // one block: shared memory when they fit, else global memory.
+  // The float32 V-cycle of the small levels S (each of at most SMALL_N
+  // points) in one block: shared memory when they fit, else global memory.
   static int small_cycle(fm_state* st, const SmallLv<T>& S, const Phys<T>& P) {
+    static_assert(sizeof(T) == 4, "float64: cluster_cycle");
     cudaStream_t s = st->stream;
     SmallSmem<T> M;
     const size_t smem = small_layout<T, KIND, DIM>(S, M, SMALL_SMEM_MAX);
@@ -941,6 +944,51 @@ struct Solver {
                                                                     st->prm.ncoarse);
     } else {
       k_vcycle_small<T, KIND, DIM><<<1, SMALL_TPB, 0, s>>>(S, P, st->prm.nu1, st->prm.nu2, st->prm.ncoarse);
+    }
+    FM_LAUNCHED();
+    return FM_OK;
+  }
+
+  // The float64 V-cycle of the small levels from l down by one cluster
+  // (fm_cluster.cuh), on the levels of the state in their own precision T.
+  static int cluster_cycle(fm_state* st, int l) {
+    SmallLv<T> S;
+    double h[MAXSMALL];
+    S.count = st->nlev - l;
+    for (int q = 0; q < S.count; ++q) {
+      S.lv[q] = make_lvl<T>(st, l + q);
+      h[q] = st->lv[l + q].h;
+    }
+    const Phys<double> P = make_phys<double>(st);
+    const auto kernel = k_vcycle_cluster<T, KIND, DIM>;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {(unsigned)CL_MAX, 1, 1};
+    cfg.blockDim = dim3(CL_TPB);
+    cfg.stream = st->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ClPlan M;
+    static std::atomic<int> size{0};  // blocks of the cluster: 16, or 8 (the portable size) where 16 do not fit
+    int nb = size.load();
+    if (!nb) {
+      FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX));
+      FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cfg.gridDim = dim3(CL_MAX);
+      cfg.dynamicSmemBytes = CL_SMEM_MAX;
+      int n = 0;
+      nb = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1 ? CL_MAX : 8;
+      cudaGetLastError();
+      size.store(nb);
+    }
+    cfg.gridDim = dim3(nb);
+    attr[0].val.clusterDim = {(unsigned)nb, 1, 1};
+    cfg.dynamicSmemBytes = cl_plan<T, KIND, DIM>(S, P, h, nb, M);
+    if (cfg.dynamicSmemBytes > CL_SMEM_MAX) return FM_EINVAL;
+    if (cudaLaunchKernelEx(&cfg, kernel, S, M, P, st->prm.nu1, st->prm.nu2, st->prm.ncoarse) != cudaSuccess) {
+      cudaGetLastError();
+      return FM_ECUDA;
     }
     FM_LAUNCHED();
     return FM_OK;
@@ -992,16 +1040,15 @@ struct Solver {
     return FM_OK;
   }
 
-  // The coarsest-grid solve in float64 (mixed path): the coarse levels from
-  // l down on their float64 copies -- the single-block V-cycle, or the
-  // coarsest level's ncoarse sweeps as colour launches -- between the two
-  // conversions.
+  // The coarsest-grid solve in float64 (mixed path): the V-cycle of the
+  // levels from l down by one cluster, or a larger coarsest level's ncoarse
+  // sweeps as colour launches on its float64 copy between two conversions.
   static int coarse_solve64(fm_state* st, int l) {
+    if (!st->coarse_fused) return cluster_cycle(st, l);
     int rc = coarse_to64(st, l);
     if (rc) return rc;
     const Phys<double> P64 = make_phys<double>(st);
-    int in_r = 0;
-    if (st->coarse_fused) {
+    {
       // colour launches of 32-thread blocks: the float64 point updates of a
       // small level spread over all multiprocessors (GB300 issues few float64
       // operations per multiprocessor and clock)
@@ -1023,14 +1070,8 @@ struct Solver {
           }
           FM_LAUNCHED();
         }
-    } else {
-      SmallLv<double> S;
-      S.count = st->nlev - l;
-      for (int q = 0; q < S.count; ++q) S.lv[q] = make_lvl_bufs<double>(st->lv64[l + q]);
-      rc = Solver<double, KIND, DIM>::small_cycle(st, S, P64);
     }
-    if (rc) return rc;
-    return coarse_from64(st, l, in_r);
+    return coarse_from64(st, l, 0);
   }
 
   static int vcycle(fm_state* st, int l, const Phys<T>& P, int* out_in_r) {
@@ -1043,10 +1084,14 @@ struct Solver {
       return smooth(st, l, P, st->prm.ncoarse, out_in_r);
     }
     if (l >= st->small_from) {
-      SmallLv<T> S;
-      S.count = st->nlev - l;
-      for (int q = 0; q < S.count; ++q) S.lv[q] = make_lvl<T>(st, l + q);
-      return small_cycle(st, S, P);
+      if constexpr (sizeof(T) == 8) {
+        return cluster_cycle(st, l);
+      } else {
+        SmallLv<T> S;
+        S.count = st->nlev - l;
+        for (int q = 0; q < S.count; ++q) S.lv[q] = make_lvl<T>(st, l + q);
+        return small_cycle(st, S, P);
+      }
     }
     // The correction of level l may sit in its r buffer between the pre- and
     // the post-smoothing (after an odd number of fused launches); the
@@ -1249,7 +1294,7 @@ static size_t carve(fm_state* st, char* base) {
   // prolongation reads it; a multi-block coarsest level's r[0] holds the
   // CDFT chemical-potential parts of its colour launches)
   for (int l = 0; l < MAXLEV; ++l) st->lv64[l] = LevelBufs{};
-  if (st->coarse64) {
+  if (st->coarse64 && st->coarse_fused) {
     for (int l = st->small_from; l < st->nlev; ++l) {
       LevelBufs& B = st->lv64[l];
       B.g = st->lv[l].g;
