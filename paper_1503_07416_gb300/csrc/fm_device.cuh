@@ -2324,42 +2324,53 @@ static __global__ void k_hist_advance(Ctl* ctl) {
 // block (cycles += in_body) and, in graph mode, sets the WHILE condition:
 // continue while the norm is finite, above tol and cycles < max_cycles.
 // Block-level body: thread 0 returns whether the instance continues.
+//
+// One block between two launches of every cycle, so its latency counts in
+// full, and on GB300 that is the length of its chain of float64 instructions:
+// warp q sums component q (its partials in four running sums a lane, then
+// shuffles), thread 0 takes one square root, of the largest weighted sum
+// (sqrt is monotone, so it is the largest of the square roots), and the
+// control block is read before the sums are known.
 template <int NQ>
 __device__ __forceinline__ bool norm_ctl_body(const double* partials, int nblk, double w, Ctl* ctl, double tol,
                                               int max_cycles, int in_body) {
-  double v[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += TPB)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) v[q] += partials[b * NQ + q];
-  __shared__ double sm[NQ][TPB / 32];
+  static_assert(NQ <= TPB / 32, "one warp per component");
+  __shared__ double sm[NQ];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int fault = 0, nonpos = 0, done = 0;
+  if (threadIdx.x == 0) {
+    fault = ctl->fault;
+    nonpos = ctl->nonpos;
+    done = ctl->cycles;
+  }
+  if (warp < NQ) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = lane; b < nblk; b += 128)
 #pragma unroll
-  for (int q = 0; q < NQ; ++q)
-    for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) sm[q][warp] = v[q];
+      for (int k = 0; k < 4; ++k)
+        if (b + 32 * k < nblk) v[k] += partials[(b + 32 * k) * NQ + warp];
+    double x = (v[0] + v[1]) + (v[2] + v[3]);
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+    if (lane == 0) sm[warp] = w * x;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double mx = 0.0;
     bool finite = true;
+#pragma unroll
     for (int q = 0; q < NQ; ++q) {
-      double x = 0.0;
-      for (int ww = 0; ww < TPB / 32; ++ww) x += sm[q][ww];
-      const double nq = sqrt(w * x);
-      if (!(nq == nq) || isinf(nq)) finite = false;
-      mx = fmax(mx, nq);
+      const double x = sm[q];
+      if (!(x == x) || isinf(x)) finite = false;
+      mx = fmax(mx, x);
     }
-    const double nrm = finite ? mx : NAN;
-    int cycles = in_body ? ctl->cycles + 1 : 0;
+    const double nrm = finite ? sqrt(mx) : NAN;
+    const int cycles = in_body ? done + 1 : 0;
     ctl->cycles = cycles;
     ctl->norm = nrm;
     if (!in_body) ctl->norm0 = nrm;
     int status = FM_OK;
-    if (ctl->fault) status = FM_ETIMEOUT;
-    else if (ctl->nonpos) status = FM_ENONPOS;
+    if (fault) status = FM_ETIMEOUT;
+    else if (nonpos) status = FM_ENONPOS;
     else if (!finite) status = FM_ENAN;
     else if (nrm > tol && cycles >= max_cycles) status = FM_ENOCONV;
     ctl->status = status;
