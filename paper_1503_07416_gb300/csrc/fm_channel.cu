@@ -15,7 +15,7 @@
 // The same scheme and solver as fm_solver.cu otherwise: float64 outer
 // residual, FAS V-cycles on the correction equation in precision T, the
 // hydrodynamic point block (smooth_point_a) evaluated through an accessor
-// that returns the ghost values, red and black launches per sweep, the
+// that returns the ghost values, the fused level kernels of fm_fused.cuh, the
 // coarsest level smoothed ncoarse times; the transfers are nodal in x and
 // cell-centred in y (a coarse cell is two fine cells: restriction and
 // injection average them, prolongation interpolates linearly between cell
@@ -26,6 +26,7 @@
 #include "fm_state.h"
 #include "fm_device.cuh"
 #include "fm_stepper.cuh"
+#include "fm_fused.cuh"
 
 namespace fm {
 namespace ch {
@@ -86,19 +87,28 @@ struct WallsT {
   T ub, ut;
 };
 
+// The injected correction and the coefficients of coarse level C, the
+// correction read from the fine level (the mean of rows 2J and 2J + 1 at 2I).
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_ch_smooth(Lvl<T> L, Phys<T> P, WallsT<T> W, int color) {
-  int i, j, k;
-  if (!colour_point(blockIdx.x * blockDim.x + threadIdx.x, color, L.g, i, j, k)) return;
-  ChAcc<T> a{L, W.ub, W.ut};
-  const Nb n = ch_neighbours(i, j, L.g);
-  smooth_point_a<T, KPFC, 2>(a, P, make_ptk<T, 2>(P, L.h), n, n.c);
-}
+struct ChInjAcc {
+  const Lvl<T>& F;
+  ChAcc<T> c;
+  __device__ __forceinline__ T e(int q, int i) const {
+    const int m = cell_of(i, c.L.g.N), nx = c.L.g.nx;
+    const int a = 2 * (m / nx) * F.g.nx + 2 * (m % nx);
+    const T v = T(0.5) * (F.e[q][a] + F.e[q][a + F.g.nx]);
+    return (i < 0 && (q == 1 || q == 2)) ? -v : v;
+  }
+  __device__ __forceinline__ T rk(int i) const { return c.rk(i); }
+  __device__ __forceinline__ T cr(int i) const { return c.cr(i); }
+  __device__ __forceinline__ T cv(int d, int i) const { return c.cv(d, i); }
+  __device__ __forceinline__ T om(int d, int i) const { return c.om(d, i); }
+};
 
 // M(e) = N(c + e) - N(c) at one cell, through the accessor (App. G.2 operator
 // in correction form, as applyM of the periodic solver).
-template <typename T>
-__device__ __forceinline__ void ch_applyM(const ChAcc<T>& a, const Phys<T>& P, T h, const Nb& n, T* M) {
+template <typename T, class A>
+__device__ __forceinline__ void ch_applyM(const A& a, const Phys<T>& P, T h, const Nb& n, T* M) {
   const T ih = T(1) / h, ih2 = ih * ih;
   const int c = n.c;
   const T rkc = a.rk(c);
@@ -136,31 +146,11 @@ __device__ __forceinline__ void ch_applyM(const ChAcc<T>& a, const Phys<T>& P, T
   M[LY::IKA] = ek - (nbr - T(4) * er) * ih2;
 }
 
-// r = f - M(e) on a level (out = L.r), or f += M(e) (coarse right-hand side).
-template <typename T, bool RHS>
-__global__ void __launch_bounds__(TPB) k_ch_resid(Lvl<T> L, Phys<T> P, WallsT<T> W) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= L.g.N) return;
-  const int i = idx % L.g.nx, j = idx / L.g.nx;
-  ChAcc<T> a{L, W.ub, W.ut};
-  T M[LY::NU], fv[LY::NU];
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) fv[q] = L.f[q][idx];
-  ch_applyM<T>(a, P, L.h, ch_neighbours(i, j, L.g), M);
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) {
-    if (RHS) L.f[q][idx] = fv[q] + M[q];
-    else L.r[q][idx] = fv[q] - M[q];
-  }
-}
-
-// Coarse cell (I, J) of fine rows 2J, 2J + 1: f_C = R(r_F) (x full weighting
+// Coarse cell idx of fine rows 2J, 2J + 1: f_C = R(r_F) (x full weighting
 // about 2I, y the mean of the two rows), e_C = eh_C = the injection (the
 // mean of the two cells at x = 2I).
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_ch_restrict(Lvl<T> F, Lvl<T> C) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= C.g.N) return;
+__device__ __forceinline__ void ch_restrict(const Lvl<T>& F, const Lvl<T>& C, int idx) {
   const int I = idx % C.g.nx, J = idx / C.g.nx;
   const int x = 2 * I, xm = x == 0 ? F.g.nx - 1 : x - 1, xp = x + 1 == F.g.nx ? 0 : x + 1;
   const int r0 = 2 * J * F.g.nx, r1 = r0 + F.g.nx;
@@ -179,32 +169,46 @@ __global__ void __launch_bounds__(TPB) k_ch_restrict(Lvl<T> F, Lvl<T> C) {
   }
 }
 
-// Coefficients of level F injected into level C (same averaging): rho^k and
-// omega^k (which = 0) or the coefficient iterate rho, u, v (which = 1).
+// Coefficients of the finest level injected into every coarser level, one
+// launch: a level's value is the mean of the two fine cells of the level
+// above at x = 2I, so level l takes the pairwise means over 2^l rows, eight
+// rows loaded at a time.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_ch_inject(Lvl<T> F, Lvl<T> C, int which) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= C.g.N) return;
-  const int I = idx % C.g.nx, J = idx / C.g.nx;
-  const int a = 2 * J * F.g.nx + 2 * I, b = a + F.g.nx;
-  if (which == 0) {
-    const_cast<T*>(C.rk)[idx] = T(0.5) * (F.rk[a] + F.rk[b]);
-    const_cast<T*>(C.om[0])[idx] = T(0.5) * (F.om[0][a] + F.om[0][b]);
-  } else {
-    const_cast<T*>(C.cr)[idx] = T(0.5) * (F.cr[a] + F.cr[b]);
-    const_cast<T*>(C.cv[0])[idx] = T(0.5) * (F.cv[0][a] + F.cv[0][b]);
-    const_cast<T*>(C.cv[1])[idx] = T(0.5) * (F.cv[1][a] + F.cv[1][b]);
+__global__ void __launch_bounds__(TPB) k_ch_inject_all(const __grid_constant__ InjAll<T> A) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= A.off[A.nl]) return;
+  int l = 1;
+  while (t >= A.off[l + 1]) ++l;
+  const int idx = t - A.off[l], I = idx % A.g[l].nx, J = idx / A.g[l].nx;
+  const int nx = A.g0.nx, nb = (1 << l) >= 8 ? (1 << l) / 8 : 1, step = (1 << l) >= 8 ? 8 : 1 << l;
+  for (int q = 0; q < A.nsrc; ++q) {
+    const T* src = A.src[q] + (size_t)(J << l) * nx + (I << l);
+    T part[MAXLEV];  // part[k]: the mean of 8 2^k rows waiting for its pair
+    T v = T(0);
+    for (int b = 0; b < nb; ++b, src += (size_t)8 * nx) {
+      T r[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) r[k] = k < step ? src[(size_t)k * nx] : T(0);
+#pragma unroll
+      for (int w = 1; w < 8; w *= 2)
+        if (w < step)
+#pragma unroll
+          for (int k = 0; k < 8; k += 2 * w) r[k] = T(0.5) * (r[k] + r[k + w]);
+      v = r[0];
+      int k = 0;
+      for (int n = b; n & 1; n >>= 1, ++k) v = T(0.5) * (part[k] + v);
+      part[k] = v;
+    }
+    A.dst[l][q][idx] = v;
   }
 }
 
-// e_F += P(e_C - eh_C): x linear between nodes, y linear between cell
-// centres (3/4 the own coarse cell, 1/4 the next one towards the fine cell),
-// the coarse correction's ghost beyond a wall mirrored (scalars) or odd
-// (velocity).
+// Fine cell idx: e_F += P(e_C - eh_C): x linear between nodes, y linear
+// between cell centres (3/4 the own coarse cell, 1/4 the next one towards the
+// fine cell), the coarse correction's ghost beyond a wall mirrored (scalars)
+// or odd (velocity).
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_ch_prolong(Lvl<T> F, Lvl<T> C) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= F.g.N) return;
+__device__ __forceinline__ void ch_prolong(const Lvl<T>& F, const Lvl<T>& C, int idx) {
   const int i = idx % F.g.nx, j = idx / F.g.nx;
   const int J = j >> 1;
   const int Jn = (j & 1) ? J + 1 : J - 1;
@@ -224,6 +228,49 @@ __global__ void __launch_bounds__(TPB) k_ch_prolong(Lvl<T> F, Lvl<T> C) {
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) F.e[q][idx] = ev[q];
 }
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_ch_prolong(Lvl<T> F, Lvl<T> C) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < F.g.N) ch_prolong(F, C, idx);
+}
+
+// Policy of the fused 2-D kernels (fm_fused.cuh).
+template <typename TT>
+struct ChPol {
+  using T = TT;
+  using K = PtK<T>;
+  using W = WallsT<T>;
+  static constexpr int NU = LY::NU, NC = 4;
+  static constexpr bool WALLS = true;
+  __host__ __device__ static K constants(const Phys<T>& P, T h) { return make_ptk<T, 2>(P, h); }
+  __device__ static const T* coef(const Lvl<T>& L, int c) {
+    return c == 0 ? L.cr : (c == 1 ? L.rk : L.cv[c - 2]);
+  }
+  // a staged ghost cell, from the wall row's values (p: its element of the first array)
+  __device__ static void ghost(T* p, int SN, bool top, const W& w) {
+    p[SN] = -p[SN];
+    p[2 * SN] = -p[2 * SN];
+    p[(NU + 2) * SN] = T(2) * (top ? w.ut : w.ub) - p[(NU + 2) * SN];
+    p[(NU + 3) * SN] = -p[(NU + 3) * SN];
+  }
+  template <class A>
+  __device__ static void update(const A& a, const Phys<T>& P, const K& k, const Nb& n, int fc) {
+    smooth_point_a<T, KPFC, 2>(a, P, k, n, fc);
+  }
+  __device__ static void update_lvl(const Lvl<T>& L, const Phys<T>& P, const K& k, const W& w, int i, int j) {
+    const Nb n = ch_neighbours(i, j, L.g);
+    smooth_point_a<T, KPFC, 2>(ChAcc<T>{L, w.ub, w.ut}, P, k, n, n.c);
+  }
+  __device__ static void apply(const Lvl<T>& F, const Phys<T>& P, const K&, const W& w, int x, int y, T* M) {
+    ch_applyM<T>(ChAcc<T>{F, w.ub, w.ut}, P, F.h, ch_neighbours(x, y, F.g), M);
+  }
+  __device__ static void apply_coarse(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, const K&, const W& w, int I,
+                                      int J, T* M) {
+    ch_applyM<T>(ChInjAcc<T>{F, ChAcc<T>{C, w.ub, w.ut}}, P, C.h, ch_neighbours(I, J, C.g), M);
+  }
+  __device__ static void restrict_lvl(const Lvl<T>& F, const Lvl<T>& C, int i) { ch_restrict(F, C, i); }
+  __device__ static void prolong_lvl(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>&, int i) { ch_prolong(F, C, i); }
+};
 
 // ---------------------------------------------------------------------------
 // float64 kernels of the finest level
@@ -429,12 +476,27 @@ struct ChannelSolver {
     return O;
   }
 
+  // rho^k and omega^k (which = 0) or the coefficient iterate rho, u, v
+  // (which = 1) of the finest level down the hierarchy.
   static int inject(fm_state* st, int which) {
-    for (int l = 0; l + 1 < st->nlev; ++l) {
-      const Lvl<T> F = make_lvl<T>(st, l), C = make_lvl<T>(st, l + 1);
-      k_ch_inject<T><<<nblocks(C.g.N), TPB, 0, st->stream>>>(F, C, which);
-      FM_LAUNCHED();
+    if (st->nlev < 2) return FM_OK;
+    InjAll<T> A;
+    memset(&A, 0, sizeof(A));
+    A.nl = st->nlev;
+    A.g0 = st->lv[0].g;
+    A.nsrc = which ? 3 : 2;
+    for (int l = 0; l < st->nlev; ++l) {
+      const LevelBufs& B = st->lv[l];
+      void* v[3] = {which ? B.cr : B.rk, which ? B.cv[0] : B.om[0], B.cv[1]};
+      for (int q = 0; q < A.nsrc; ++q) {
+        if (l == 0) A.src[q] = (const T*)v[q];
+        else A.dst[l][q] = (T*)v[q];
+      }
+      A.g[l] = B.g;
+      A.off[l + 1] = l == 0 ? 0 : A.off[l] + B.g.N;
     }
+    k_ch_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
+    FM_LAUNCHED();
     return FM_OK;
   }
 
@@ -465,43 +527,48 @@ struct ChannelSolver {
     return FM_OK;
   }
 
-  static int smooth(fm_state* st, const Lvl<T>& L, const Phys<T>& P, int iters) {
-    for (int it = 0; it < iters; ++it)
-      for (int color = 0; color < 2; ++color) {
-        k_ch_smooth<T><<<nblocks(L.g.N / 2), TPB, 0, st->stream>>>(L, P, wallsT(st), color);
-        FM_LAUNCHED();
-      }
-    return FM_OK;
-  }
-
-  static int vcycle(fm_state* st, int l, const Phys<T>& P) {
+  // *out_in_r: on return the correction of level l is in its r buffer (1) or in e (0).
+  static int vcycle(fm_state* st, int l, const Phys<T>& P, int* out_in_r) {
+    using Pol = ChPol<T>;
     cudaStream_t s = st->stream;
-    const Lvl<T> F = make_lvl<T>(st, l);
-    if (l == st->nlev - 1) return smooth(st, F, P, st->prm.ncoarse);
-    int rc = smooth(st, F, P, st->prm.nu1);
-    if (rc) return rc;
+    const WallsT<T> W = wallsT(st);
+    *out_in_r = 0;
+    if (l >= fz_small_from<T>(st)) {
+      SmallLv<T> S;
+      S.count = st->nlev - l;
+      for (int q = 0; q < S.count; ++q) S.lv[q] = make_lvl<T>(st, l + q);
+      FM_CUDA(fz_small<Pol>(S, P, W, st->prm, &st->launches, s));
+      return FM_OK;
+    }
+    const Lvl<T> L = make_lvl<T>(st, l);
+    if (l == st->nlev - 1) {
+      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, s));
+      return FM_OK;
+    }
     const Lvl<T> C = make_lvl<T>(st, l + 1);
-    k_ch_resid<T, false><<<nblocks(F.g.N), TPB, 0, s>>>(F, P, wallsT(st));
-    FM_LAUNCHED();
-    k_ch_restrict<T><<<nblocks(C.g.N), TPB, 0, s>>>(F, C);
-    FM_LAUNCHED();
-    k_ch_resid<T, true><<<nblocks(C.g.N), TPB, 0, s>>>(C, P, wallsT(st));
-    FM_LAUNCHED();
-    rc = vcycle(st, l + 1, P);
+    int c_in_r = 0;
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, s));
+    const Lvl<T> F = fz_view(L, *out_in_r);
+    FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
+    const int rc = vcycle(st, l + 1, P, &c_in_r);
     if (rc) return rc;
-    k_ch_prolong<T><<<nblocks(F.g.N), TPB, 0, s>>>(F, C);
+    k_ch_prolong<T><<<nblocks(F.g.N), TPB, 0, s>>>(F, fz_view(C, c_in_r));
     FM_LAUNCHED();
-    return smooth(st, F, P, st->prm.nu2);
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
+    return FM_OK;
   }
 
   static int enqueue_body(fm_state* st, cudaGraphConditionalHandle hdl, int use_handle) {
     int rc = inject(st, 1);
     if (rc) return rc;
-    rc = vcycle(st, 0, make_phys<T>(st));
+    int in_r = 0;
+    rc = vcycle(st, 0, make_phys<T>(st), &in_r);
     if (rc) return rc;
     const Geo G = st->lv[0].g;
-    k_update64<LY::NU, T><<<nblocks(G.N), TPB, 0, st->stream>>>(make_fields(st), out0(st, true, nullptr), G.N,
-                                                                st->prm.delta);
+    Resid64Out O = out0(st, true, nullptr);
+    if (in_r)  // the correction after an odd number of launches
+      for (int q = 0; q < LY::NU; ++q) O.e0[q] = st->lv[0].r[q];
+    k_update64<LY::NU, T><<<nblocks(G.N), TPB, 0, st->stream>>>(make_fields(st), O, G.N, st->prm.delta);
     FM_LAUNCHED();
     return enqueue_resid_norm(st, 1, hdl, use_handle);
   }

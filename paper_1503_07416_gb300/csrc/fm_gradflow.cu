@@ -33,6 +33,7 @@
 #include "fm_state.h"
 #include "fm_device.cuh"
 #include "fm_stepper.cuh"
+#include "fm_fused.cuh"
 
 namespace fm {
 namespace gf {
@@ -53,7 +54,7 @@ struct GK {
 };
 
 template <typename T, int DIM>
-__device__ __forceinline__ GK<T> make_gk(const Phys<T>& P, T h) {
+__host__ __device__ __forceinline__ GK<T> make_gk(const Phys<T>& P, T h) {
   GK<T> K;
   K.ih2 = T(1) / (h * h);
   K.c = T(2 * DIM) * K.ih2;
@@ -63,46 +64,48 @@ __device__ __forceinline__ GK<T> make_gk(const Phys<T>& P, T h) {
   return K;
 }
 
-// Correction-form chemical potential of CDFT at idx: ln(c + e) - ln c + 2 c_e e.
-template <typename T>
-__device__ __forceinline__ T mcorr_gf(const T* e, const T* c, int idx, T ce) {
-  const T x = e[idx];
-  return log1p_t(x / c[idx]) + T(2) * ce * x;
+// Sum of a value over the neighbours.
+template <int DIM, class F>
+__device__ __forceinline__ auto nb_sum(const Nb& n, F&& v) {
+  auto s = v(n.m[0]) + v(n.p[0]) + v(n.m[1]) + v(n.p[1]);
+  if constexpr (DIM == 3) s += v(n.m[2]) + v(n.p[2]);
+  return s;
 }
 
-// M(e) = N(c + e) - N(c) at one point (all components).
-template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void gf_applyM(const Lvl<T>& L, const Phys<T>& P, const GK<T>& K, const Nb& n, T* M) {
+// M(e) = N(c + e) - N(c) at one point (all components), written against an
+// accessor of e(q, i) and the coefficient density cr(i).
+template <typename T, int KIND, int DIM, class A>
+__device__ __forceinline__ void gf_applyM(const A& a, const Phys<T>& P, const GK<T>& K, const Nb& n, T* M) {
+  auto nbs = [&](int q) { return nb_sum<DIM>(n, [&](int i) { return a.e(q, i); }); };
   if constexpr (KIND == KPFC) {
-    const T er = L.e[0][n.c], em = L.e[1][n.c], ek = L.e[2][n.c];
-    const T psi = L.cr[n.c] - T(1.5);
-    M[0] = er + K.a * em - K.sih2 * nbsum<T, DIM>(L.e[1], n);
-    M[1] = em - er * (psi * psi + psi * er + er * er * T(1.0 / 3.0)) - P.alpha * er + K.c * ek
-         - K.ih2 * nbsum<T, DIM>(L.e[2], n);
-    M[2] = ek + K.c * er - K.ih2 * nbsum<T, DIM>(L.e[0], n);
+    const T er = a.e(0, n.c), em = a.e(1, n.c), ek = a.e(2, n.c);
+    const T psi = a.cr(n.c) - T(1.5);
+    M[0] = er + K.a * em - K.sih2 * nbs(1);
+    M[1] = em - er * (psi * psi + psi * er + er * er * T(1.0 / 3.0)) - P.alpha * er + K.c * ek - K.ih2 * nbs(2);
+    M[2] = ek + K.c * er - K.ih2 * nbs(0);
   } else {
-    T sm = mcorr_gf(L.e[0], L.cr, n.m[0], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[0], P.ce)
-         + mcorr_gf(L.e[0], L.cr, n.m[1], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[1], P.ce);
-    if constexpr (DIM == 3) sm += mcorr_gf(L.e[0], L.cr, n.m[2], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[2], P.ce);
-    M[0] = L.e[0][n.c] + K.a * mcorr_gf(L.e[0], L.cr, n.c, P.ce) - K.sih2 * sm;
+    auto mc = [&](int i) { return cdft_mc<T>(a.e(0, i), a.cr(i), P.ce); };
+    M[0] = a.e(0, n.c) + K.a * mc(n.c) - K.sih2 * nb_sum<DIM>(n, mc);
   }
 }
 
-// Point-block update of one point (see the file comment), projection, damping.
-template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void gf_smooth_point(const Lvl<T>& L, const Phys<T>& P, const GK<T>& K, const Nb& n) {
+// Point-block update of one point (see the file comment), projection, damping;
+// the right-hand side is read at index fc.
+template <typename T, int KIND, int DIM, class A>
+__device__ __forceinline__ void gf_smooth_point(const A& a, const Phys<T>& P, const GK<T>& K, const Nb& n, int fc) {
   const int c = n.c;
-  const T crc = L.cr[c];
+  const T crc = a.cr(c);
   const T w = P.w;
+  auto nbs = [&](int q) { return nb_sum<DIM>(n, [&](int i) { return a.e(q, i); }); };
   if constexpr (KIND == KPFC) {
-    const T eo0 = L.e[0][c], eo1 = L.e[1][c], eo2 = L.e[2][c];
-    const T b1 = L.f[0][c] + K.sih2 * nbsum<T, DIM>(L.e[1], n);
-    const T b3 = L.f[2][c] + K.ih2 * nbsum<T, DIM>(L.e[0], n);
+    const T eo0 = a.e(0, c), eo1 = a.e(1, c), eo2 = a.e(2, c);
+    const T b1 = a.f(0, fc) + K.sih2 * nbs(1);
+    const T b3 = a.f(2, fc) + K.ih2 * nbs(0);
     const T psc = crc - T(1.5);
     const T p = psc + eo0;                                                  // current psi
     const T cub = eo0 * (psc * psc + psc * eo0 + eo0 * eo0 * T(1.0 / 3.0));  // [(psc+e)^3 - psc^3]/3
     const T q = p * p + P.alpha;
-    const T b2 = L.f[1][c] + K.ih2 * nbsum<T, DIM>(L.e[2], n) + cub - p * p * eo0;
+    const T b2 = a.f(1, fc) + K.ih2 * nbs(2) + cub - p * p * eo0;
     const T qc = q + K.c * K.c;
     const T em = (b2 + qc * b1 - K.c * b3) * rcp_blk(T(1) + K.a * qc);
     T er = b1 - K.a * em;
@@ -111,15 +114,13 @@ __device__ __forceinline__ void gf_smooth_point(const Lvl<T>& L, const Phys<T>& 
       if (x <= K.proj) er = sqrt_t(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
     }
     const T ek = b3 - K.c * er;
-    L.e[0][c] = (T(1) - w) * er + w * eo0;
-    L.e[1][c] = (T(1) - w) * em + w * eo1;
-    L.e[2][c] = (T(1) - w) * ek + w * eo2;
+    a.set_e(0, c, (T(1) - w) * er + w * eo0);
+    a.set_e(1, c, (T(1) - w) * em + w * eo1);
+    a.set_e(2, c, (T(1) - w) * ek + w * eo2);
   } else {
-    const T eo = L.e[0][c];
-    T sm = mcorr_gf(L.e[0], L.cr, n.m[0], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[0], P.ce)
-         + mcorr_gf(L.e[0], L.cr, n.m[1], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[1], P.ce);
-    if constexpr (DIM == 3) sm += mcorr_gf(L.e[0], L.cr, n.m[2], P.ce) + mcorr_gf(L.e[0], L.cr, n.p[2], P.ce);
-    const T b = L.f[0][c] + K.sih2 * sm;
+    const T eo = a.e(0, c);
+    auto mc = [&](int i) { return cdft_mc<T>(a.e(0, i), a.cr(i), P.ce); };
+    const T b = a.f(0, fc) + K.sih2 * nb_sum<DIM>(n, mc);
     // one Newton step on e + a (log1p(e/c) + 2 c_e e) = b about the current e
     const T F = eo + K.a * (log1p_t(eo / crc) + T(2) * P.ce * eo) - b;
     const T dF = T(1) + K.a * (T(1) / (crc + eo) + T(2) * P.ce);
@@ -128,15 +129,61 @@ __device__ __forceinline__ void gf_smooth_point(const Lvl<T>& L, const Phys<T>& 
       const T x = crc + en;
       if (x <= K.proj) en = sqrt_t(x * x + P.delta * P.delta) - crc;
     }
-    L.e[0][c] = (T(1) - w) * en + w * eo;
+    a.set_e(0, c, (T(1) - w) * en + w * eo);
   }
 }
+
+template <typename T>
+__device__ __forceinline__ LvlAcc<T> lvl_acc(const Lvl<T>& L) { return LvlAcc<T>{L, L.f, L.om}; }
+
+// Policy of the fused 2-D kernels (fm_fused.cuh).
+struct GfW {};
+template <typename TT, int KIND>
+struct GfPol {
+  using T = TT;
+  using K = GK<T>;
+  using W = GfW;
+  static constexpr int NU = GL<KIND>::NU, NC = 1;
+  static constexpr bool WALLS = false;
+  __host__ __device__ static K constants(const Phys<T>& P, T h) { return make_gk<T, 2>(P, h); }
+  __device__ static const T* coef(const Lvl<T>& L, int) { return L.cr; }
+  template <class A>
+  __device__ static void update(const A& a, const Phys<T>& P, const K& k, const Nb& n, int fc) {
+    gf_smooth_point<T, KIND, 2>(a, P, k, n, fc);
+  }
+  __device__ static void update_lvl(const Lvl<T>& L, const Phys<T>& P, const K& k, const W&, int i, int j) {
+    const Nb n = neighbours(i, j, 0, L.g);
+    gf_smooth_point<T, KIND, 2>(lvl_acc(L), P, k, n, n.c);
+  }
+  __device__ static void apply(const Lvl<T>& F, const Phys<T>& P, const K& k, const W&, int x, int y, T* M) {
+    gf_applyM<T, KIND, 2>(lvl_acc(F), P, k, neighbours(x, y, 0, F.g), M);
+  }
+  // every coarse coefficient is the injection of the fine one: M_C at (I, J)
+  // on the fine arrays at 2I, 2J and two points beside them
+  __device__ static void apply_coarse(const Lvl<T>& F, const Lvl<T>&, const Phys<T>& P, const K& kc, const W&, int I,
+                                      int J, T* M) {
+    const int nx = F.g.nx, ny = F.g.ny, x = 2 * I, y = 2 * J;
+    Nb n;
+    n.c = y * nx + x;
+    n.m[0] = n.c + (x == 0 ? nx - 2 : -2);
+    n.p[0] = n.c + (x + 2 >= nx ? 2 - nx : 2);
+    n.m[1] = n.c + (y == 0 ? (ny - 2) * nx : -2 * nx);
+    n.p[1] = n.c + (y + 2 >= ny ? (2 - ny) * nx : 2 * nx);
+    n.m[2] = n.p[2] = n.c;
+    gf_applyM<T, KIND, 2>(lvl_acc(F), P, kc, n, M);
+  }
+  __device__ static void restrict_lvl(const Lvl<T>& F, const Lvl<T>& C, int i) { restrict_point<T, NU, 2>(F, C, i); }
+  __device__ static void prolong_lvl(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int i) {
+    prolong_point<T, NU, 2>(F, C, P, i);
+  }
+};
 
 template <typename T, int KIND, int DIM>
 __global__ void __launch_bounds__(TPB) k_gf_smooth(Lvl<T> L, Phys<T> P, int color) {
   int i, j, k;
   if (!colour_point(blockIdx.x * blockDim.x + threadIdx.x, color, L.g, i, j, k)) return;
-  gf_smooth_point<T, KIND, DIM>(L, P, make_gk<T, DIM>(P, L.h), neighbours(i, j, k, L.g));
+  const Nb n = neighbours(i, j, k, L.g);
+  gf_smooth_point<T, KIND, DIM>(lvl_acc(L), P, make_gk<T, DIM>(P, L.h), n, n.c);
 }
 
 // r = f - M(e) on a level.
@@ -150,7 +197,7 @@ __global__ void __launch_bounds__(TPB) k_gf_resid(Lvl<T> L, Phys<T> P) {
   T M[NU], fv[NU];
 #pragma unroll
   for (int q = 0; q < NU; ++q) fv[q] = L.f[q][idx];
-  gf_applyM<T, KIND, DIM>(L, P, make_gk<T, DIM>(P, L.h), neighbours(i, j, k, L.g), M);
+  gf_applyM<T, KIND, DIM>(lvl_acc(L), P, make_gk<T, DIM>(P, L.h), neighbours(i, j, k, L.g), M);
 #pragma unroll
   for (int q = 0; q < NU; ++q) L.r[q][idx] = fv[q] - M[q];
 }
@@ -173,7 +220,7 @@ __global__ void __launch_bounds__(TPB) k_gf_coarse_rhs(Lvl<T> C, Phys<T> P) {
   T M[NU], fv[NU];
 #pragma unroll
   for (int q = 0; q < NU; ++q) fv[q] = C.f[q][idx];
-  gf_applyM<T, KIND, DIM>(C, P, make_gk<T, DIM>(P, C.h), neighbours(i, j, k, C.g), M);
+  gf_applyM<T, KIND, DIM>(lvl_acc(C), P, make_gk<T, DIM>(P, C.h), neighbours(i, j, k, C.g), M);
 #pragma unroll
   for (int q = 0; q < NU; ++q) C.f[q][idx] = fv[q] + M[q];
 }
@@ -408,6 +455,39 @@ struct GFSolver {
     return FM_OK;
   }
 
+  // 2-D: the fused level kernels (fm_fused.cuh).  *out_in_r: on return the
+  // correction of level l is in its r buffer (1) or in e (0).
+  static int vcycle2(fm_state* st, int l, const Phys<T>& P, int* out_in_r) {
+    using Pol = GfPol<T, KIND>;
+    cudaStream_t s = st->stream;
+    const GfW W;
+    *out_in_r = 0;
+    if (l >= fz_small_from<T>(st)) {
+      SmallLv<T> S;
+      S.count = st->nlev - l;
+      for (int q = 0; q < S.count; ++q) S.lv[q] = make_lvl<T>(st, l + q);
+      FM_CUDA(fz_small<Pol>(S, P, W, st->prm, &st->launches, s));
+      return FM_OK;
+    }
+    const Lvl<T> L = make_lvl<T>(st, l);
+    if (l == st->nlev - 1) {
+      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, s));
+      return FM_OK;
+    }
+    const Lvl<T> C = make_lvl<T>(st, l + 1);
+    int c_in_r = 0;
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, s));
+    const Lvl<T> F = fz_view(L, *out_in_r);
+    FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
+    const int rc = vcycle2(st, l + 1, P, &c_in_r);
+    if (rc) return rc;
+    k_gf_prolong<T, NU, 2><<<nblocks(F.g.N), TPB, 0, s>>>(F, fz_view(C, c_in_r), P);
+    FM_LAUNCHED();
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
+    return FM_OK;
+  }
+
+  // 3-D: a launch per colour and transfer.
   static int vcycle(fm_state* st, int l, const Phys<T>& P) {
     cudaStream_t s = st->stream;
     const Lvl<T> F = make_lvl<T>(st, l);
@@ -451,14 +531,19 @@ struct GFSolver {
   static int enqueue_body(fm_state* st, cudaGraphConditionalHandle hdl, int use_handle) {
     int rc = inject_coefficient(st);
     if (rc) return rc;
-    rc = vcycle(st, 0, make_phys<T>(st));
+    int in_r = 0;
+    if constexpr (DIM == 2) rc = vcycle2(st, 0, make_phys<T>(st), &in_r);
+    else rc = vcycle(st, 0, make_phys<T>(st));
     if (rc) return rc;
     const Geo G = st->lv[0].g;
+    Resid64Out O = out0(st, true, nullptr);
+    if (in_r)  // the correction after an odd number of launches
+      for (int q = 0; q < NU; ++q) O.e0[q] = st->lv[0].r[q];
     Fields64 F;
     memset(&F, 0, sizeof(F));
     for (int q = 0; q < NU; ++q) F.g[q] = st->g[q];
     F.nonpos = KIND == KCDFT ? &static_cast<Ctl*>(st->ctl)->nonpos : nullptr;
-    k_update64<NU, T><<<nblocks(G.N), TPB, 0, st->stream>>>(F, out0(st, true, nullptr), G.N, st->prm.delta);
+    k_update64<NU, T><<<nblocks(G.N), TPB, 0, st->stream>>>(F, O, G.N, st->prm.delta);
     FM_LAUNCHED();
     return enqueue_resid_norm(st, 1, hdl, use_handle);
   }
