@@ -51,6 +51,155 @@ struct ClDim {
   static constexpr int SETS = CL_TPB / 32 / R;             // warps of each role in a block
 };
 
+// --------------------------------------------------------------------------
+// The point update by roles
+// --------------------------------------------------------------------------
+// The point a thread updates: its index, its neighbours' indices and records.
+template <int DIM>
+struct RolePt {
+  int idx;  // -1: none
+  int ni[2 * DIM];
+  const double* nr[2 * DIM];  // m, p of each direction
+};
+// What role 0 carries from the first half of an update to the second.
+struct RoleRegs {
+  double er, cub;
+};
+
+// smooth_point_a's update of the point t in slot p of a pass, split over the
+// roles; a block barrier between the halves.  An accessor A gives rk(i),
+// cr(i), cv(d, i), f(q, i), the point's own record recp(i) and velocity-block
+// inverse ivp(i), keep_mc(i, e0, ce), and xch(k, p): value k of slot p in the
+// exchange area (0 .. DIM - 1 velocity right-hand sides, DIM and DIM + 1 the
+// kappa and mu sums).  Every value of another point is loaded before the first
+// use, so that remote reads overlap.
+template <int KIND, int DIM>
+struct RoleUpdate {
+  using D = ClDim<KIND, DIM>;
+  using LY = Layout<KIND, DIM>;
+  static constexpr int AUX = 1 + DIM;
+
+  static __device__ __forceinline__ double sum(const double (&v)[2 * DIM]) {
+    double s = v[0] + v[1];
+#pragma unroll
+    for (int k = 2; k < 2 * DIM; ++k) s += v[k];
+    return s;
+  }
+
+  template <class A>
+  static __device__ __forceinline__ void first(const A& a, const Phys<double>& P, const PtK<double>& K,
+                                               const RolePt<DIM>& t, int p, int role, RoleRegs& g) {
+    if (role == 0) {
+      double u[2 * DIM], r[2 * DIM];
+#pragma unroll
+      for (int k = 0; k < 2 * DIM; ++k) {
+        u[k] = t.nr[k][1 + k / 2];
+        r[k] = a.rk(t.ni[k]);
+      }
+      const double crc = a.cr(t.idx), f0 = a.f(0, t.idx);
+      double div = 0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) div += r[2 * d + 1] * u[2 * d + 1] - r[2 * d] * u[2 * d];
+      double er = f0 - K.c_div * div;
+      const double x = crc + er;
+      if (x <= K.proj) er = sqrt(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
+      if constexpr (KIND == KPFC) {
+        const double psi = crc - 1.5;
+        g.cub = er * (psi * psi + psi * er + er * er * (1.0 / 3.0)) + P.alpha * er;
+      }
+      g.er = er;
+    } else if (role == AUX) {
+      if constexpr (KIND == KPFC) {
+        double v[2 * DIM], k2[2 * DIM];
+#pragma unroll
+        for (int k = 0; k < 2 * DIM; ++k) {
+          v[k] = t.nr[k][0];
+          k2[k] = t.nr[k][LY::IKA];
+        }
+        a.xch(DIM, p) = a.f(LY::IKA, t.idx) + sum(v) * K.ih2;
+        a.xch(DIM + 1, p) = a.f(LY::IMU, t.idx) + sum(k2) * K.ih2;
+      }
+    } else {
+#pragma unroll
+      for (int d = 0; d < DIM; ++d)
+        if (role == 1 + d) {
+          double v[2 * DIM], q[2], m[2], c[2][DIM], u[2][DIM];
+#pragma unroll
+          for (int k = 0; k < 2 * DIM; ++k) v[k] = t.nr[k][1 + d];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            m[k] = t.nr[2 * d + k][KIND == KPFC ? LY::IMU : D::NR - 1];
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) {
+              u[k][b] = t.nr[2 * d + k][1 + b];
+              c[k][b] = a.cv(b, t.ni[2 * d + k]);
+            }
+          }
+          const double fd = a.f(1 + d, t.idx), cs = K.c_sih * a.rk(t.idx);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            q[k] = 0;
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) q[k] += u[k][b] * (2.0 * c[k][b] + u[k][b]);
+          }
+          a.xch(d, p) = fd - cs * (0.25 * (q[1] - q[0]) + 0.5 * (m[1] - m[0])) + K.c_v * sum(v);
+        }
+    }
+  }
+
+  template <class A>
+  static __device__ __forceinline__ void second(const A& a, const Phys<double>& P, const PtK<double>& K,
+                                                const RolePt<DIM>& t, int p, int role, const RoleRegs& g) {
+    const double w = P.w;
+    double* eo = a.recp(t.idx);
+    if (role == 0) {
+      if constexpr (KIND == KPFC) {
+        const double c4 = 2.0 * DIM * K.ih2;
+        const double ek = a.xch(DIM, p) - c4 * g.er;
+        const double em = a.xch(DIM + 1, p) + g.cub - c4 * ek;
+        eo[LY::IKA] = (1.0 - w) * ek + w * eo[LY::IKA];
+        eo[LY::IMU] = (1.0 - w) * em + w * eo[LY::IMU];
+      }
+      const double er = (1.0 - w) * g.er + w * eo[0];
+      eo[0] = er;
+      if constexpr (KIND == KCDFT) a.keep_mc(t.idx, er, P.ce);
+    } else if (role <= DIM) {
+      const double* v = a.ivp(t.idx);
+      double eg;
+      if constexpr (DIM == 2)
+        eg = role == 1 ? v[0] * a.xch(0, p) + v[1] * a.xch(1, p) : v[0] * a.xch(1, p) - v[1] * a.xch(0, p);
+      else
+        eg = v[3 * role - 3] * a.xch(0, p) + v[3 * role - 2] * a.xch(1, p) + v[3 * role - 1] * a.xch(2, p);
+      eo[role] = (1.0 - w) * eg + w * eo[role];
+    }
+  }
+};
+
+// The inverse of the velocity block at a point (see smooth_point_a).
+template <int DIM>
+__device__ __forceinline__ void invert_block(const PtK<double>& K, double rk, const double* om, double* v) {
+  const double Ad = rk + K.c_ad, bs = K.c_b * rk;
+  if constexpr (DIM == 2) {
+    const double b = bs * om[0], inv = 1.0 / (Ad * Ad + b * b);
+    v[0] = Ad * inv;
+    v[1] = b * inv;
+  } else {
+    const double b[3] = {bs * om[0], bs * om[1], bs * om[2]};
+    const double inv = 1.0 / (Ad * (Ad * Ad + b[0] * b[0] + b[1] * b[1] + b[2] * b[2]));
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        // Ad^2 I - Ad [b]_x + b b^T, [b]_x rhs = b x rhs
+        const double x = r == c ? Ad * Ad : ((c - r + 3) % 3 == 1 ? Ad : -Ad) * b[3 - r - c];
+        v[3 * r + c] = (x + b[r] * b[c]) * inv;
+      }
+  }
+}
+
+// --------------------------------------------------------------------------
+// The V-cycle of the small levels by a cluster
+// --------------------------------------------------------------------------
 // Shared-memory offsets (doubles) and constants of the levels; the same in
 // every block.  Block r owns the points [r << sh, (r + 1) << sh) of a level.
 struct ClPlan {
@@ -123,11 +272,12 @@ struct ClAcc {
   __device__ __forceinline__ double cr(int i) const { return L.co[L.g.N + i]; }
   __device__ __forceinline__ double cv(int d, int i) const { return L.co[(2 + d) * L.g.N + i]; }
   __device__ __forceinline__ double om(int d, int i) const { return L.co[(2 + DIM + d) * L.g.N + i]; }
+  __device__ __forceinline__ double* recp(int i) const { return L.rec + own(i) * D::NR; }
+  __device__ __forceinline__ const double* ivp(int i) const { return L.iv + own(i) * D::NV; }
+  __device__ __forceinline__ double& xch(int k, int p) const { return L.rhs[(k << (L.sh - 1)) + p]; }
   // the chemical-potential part of point i's current correction (CDFT)
-  __device__ __forceinline__ double keep_mc(int i, double e0, double ce) const {
-    const double m = cdft_mc<double>(e0, cr(i), ce);
-    L.rec[own(i) * D::NR + D::NR - 1] = m;
-    return m;
+  __device__ __forceinline__ void keep_mc(int i, double e0, double ce) const {
+    recp(i)[D::NR - 1] = cdft_mc<double>(e0, cr(i), ce);
   }
   __device__ __forceinline__ double nbs(int q, const Nb& n) const {
     double s = e(q, n.m[0]) + e(q, n.p[0]) + e(q, n.m[1]) + e(q, n.p[1]);
@@ -162,6 +312,8 @@ struct ClCycle {
   using D = ClDim<KIND, DIM>;
   using LY = Layout<KIND, DIM>;
   using Acc = ClAcc<KIND, DIM>;
+  using Up = RoleUpdate<KIND, DIM>;
+  using Pt = RolePt<DIM>;
   static constexpr int NU = D::NU;
 
   // fn(idx, p, role) for this block's points by the warps of each role; p
@@ -195,33 +347,13 @@ struct ClCycle {
     const int n = 1 << L.sh, first = (int)cl_rank() << L.sh;
     for (int p = threadIdx.x; p < n && first + p < L.g.N; p += CL_TPB) {
       const int i = first + p;
-      const double Ad = a.rk(i) + K.c_ad, bs = K.c_b * a.rk(i);
-      double* v = L.iv + p * D::NV;
-      if constexpr (DIM == 2) {
-        const double b = bs * a.om(0, i), inv = 1.0 / (Ad * Ad + b * b);
-        v[0] = Ad * inv;
-        v[1] = b * inv;
-      } else {
-        const double b[3] = {bs * a.om(0, i), bs * a.om(1, i), bs * a.om(2, i)};
-        const double inv = 1.0 / (Ad * (Ad * Ad + b[0] * b[0] + b[1] * b[1] + b[2] * b[2]));
+      double om[LY::NOM];
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            // Ad^2 I - Ad [b]_x + b b^T, [b]_x rhs = b x rhs
-            const double x = r == c ? Ad * Ad : ((c - r + 3) % 3 == 1 ? Ad : -Ad) * b[3 - r - c];
-            v[3 * r + c] = (x + b[r] * b[c]) * inv;
-          }
-      }
+      for (int d = 0; d < LY::NOM; ++d) om[d] = a.om(d, i);
+      invert_block<DIM>(K, a.rk(i), om, L.iv + p * D::NV);
     }
   }
 
-  // The point of one colour a thread updates: neighbours' indices and records.
-  struct Pt {
-    int idx;  // -1: none
-    int ni[2 * DIM];
-    const double* nr[2 * DIM];  // m, p of each direction
-  };
   static __device__ __forceinline__ Pt point(const ClLvl& L, int p, int c) {
     Pt t;
     t.idx = -1;
@@ -242,103 +374,13 @@ struct ClCycle {
     for (int k = 0; k < 2 * DIM; ++k) t.nr[k] = a.rec(t.ni[k]);
     return t;
   }
-  static __device__ __forceinline__ double sum(const double (&v)[2 * DIM]) {
-    double s = v[0] + v[1];
-#pragma unroll
-    for (int k = 2; k < 2 * DIM; ++k) s += v[k];
-    return s;
-  }
-
-  // One colour pass over this block's points: slot p of `half` slots, role.
-  // Every value of another point is loaded before the first use, so that the
-  // remote reads overlap.
   static __device__ __forceinline__ void pass(const ClLvl& L, const Phys<double>& P, const PtK<double>& K,
                                               const Pt& t, int p, int role) {
-    constexpr int AUX = 1 + DIM;
     const Acc a{L};
-    const int half = L.sh - 1;
-    const double w = P.w;
-    double* eo = L.rec + (t.idx < 0 ? 0 : a.own(t.idx) * D::NR);
-    double er = 0, psi = 0, cub = 0;
-    if (t.idx >= 0) {
-      if (role == 0) {
-        double u[2 * DIM], r[2 * DIM];
-#pragma unroll
-        for (int k = 0; k < 2 * DIM; ++k) {
-          u[k] = t.nr[k][1 + k / 2];
-          r[k] = a.rk(t.ni[k]);
-        }
-        const double crc = a.cr(t.idx), f0 = a.f(0, t.idx);
-        double div = 0;
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) div += r[2 * d + 1] * u[2 * d + 1] - r[2 * d] * u[2 * d];
-        er = f0 - K.c_div * div;
-        const double x = crc + er;
-        if (x <= K.proj) er = sqrt(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
-        if constexpr (KIND == KPFC) {
-          psi = crc - 1.5;
-          cub = er * (psi * psi + psi * er + er * er * (1.0 / 3.0)) + P.alpha * er;
-        }
-      } else if (KIND == KPFC && role == AUX) {
-        double v[2 * DIM], k2[2 * DIM];
-#pragma unroll
-        for (int k = 0; k < 2 * DIM; ++k) {
-          v[k] = t.nr[k][0];
-          k2[k] = t.nr[k][LY::IKA];
-        }
-        L.rhs[(DIM << half) + p] = a.f(LY::IKA, t.idx) + sum(v) * K.ih2;
-        L.rhs[((DIM + 1) << half) + p] = a.f(LY::IMU, t.idx) + sum(k2) * K.ih2;
-      } else {
-#pragma unroll
-        for (int d = 0; d < DIM; ++d)
-          if (role == 1 + d) {
-            double v[2 * DIM], q[2], m[2], c[2][DIM], u[2][DIM];
-#pragma unroll
-            for (int k = 0; k < 2 * DIM; ++k) v[k] = t.nr[k][1 + d];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              m[k] = t.nr[2 * d + k][KIND == KPFC ? LY::IMU : D::NR - 1];
-#pragma unroll
-              for (int b = 0; b < DIM; ++b) {
-                u[k][b] = t.nr[2 * d + k][1 + b];
-                c[k][b] = a.cv(b, t.ni[2 * d + k]);
-              }
-            }
-            const double fd = a.f(1 + d, t.idx), cs = K.c_sih * a.rk(t.idx);
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              q[k] = 0;
-#pragma unroll
-              for (int b = 0; b < DIM; ++b) q[k] += u[k][b] * (2.0 * c[k][b] + u[k][b]);
-            }
-            L.rhs[(d << half) + p] = fd - cs * (0.25 * (q[1] - q[0]) + 0.5 * (m[1] - m[0])) + K.c_v * sum(v);
-          }
-      }
-    }
+    RoleRegs g;
+    if (t.idx >= 0) Up::first(a, P, K, t, p, role, g);
     __syncthreads();
-    if (t.idx >= 0) {
-      const double* h = L.rhs + p;
-      if (role == 0) {
-        if constexpr (KIND == KPFC) {
-          const double c4 = 2.0 * DIM * K.ih2;
-          const double ek = h[DIM << half] - c4 * er;
-          const double em = h[(DIM + 1) << half] + cub - c4 * ek;
-          eo[LY::IKA] = (1.0 - w) * ek + w * eo[LY::IKA];
-          eo[LY::IMU] = (1.0 - w) * em + w * eo[LY::IMU];
-        }
-        er = (1.0 - w) * er + w * eo[0];
-        eo[0] = er;
-        if constexpr (KIND == KCDFT) a.keep_mc(t.idx, er, P.ce);
-      } else if (role <= DIM) {
-        const double* v = L.iv + a.own(t.idx) * D::NV;
-        double eg;
-        if constexpr (DIM == 2)
-          eg = role == 1 ? v[0] * h[0] + v[1] * h[1 << half] : v[0] * h[1 << half] - v[1] * h[0];
-        else
-          eg = v[3 * role - 3] * h[0] + v[3 * role - 2] * h[1 << half] + v[3 * role - 1] * h[2 << half];
-        eo[role] = (1.0 - w) * eg + w * eo[role];
-      }
-    }
+    if (t.idx >= 0) Up::second(a, P, K, t, p, role, g);
     cl_sync();
   }
 
@@ -524,6 +566,137 @@ __global__ void __launch_bounds__(CL_TPB) k_vcycle_cluster(const __grid_constant
   for (int t = threadIdx.x; t < n0 * NU; t += CL_TPB) {
     const int p = t & (n0 - 1), q = t >> L0.sh;
     if (first + p < L0.g.N) S.lv[0].e[q][first + p] = to_t<TS>(L0.rec[p * D::NR + q]);
+  }
+}
+
+// --------------------------------------------------------------------------
+// Sweeps of a larger 2-D coarsest level
+// --------------------------------------------------------------------------
+// NS (1 or 2) red-black sweeps in float64 of a float32 level on 8 x 4 tiles,
+// one tile a block, the point updates by roles: red on the tile and its rings
+// 2 NS - 1, black one ring less, and so on, as in the tile form of the fused
+// sweeps.  The tile and its halo are widened as they are staged (integer
+// conversions); the correction is read from ein (float32 or float64) and the
+// tile's is written to eout (another buffer).  The launch is bound by the
+// float64 pipe: 70, 48, 30 and 16 points a pass for two sweeps, so 3, 2, 1
+// and 1 warps of each role; smaller tiles recompute more than the idle
+// multiprocessors give, larger ones leave multiprocessors without a tile (a
+// 64^2 level has 128 tiles).  Two sweeps of a 64^2 level, kernel time: 12 us
+// (PFC) and 15 us (CDFT) against 32 and 37 us for four colour launches between
+// two conversions.
+constexpr int CT_TX = 8, CT_TY = 4, CT_SETS = 3;
+// Largest level swept on tiles: two tiles a multiprocessor.  Beyond it the
+// recomputed halo (2.6 point updates for one) costs more than the launches.
+constexpr int CT_MAXN = 8192;
+
+template <int KIND>
+__host__ __device__ constexpr int ct_threads() { return ClDim<KIND, 2>::R * CT_SETS * 32; }
+
+template <int KIND, int NS>
+struct CtSmem {
+  static constexpr int H = 2 * NS, SW = CT_TX + 2 * H, SN = SW * (CT_TY + 2 * H);
+  using D = ClDim<KIND, 2>;
+  double rec[SN * D::NR], iv[SN * D::NV], co[4][SN], f[D::NU][SN], x[4][CT_SETS * 32];
+};
+
+template <int KIND, int NS>
+struct CtAcc {
+  using D = ClDim<KIND, 2>;
+  CtSmem<KIND, NS>& S;
+  __device__ __forceinline__ double rk(int i) const { return S.co[0][i]; }
+  __device__ __forceinline__ double cr(int i) const { return S.co[1][i]; }
+  __device__ __forceinline__ double cv(int d, int i) const { return S.co[2 + d][i]; }
+  __device__ __forceinline__ double f(int q, int i) const { return S.f[q][i]; }
+  __device__ __forceinline__ double* recp(int i) const { return S.rec + i * D::NR; }
+  __device__ __forceinline__ const double* ivp(int i) const { return S.iv + i * D::NV; }
+  __device__ __forceinline__ double& xch(int k, int p) const { return S.x[k][p]; }
+  __device__ __forceinline__ void keep_mc(int i, double e0, double ce) const {
+    recp(i)[D::NR - 1] = cdft_mc<double>(e0, cr(i), ce);
+  }
+};
+
+template <typename T>
+struct CtPtr {
+  T* p[5];
+};
+
+template <int KIND, int NS, typename EI, typename EO>
+__global__ void __launch_bounds__(ct_threads<KIND>()) k_coarse64_tile(const __grid_constant__ Lvl<float> L,
+                                                                      CtPtr<const EI> ein, CtPtr<EO> eout,
+                                                                      Phys<double> P, PtK<double> K, int ntx) {
+  using D = ClDim<KIND, 2>;
+  using SM = CtSmem<KIND, NS>;
+  using Up = RoleUpdate<KIND, 2>;
+  constexpr int NU = D::NU, H = SM::H, SW = SM::SW, SN = SM::SN, TPBK = ct_threads<KIND>();
+  static_assert((CT_TX / 2 + 2 * NS - 1) * (CT_TY + 4 * NS - 2) <= CT_SETS * 32, "a thread updates one point of a pass");
+  __shared__ SM S;
+  const CtAcc<KIND, NS> a{S};
+  const int nx = L.g.nx, ny = L.g.ny;
+  const int x0 = (blockIdx.x % ntx) * CT_TX, y0 = (blockIdx.x / ntx) * CT_TY;
+  // two threads a cell: the correction and densities, the right-hand side and velocities
+  for (int t = threadIdx.x; t < 2 * SN; t += TPBK) {
+    const int c = t < SN ? t : t - SN;
+    const int g = wrapi(y0 - H + c / SW, ny) * nx + wrapi(x0 - H + c % SW, nx);
+    if (t < SN) {
+      EI e[NU];
+      const float rk = L.rk[g], cr = L.cr[g];
+#pragma unroll
+      for (int q = 0; q < NU; ++q) e[q] = ein.p[q][g];
+#pragma unroll
+      for (int q = 0; q < NU; ++q) S.rec[c * D::NR + q] = from_t<EI>(e[q]);
+      S.co[0][c] = widen(rk);
+      S.co[1][c] = widen(cr);
+    } else {
+      float f[NU];
+      const float u = L.cv[0][g], v = L.cv[1][g], om = L.om[0][g], rk = L.rk[g];
+#pragma unroll
+      for (int q = 0; q < NU; ++q) f[q] = L.f[q][g];
+#pragma unroll
+      for (int q = 0; q < NU; ++q) S.f[q][c] = widen(f[q]);
+      S.co[2][c] = widen(u);
+      S.co[3][c] = widen(v);
+      const double w = widen(om);
+      invert_block<2>(K, widen(rk), &w, S.iv + c * D::NV);
+    }
+  }
+  __syncthreads();
+  if constexpr (KIND == KCDFT) {  // the black cells the first pass reads
+    for (int t = threadIdx.x; t < SN / 2; t += TPBK) {
+      const int ly = t / (SW / 2), lx = 2 * (t - ly * (SW / 2)) + ((x0 + y0 + ly + 1) & 1);
+      const int c = ly * SW + lx;
+      a.keep_mc(c, S.rec[c * D::NR], P.ce);
+    }
+    __syncthreads();
+  }
+  const int warp = threadIdx.x >> 5, role = warp % D::R;
+  const int p = (warp / D::R) * 32 + (threadIdx.x & 31);
+#pragma unroll
+  for (int pass = 0; pass < 2 * NS; ++pass) {
+    const int ring = 2 * NS - 1 - pass, hw = CT_TX / 2 + ring;
+    RolePt<2> t;
+    RoleRegs g;
+    t.idx = -1;
+    if (p < hw * (CT_TY + 2 * ring)) {
+      const int ry = p / hw;
+      const int rx = 2 * (p - ry * hw) + (((pass & 1) + x0 + ring + y0 - ring + ry) & 1);
+      t.idx = (H - ring + ry) * SW + H - ring + rx;
+      t.ni[0] = t.idx - 1;
+      t.ni[1] = t.idx + 1;
+      t.ni[2] = t.idx - SW;
+      t.ni[3] = t.idx + SW;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) t.nr[k] = S.rec + t.ni[k] * D::NR;
+      Up::first(a, P, K, t, p, role, g);
+    }
+    __syncthreads();
+    if (t.idx >= 0) Up::second(a, P, K, t, p, role, g);
+    __syncthreads();
+  }
+  for (int t = threadIdx.x; t < CT_TX * CT_TY * NU; t += TPBK) {
+    const int q = t / (CT_TX * CT_TY), c = t % (CT_TX * CT_TY);
+    const int gx = x0 + c % CT_TX, gy = y0 + c / CT_TX;
+    if (gx < nx && gy < ny)
+      eout.p[q][gy * nx + gx] = to_t<EO>(S.rec[((H + c / CT_TX) * SW + H + c % CT_TX) * D::NR + q]);
   }
 }
 

@@ -1040,11 +1040,60 @@ struct Solver {
     return FM_OK;
   }
 
+  // ncoarse float64 sweeps of the float32 coarsest level l on tiles, two a
+  // launch (k_coarse64_tile); between launches the correction stays in
+  // float64, in the e and r buffers of the level's float64 copy in turn.
+  static int coarse_tiles64(fm_state* st, int l, int* out_in_r) {
+    if constexpr (DIM == 2 && sizeof(T) == 4) {
+      const Lvl<float> L = make_lvl<float>(st, l);
+      const Phys<double> P = make_phys<double>(st);
+      const PtK<double> K = make_ptk<double, 2>(P, st->lv[l].h);
+      const int ntx = (L.g.nx + CT_TX - 1) / CT_TX, nblk = ntx * ((L.g.ny + CT_TY - 1) / CT_TY);
+      CtPtr<const float> ef{};
+      CtPtr<float> of{};
+      CtPtr<double> b[2] = {};
+      const int n = st->prm.ncoarse;
+      for (int q = 0; q < LY::NU; ++q) {
+        ef.p[q] = L.e[q];
+        of.p[q] = n > 2 ? L.e[q] : L.r[q];  // (one launch: not over the values its tiles still read)
+        b[0].p[q] = (double*)st->lv64[l].e[q];
+        b[1].p[q] = (double*)st->lv64[l].r[q];
+      }
+      *out_in_r = n > 2 ? 0 : 1;
+      for (int it = 0, k = 0; it < n; it += 2, ++k) {
+        CtPtr<const double> ed{};
+        for (int q = 0; q < LY::NU; ++q) ed.p[q] = b[(k + 1) & 1].p[q];
+        const bool two = it + 2 <= n;
+        auto go = [&](auto ns) {
+          constexpr int NS = decltype(ns)::value;
+          constexpr int TH = ct_threads<KIND>();
+          if (k == 0 && it + 2 >= n)
+            k_coarse64_tile<KIND, NS, float, float><<<nblk, TH, 0, st->stream>>>(L, ef, of, P, K, ntx);
+          else if (k == 0)
+            k_coarse64_tile<KIND, NS, float, double><<<nblk, TH, 0, st->stream>>>(L, ef, b[0], P, K, ntx);
+          else if (it + 2 < n)
+            k_coarse64_tile<KIND, NS, double, double><<<nblk, TH, 0, st->stream>>>(L, ed, b[k & 1], P, K, ntx);
+          else
+            k_coarse64_tile<KIND, NS, double, float><<<nblk, TH, 0, st->stream>>>(L, ed, of, P, K, ntx);
+        };
+        if (two) go(std::integral_constant<int, 2>{});
+        else go(std::integral_constant<int, 1>{});
+        FM_LAUNCHED();
+      }
+    }
+    return FM_OK;
+  }
+
   // The coarsest-grid solve in float64 (mixed path): the V-cycle of the
-  // levels from l down by one cluster, or a larger coarsest level's ncoarse
-  // sweeps as colour launches on its float64 copy between two conversions.
-  static int coarse_solve64(fm_state* st, int l) {
+  // levels from l down by one cluster; or a larger coarsest level's ncoarse
+  // sweeps, on tiles (2-D, at most CT_MAXN points) or as colour launches on
+  // its float64 copy between two conversions.
+  // *out_in_r: on return the correction of level l is in its r buffer.
+  static int coarse_solve64(fm_state* st, int l, int* out_in_r) {
     if (!st->coarse_fused) return cluster_cycle(st, l);
+    if constexpr (DIM == 2 && sizeof(T) == 4) {
+      if (st->lv[l].g.N <= CT_MAXN) return coarse_tiles64(st, l, out_in_r);
+    }
     int rc = coarse_to64(st, l);
     if (rc) return rc;
     const Phys<double> P64 = make_phys<double>(st);
@@ -1078,7 +1127,7 @@ struct Solver {
     cudaStream_t s = st->stream;
     *out_in_r = 0;
     if constexpr (sizeof(T) == 4) {
-      if (l >= st->small_from && st->coarse64) return coarse_solve64(st, l);
+      if (l >= st->small_from && st->coarse64) return coarse_solve64(st, l, out_in_r);
     }
     if (l >= st->small_from && st->coarse_fused) {  // the coarsest level: ncoarse fused sweeps
       return smooth(st, l, P, st->prm.ncoarse, out_in_r);
