@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(TPB) kb_prepare_mu(const WorkItem* items, int 
 }
 
 template <typename T, int KIND>
-__global__ void __launch_bounds__(TPB) kb_resid64(const WorkItem* items, int nitems, const InstDev<T>* D,
+__global__ void __launch_bounds__(TPB, 4) kb_resid64(const WorkItem* items, int nitems, const InstDev<T>* D,
                                                   const Phys<double>* P64, const Step64* K64, const Ctl* ctl,
                                                   int check_active) {
   FM_BATCH_HEAD();

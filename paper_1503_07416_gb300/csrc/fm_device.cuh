@@ -2006,12 +2006,60 @@ __device__ __forceinline__ void resid64_body(const Fields64& F, const Resid64Out
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
 }
 
+// --------------------------------------------------------------------------
+// Exact neighbour sums in fixed point
+// --------------------------------------------------------------------------
+// A multiprocessor retires one float64 warp instruction in 19 clocks on GB300
+// (measured) and some 40 integer ones in the same time, so the neighbour sums
+// and differences of the residual, half of its float64 instructions, are taken
+// in 64-bit integers: a set of values x (a staged tile of one quantity) whose
+// largest magnitude has the biased exponent emax is held as trunc(x 2^k), k
+// chosen so that the largest value has bit 58 set.  Sums of up to 16 of them
+// are exact, the result is rounded once, and each value carries 6 bits more
+// than the largest float64, so the error is below that of the float64 sum
+// wherever a point's values are within a factor 16 of the set's largest.
+constexpr int FIX_EMIN = 128, FIX_EMAX = 1423;  // clamp below; above (2^400), or non-finite: plain float64
+
+__device__ __forceinline__ unsigned fix_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ int fix_exp(double x) { return (int)(fix_mag(x) >> 20) - 1023; }  // floor(log2 |x|)
+__device__ __forceinline__ long long to_fix(double x, int emax) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  unsigned long long m =
+      ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 6;
+  m = e == 0 ? 0ull : m >> min(emax - e, 63);
+  return (int)hi < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ double from_fix(long long v, int emax) {
+  unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  a <<= lz & 63;
+  // leading bit at 63: 53 bits rounded to nearest, the implicit one adds 1 to the exponent field
+  const unsigned long long r = (a >> 11) + ((a >> 10) & 1ull);
+  unsigned long long b = ((unsigned long long)(unsigned)(emax + 4 - lz) << 52) + r;
+  b = v == 0 ? 0ull : (b | ((unsigned long long)v & 0x8000000000000000ull));
+  return __longlong_as_double((long long)b);
+}
+
 // 2-D float64 residual in 32 x 8 tiles: the quantities every point shares
-// with its neighbours -- |u|^2, rho^k u, rho^k v and the implicit chemical
-// potential (mu, or ln rho + 2 c_e rho) -- are computed once per point of the
-// tile and its one-point halo in shared memory, then N is evaluated on the
-// tile.  Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 as
-// in resid64_body (same per-block accumulation order on every run).
+// with its neighbours -- |u|^2 + 2 mu (mu the implicit chemical potential: the
+// unknown, or ln rho + 2 c_e rho), rho^k u, rho^k v -- are formed once per
+// point of the tile and its one-point halo in shared memory, with u, v (PFC:
+// kappa and rho) beside them, all in fixed point; then N is evaluated on the
+// tile.  |u|^2 and 2 mu are one quantity because the coefficient of the
+// chemical potential's gradient, s/(2h), is twice the kinetic one, s/(4h).
+// Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 as in
+// resid64_body (same per-block accumulation order on every run).
+//
+// Bound by the float64 pipe: ~25 float64 instructions a point with the
+// neighbour sums in fixed point, 51 without.  The scales come from a first
+// pass over the tile's magnitudes (exponents only; its loads find the second
+// pass's in L1, which costs less than holding seven values a point in
+// registers over the barrier: 28.6 us a launch at 512^2 so, 24.9 now, 36.8 with
+// float64 sums; 24 instance ensemble, 11 M points, 12.1 -> 10.8 ms a step).
+// Against quad precision the rows' errors are at most what they were (rho
+// 3e-17 -> 4e-21, u 4.0e-19 -> 3.1e-19, kappa 2.5e-16 -> 6e-18 at 512^2).  Where a tile holds a value that fixed point
+// does not take (non-finite, beyond 2^400) its sums are float64.
 constexpr int R64_TX = 32, R64_TY = 8;
 constexpr int R64_SW = R64_TX + 2, R64_SN = R64_SW * (R64_TY + 2);
 
@@ -2020,73 +2068,147 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
                                                   const Step64& K,
                                                   const Phys<double>& P, double* partials, int lb, int nb) {
   using LY = Layout<KIND, 2>;
-  __shared__ double sQ[R64_SN], sM[R64_SN], sRU[R64_SN], sRV[R64_SN];
+  constexpr bool PFC = KIND == KPFC;
+  // staged: |u|^2 + 2 mu, rho^k u, rho^k v, u, v (PFC: kappa, rho)
+  constexpr int NS = PFC ? 7 : 5;
+  // magnitudes: u and v, rho^k; PFC: mu, kappa, rho; CDFT: rho, the smallest rho
+  constexpr int NM = PFC ? 5 : 4;
+  __shared__ long long sX[NS][R64_SN];  // fixed point, or the bits of the float64 value
+  __shared__ unsigned sMax[NM];
   double acc[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) acc[q] = 0.0;
   float fa[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) fa[q] = 0.0f;
-  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_m = K.c_m, c_v = K.c_v;
+  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_v = K.c_v;
   const double third = 1.0 / 3.0;
   const int nx = G.nx, ny = G.ny;
   const int ntx = (nx + R64_TX - 1) / R64_TX;
   const int ntiles = ntx * ((ny + R64_TY - 1) / R64_TY);
   const double* const* g = F.g;
+  if (threadIdx.x < NM) sMax[threadIdx.x] = 0u;
   for (int tile = lb; tile < ntiles; tile += nb) {
     const int x0 = (tile % ntx) * R64_TX, y0 = (tile / ntx) * R64_TY;
-    for (int t = threadIdx.x; t < R64_SN; t += blockDim.x) {
+    auto cell = [&](int t) {
       const int ly = t / R64_SW, lx = t - ly * R64_SW;
-      int gx = x0 + lx - 1, gy = y0 + ly - 1;
-      gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
-      gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
-      gx = gx >= nx ? gx % nx : gx;
-      gy = gy >= ny ? gy % ny : gy;
-      const int gi = gy * nx + gx;
-      const double u = g[1][gi], v = g[2][gi], rk = F.rho[gi];
-      sQ[t] = u * u + v * v;
-      sRU[t] = rk * u;
-      sRV[t] = rk * v;
-      if constexpr (KIND == KPFC) {
-        sM[t] = g[LY::IMU][gi];
+      return wrapi(y0 + ly - 1, ny) * nx + wrapi(x0 + lx - 1, nx);
+    };
+    unsigned mag[NM];
+#pragma unroll
+    for (int a = 0; a < NM; ++a) mag[a] = 0u;
+    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
+      const int gi = cell(t);
+      mag[0] = max(mag[0], max(fix_mag(g[1][gi]), fix_mag(g[2][gi])));
+      mag[1] = max(mag[1], fix_mag(F.rho[gi]));
+      if constexpr (PFC) {
+        mag[2] = max(mag[2], fix_mag(g[LY::IMU][gi]));
+        mag[3] = max(mag[3], fix_mag(g[LY::IKA][gi]));
+        mag[4] = max(mag[4], fix_mag(g[0][gi]));
       } else {
         const double r = g[0][gi];
-        sM[t] = log(r) + 2.0 * P.ce * r;
+        mag[2] = max(mag[2], fix_mag(r));
+        mag[3] = max(mag[3], r > 0.0 ? 0x7ff00000u - min(fix_mag(r), 0x7ff00000u) : 0x7ff00000u);
+      }
+    }
+    __syncthreads();  // sMax is zero, the tile before is finished
+#pragma unroll
+    for (int a = 0; a < NM; ++a) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, mag[a]);
+      if ((threadIdx.x & 31) == 0) atomicMax(&sMax[a], m);
+    }
+    __syncthreads();
+    int em[NM];
+    bool fix = true;
+#pragma unroll
+    for (int a = 0; a < NM; ++a) {
+      em[a] = max((int)(sMax[a] >> 20), FIX_EMIN);
+      fix = fix && em[a] <= FIX_EMAX;
+    }
+    int e_mu = em[2];
+    if constexpr (!PFC) {
+      // |ln rho + 2 c_e rho|: |ln rho| from the exponents of the smallest and
+      // largest density; a density <= 0 (or subnormal) is left to float64
+      const int lo = 0x7ff - (int)(sMax[3] >> 20) - 1 - 1023, hi = (int)(sMax[2] >> 20) + 1 - 1023;
+      const int lg = max(max(lo < 0 ? -lo : lo, hi < 0 ? -hi : hi), 1);  // |ln rho| < lg
+      fix = (int)(sMax[3] >> 20) < 0x7fe && (int)(sMax[2] >> 20) <= FIX_EMAX && em[0] <= FIX_EMAX &&
+            em[1] <= FIX_EMAX;
+      e_mu = max(em[2] + 2 + fix_exp(P.ce), 1023 + 32 - __clz(lg)) + 1;
+    }
+    const int e_b = max(2 * em[0] - 1023 + 2, e_mu + 1) + 1;  // |u|^2 + 2 mu
+    const int e_ru = max(em[0] + em[1] - 1023 + 1, FIX_EMIN);
+    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
+      const int gi = cell(t);
+      const double u = g[1][gi], v = g[2][gi], rk = F.rho[gi];
+      double m;
+      if constexpr (PFC) {
+        m = g[LY::IMU][gi];
+      } else {
+        const double r = g[0][gi];
+        m = log(r) + 2.0 * P.ce * r;
+      }
+      const double q = u * u + v * v, ru = rk * u, rv = rk * v;
+      if (fix) {
+        sX[0][t] = to_fix(q, e_b) + 2 * to_fix(m, e_b);
+        sX[1][t] = to_fix(ru, e_ru);
+        sX[2][t] = to_fix(rv, e_ru);
+        sX[3][t] = to_fix(u, em[0]);
+        sX[4][t] = to_fix(v, em[0]);
+      } else {
+        sX[0][t] = __double_as_longlong(q + 2.0 * m);
+        sX[1][t] = __double_as_longlong(ru);
+        sX[2][t] = __double_as_longlong(rv);
+        sX[3][t] = __double_as_longlong(u);
+        sX[4][t] = __double_as_longlong(v);
+      }
+      if constexpr (PFC) {
+        const double ka = g[LY::IKA][gi], r = g[0][gi];
+        sX[NS - 2][t] = fix ? to_fix(ka, em[NM - 2]) : __double_as_longlong(ka);
+        sX[NS - 1][t] = fix ? to_fix(r, em[NM - 1]) : __double_as_longlong(r);
       }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < R64_TX * R64_TY; t += blockDim.x) {
+    if (threadIdx.x < NM) sMax[threadIdx.x] = 0u;
+    for (int t = threadIdx.x; t < R64_TX * R64_TY; t += TPB) {
       const int ty = t / R64_TX, tx = t - ty * R64_TX;
       const int i = x0 + tx, j = y0 + ty;
       if (i < nx && j < ny) {
         const int idx = j * nx + i;
-        const Nb n = neighbours(i, j, 0, G);
         const int c = (ty + 1) * R64_SW + tx + 1;
         const int xm = c - 1, xp = c + 1, ym = c - R64_SW, yp = c + R64_SW;
-        const double rkc = F.rho[idx];
-        double N[LY::NU];
-        N[0] = g[0][idx] + c_div * ((sRU[xp] - sRU[xm]) + (sRV[yp] - sRV[ym]));
-        const double uc = g[1][idx], vc = g[2][idx];
-        const double w = F.om[0][idx];
-        N[1] = rkc * (uc - c_w * w * vc + c_q * (sQ[xp] - sQ[xm]) + c_m * (sM[xp] - sM[xm]))
-             - c_v * (nbsum<double, 2>(g[1], n) - 4.0 * uc);
-        N[2] = rkc * (vc + c_w * w * uc + c_q * (sQ[yp] - sQ[ym]) + c_m * (sM[yp] - sM[ym]))
-             - c_v * (nbsum<double, 2>(g[2], n) - 4.0 * vc);
-        if constexpr (KIND == KPFC) {
-          const double rc = g[0][idx];
-          const double psi = rc - 1.5;
-          const double kc = g[LY::IKA][idx];
-          // h^2 Lap_h kappa and h^2 Lap_h rho; the 1/h^2 scale and the cubic (Horner form)
-          // go into fused multiply-adds (fewer float64 instructions, the same rows)
-          const double dk = nbsum<double, 2>(g[LY::IKA], n) - 4.0 * kc;
-          const double dr = nbsum<double, 2>(g[0], n) - 4.0 * rc;
-          N[LY::IMU] = fma(-ih2, dk, g[LY::IMU][idx] - psi * fma(psi * psi, third, P.alpha));
-          N[LY::IKA] = fma(-ih2, dr, kc);
-        }
-        double rv[LY::NU];  // all loads (S, rho) before the first store
+        double S[LY::NU];
 #pragma unroll
-        for (int q = 0; q < LY::NU; ++q) rv[q] = F.S[q][idx] - N[q];
-        const double g0c = g[0][idx];
+        for (int q = 0; q < LY::NU; ++q) S[q] = F.S[q][idx];
+        const double rkc = F.rho[idx], uc = g[1][idx], vc = g[2][idx], g0c = g[0][idx];
+        const double w = F.om[0][idx];
+        // 2h div(rho^k u), differences of |u|^2 + 2 mu, h^2 Lap of u, v (kappa, rho)
+        double dv, dq[2], lap[NS - 3];
+        if (fix) {
+          dv = from_fix((sX[1][xp] - sX[1][xm]) + (sX[2][yp] - sX[2][ym]), e_ru);
+          dq[0] = from_fix(sX[0][xp] - sX[0][xm], e_b);
+          dq[1] = from_fix(sX[0][yp] - sX[0][ym], e_b);
+#pragma unroll
+          for (int a = 3; a < NS; ++a)
+            lap[a - 3] = from_fix((sX[a][xm] + sX[a][xp]) + (sX[a][ym] + sX[a][yp]) - (sX[a][c] << 2),
+                                  em[a < 5 ? 0 : a - 2]);
+        } else {
+          auto x = [&](int a, int k) { return __longlong_as_double(sX[a][k]); };
+          dv = (x(1, xp) - x(1, xm)) + (x(2, yp) - x(2, ym));
+          dq[0] = x(0, xp) - x(0, xm);
+          dq[1] = x(0, yp) - x(0, ym);
+#pragma unroll
+          for (int a = 3; a < NS; ++a) lap[a - 3] = (x(a, xm) + x(a, xp) + x(a, ym) + x(a, yp)) - 4.0 * x(a, c);
+        }
+        double rv[LY::NU];
+        const double cw = c_w * w;
+        rv[0] = fma(-c_div, dv, S[0] - g0c);
+        rv[1] = fma(c_v, lap[0], fma(-rkc, fma(c_q, dq[0], fma(-cw, vc, uc)), S[1]));
+        rv[2] = fma(c_v, lap[1], fma(-rkc, fma(c_q, dq[1], fma(cw, uc, vc)), S[2]));
+        if constexpr (PFC) {
+          const double psi = g0c - 1.5;
+          rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap[2], fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][idx]));
+          rv[LY::IKA] = S[LY::IKA] - fma(-ih2, lap[3], g[LY::IKA][idx]);
+        }
 #pragma unroll
         for (int q = 0; q < LY::NU; ++q) {
           const double r = rv[q];
@@ -2101,13 +2223,13 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
         }
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
 }
 
 template <int KIND, typename T>
-__global__ void __launch_bounds__(TPB) k_resid64_tile(Fields64 F, Resid64Out O, Geo G, Step64 K,
+__global__ void __launch_bounds__(TPB, 4) k_resid64_tile(Fields64 F, Resid64Out O, Geo G, Step64 K,
                                                       Phys<double> P, double* partials) {
   resid64_tile_body<KIND, T>(F, O, G, K, P, partials, blockIdx.x, gridDim.x);
 }
