@@ -263,15 +263,18 @@ static cudaError_t fz_launch_smooth(const Lvl<typename M::T>& L, const Phys<type
 }
 
 // `iters` sweeps of a level (the correction in r if *in_r), two a launch while
-// two are left.  Tiles of 32 x 16 on levels of at least 256 x 128 points,
-// 16 x 8 below, where 32 x 16 would leave most multiprocessors without a tile.
+// two are left.  Tiles of 32 x 16 on levels of at least 256^2 points, 16 x 8
+// below, where 32 x 16 leaves multiprocessors without a tile: a cycle of 20
+// sweeps takes 59.9 / 55.6 us (flow), 84.1 / 75.2 us (channel) with the large
+// and the small tiles at 256 x 128, 63.5 / 63.6 and 92.4 / 96.1 us at 256^2,
+// 78.8 / 81.7 and 127 / 140 us at 512 x 256; float64 alike.
 // float64 takes one sweep a launch: the two-sweep tile's wider halo is 1.3 to
 // 1.7 times the point updates, which are what bounds it.
 template <class M>
 static cudaError_t fz_smooth(const Lvl<typename M::T>& L, const Phys<typename M::T>& P, const typename M::W& W,
                              int iters, int* in_r, long long* launches, cudaStream_t s) {
   const typename M::K K = M::constants(P, L.h);
-  const bool big = L.g.N >= 256 * 128;
+  const bool big = L.g.N >= 256 * 256;
   for (int it = 0; it < iters;) {
     cudaError_t e;
     if (sizeof(typename M::T) == 4 && it + 2 <= iters) {
