@@ -1671,10 +1671,47 @@ struct Fields64 {
   const int* hist;            // extrapolated initial iterate: g already holds g^0 when *hist > 0 (or null)
 };
 
+// --------------------------------------------------------------------------
+// Exact neighbour sums in fixed point
+// --------------------------------------------------------------------------
+// A multiprocessor retires one float64 warp instruction in 19 clocks on GB300
+// (measured) and some 40 integer ones in the same time, so the neighbour sums
+// and differences of the residual, half of its float64 instructions, are taken
+// in 64-bit integers: a set of values x (a staged tile of one quantity) whose
+// largest magnitude has the biased exponent emax is held as trunc(x 2^k), k
+// chosen so that the largest value has bit 58 set.  Sums of up to 16 of them
+// are exact, the result is rounded once, and each value carries 6 bits more
+// than the largest float64, so the error is below that of the float64 sum
+// wherever a point's values are within a factor 16 of the set's largest.
+constexpr int FIX_EMIN = 128, FIX_EMAX = 1423;  // clamp below; above (2^400), or non-finite: plain float64
+
+__device__ __forceinline__ unsigned fix_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ int fix_exp(double x) { return (int)(fix_mag(x) >> 20) - 1023; }  // floor(log2 |x|)
+__device__ __forceinline__ long long to_fix(double x, int emax) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  unsigned long long m =
+      ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 6;
+  m = e == 0 ? 0ull : m >> min(emax - e, 63);
+  return (int)hi < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ double from_fix(long long v, int emax) {
+  unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  a <<= lz & 63;
+  // leading bit at 63: 53 bits rounded to nearest, the implicit one adds 1 to the exponent field
+  const unsigned long long r = (a >> 11) + ((a >> 10) & 1ull);
+  unsigned long long b = ((unsigned long long)(unsigned)(emax + 4 - lz) << 52) + r;
+  b = v == 0 ? 0ull : (b | ((unsigned long long)v & 0x8000000000000000ull));
+  return __longlong_as_double((long long)b);
+}
+
 // omega^k, S and the initial iterate g^0 (kappa^0 = Lap_h rho^k for PFC).
-template <int KIND, int DIM>
+// FIX: the neighbour sums in fixed point (eu, er: the exponents of the largest
+// velocity and density).
+template <int KIND, int DIM, bool FIX = false>
 __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, const Step64& K,
-                                              const Phys<double>& P, int idx) {
+                                              const Phys<double>& P, int idx, int eu = 0, int er = 0) {
   using LY = Layout<KIND, DIM>;
   if (idx >= G.N) return;
   int i, j, k;
@@ -1684,22 +1721,49 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
   const double* u = F.vel[0];
   const double* v = F.vel[1];
   double w[3];
+  // (b_{+i} - b_{-i}) - (a_{+j} - a_{-j})
+  auto rot = [&](const double* b, int i, const double* a, int j) {
+    if constexpr (FIX)
+      return from_fix((to_fix(b[n.p[i]], eu) - to_fix(b[n.m[i]], eu)) - (to_fix(a[n.p[j]], eu) - to_fix(a[n.m[j]], eu)),
+                      eu);
+    else
+      return (b[n.p[i]] - b[n.m[i]]) - (a[n.p[j]] - a[n.m[j]]);
+  };
+  auto lap = [&](const double* a, int e) {  // h^2 Lap
+    if constexpr (FIX) {
+      long long s = 0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) s += to_fix(a[n.m[d]], e) + to_fix(a[n.p[d]], e);
+      return from_fix(s - 2 * DIM * to_fix(a[n.c], e), e);
+    } else {
+      return nbsum<double, DIM>(a, n) - 2.0 * DIM * a[n.c];
+    }
+  };
   if constexpr (DIM == 2) {
-    w[0] = K.hih * ((v[n.p[0]] - v[n.m[0]]) - (u[n.p[1]] - u[n.m[1]]));
+    w[0] = K.hih * rot(v, 0, u, 1);
   } else {
     const double* ww = F.vel[2];
-    w[0] = K.hih * ((ww[n.p[1]] - ww[n.m[1]]) - (v[n.p[2]] - v[n.m[2]]));
-    w[1] = K.hih * ((u[n.p[2]] - u[n.m[2]]) - (ww[n.p[0]] - ww[n.m[0]]));
-    w[2] = K.hih * ((v[n.p[0]] - v[n.m[0]]) - (u[n.p[1]] - u[n.m[1]]));
+    w[0] = K.hih * rot(ww, 1, v, 2);
+    w[1] = K.hih * rot(u, 2, ww, 0);
+    w[2] = K.hih * rot(v, 0, u, 1);
   }
   const double rkc = F.rho[n.c];
   if constexpr (KIND == KCDFT) {
     if (F.nonpos && rkc <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
   }
   double div = 0;
+  if constexpr (FIX) {
+    const int e = max(eu + er - 1023 + 1, FIX_EMIN);
+    long long s = 0;
 #pragma unroll
-  for (int d = 0; d < DIM; ++d)
-    div += F.rho[n.p[d]] * F.vel[d][n.p[d]] - F.rho[n.m[d]] * F.vel[d][n.m[d]];
+    for (int d = 0; d < DIM; ++d)
+      s += to_fix(F.rho[n.p[d]] * F.vel[d][n.p[d]], e) - to_fix(F.rho[n.m[d]] * F.vel[d][n.m[d]], e);
+    div = from_fix(s, e);
+  } else {
+#pragma unroll
+    for (int d = 0; d < DIM; ++d)
+      div += F.rho[n.p[d]] * F.vel[d][n.p[d]] - F.rho[n.m[d]] * F.vel[d][n.m[d]];
+  }
   const double c_w = K.c_w, c_v = K.c_v, c_e = K.c_m;
   const double s0 = rkc - K.c_div * div;
   double uc[3], wx[3], sv[3];  // all loads before the first store
@@ -1708,7 +1772,7 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
   cross<double, DIM>(w, uc, wx);
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    double sa = rkc * (uc[a] - c_w * wx[a]) + c_v * (nbsum<double, DIM>(F.vel[a], n) - 2.0 * DIM * uc[a]);
+    double sa = rkc * (uc[a] - c_w * wx[a]) + c_v * lap(F.vel[a], eu);
     if constexpr (KIND == KCDFT) {
       const double Ep = 2.0 * P.ce * F.rho[n.p[a]] + F.conv[n.p[a]];
       const double Em = 2.0 * P.ce * F.rho[n.m[a]] + F.conv[n.m[a]];
@@ -1716,7 +1780,7 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
     }
     sv[a] = sa;
   }
-  const double lapr = (KIND == KPFC) ? (nbsum<double, DIM>(F.rho, n) - 2.0 * DIM * rkc) * ih2 : 0.0;
+  const double lapr = (KIND == KPFC) ? lap(F.rho, er) * ih2 : 0.0;
   const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
   F.S[0][idx] = s0;
 #pragma unroll
@@ -1742,6 +1806,44 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
 template <int KIND, int DIM>
 __global__ void __launch_bounds__(TPB) k_prepare(Fields64 F, Geo G, Step64 K, Phys<double> P) {
   prepare_point<KIND, DIM>(F, G, K, P, blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// Largest of every thread's values into mag, one atomic a block and value.
+template <int NM>
+__device__ __forceinline__ void grid_max(const unsigned (&m)[NM], unsigned* mag) {
+  __shared__ unsigned sm[NM];
+  if (threadIdx.x < NM) sm[threadIdx.x] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < NM; ++a) {
+    const unsigned x = __reduce_max_sync(0xffffffffu, m[a]);
+    if ((threadIdx.x & 31) == 0) atomicMax(&sm[a], x);
+  }
+  __syncthreads();
+  if (threadIdx.x < NM) atomicMax(&mag[threadIdx.x], sm[threadIdx.x]);
+}
+
+// 3-D: the largest magnitudes (high words) of the velocity and the density
+// into mag[0 .. 1] (zero before), and k_prepare with its neighbour sums scaled
+// by them.  k_prepare is bound by the float64 pipe, 60 instructions a point in
+// 3-D, 27 in fixed point; the extra pass reads four arrays.
+template <int DIM>
+__global__ void __launch_bounds__(TPB) k_prepare_mag(Fields64 F, int N, unsigned* mag) {
+  unsigned m[2] = {0u, 0u};
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x) {
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) m[0] = max(m[0], fix_mag(F.vel[d][idx]));
+    m[1] = max(m[1], fix_mag(F.rho[idx]));
+  }
+  grid_max(m, mag);
+}
+
+template <int KIND, int DIM>
+__global__ void __launch_bounds__(TPB) k_prepare_fix(Fields64 F, Geo G, Step64 K, Phys<double> P, const unsigned* mag) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int eu = max((int)(mag[0] >> 20), FIX_EMIN), er = max((int)(mag[1] >> 20), FIX_EMIN);
+  if (max(eu, er) <= FIX_EMAX) prepare_point<KIND, DIM, true>(F, G, K, P, idx, eu, er);
+  else prepare_point<KIND, DIM>(F, G, K, P, idx);
 }
 
 // PFC: mu^0 = psi^3/3 + alpha psi + Lap_h kappa^0 + S_mu (value of the mu row at rho^k).
@@ -2006,41 +2108,6 @@ __device__ __forceinline__ void resid64_body(const Fields64& F, const Resid64Out
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
 }
 
-// --------------------------------------------------------------------------
-// Exact neighbour sums in fixed point
-// --------------------------------------------------------------------------
-// A multiprocessor retires one float64 warp instruction in 19 clocks on GB300
-// (measured) and some 40 integer ones in the same time, so the neighbour sums
-// and differences of the residual, half of its float64 instructions, are taken
-// in 64-bit integers: a set of values x (a staged tile of one quantity) whose
-// largest magnitude has the biased exponent emax is held as trunc(x 2^k), k
-// chosen so that the largest value has bit 58 set.  Sums of up to 16 of them
-// are exact, the result is rounded once, and each value carries 6 bits more
-// than the largest float64, so the error is below that of the float64 sum
-// wherever a point's values are within a factor 16 of the set's largest.
-constexpr int FIX_EMIN = 128, FIX_EMAX = 1423;  // clamp below; above (2^400), or non-finite: plain float64
-
-__device__ __forceinline__ unsigned fix_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-__device__ __forceinline__ int fix_exp(double x) { return (int)(fix_mag(x) >> 20) - 1023; }  // floor(log2 |x|)
-__device__ __forceinline__ long long to_fix(double x, int emax) {
-  const unsigned hi = (unsigned)__double2hiint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  unsigned long long m =
-      ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 6;
-  m = e == 0 ? 0ull : m >> min(emax - e, 63);
-  return (int)hi < 0 ? -(long long)m : (long long)m;
-}
-__device__ __forceinline__ double from_fix(long long v, int emax) {
-  unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int lz = __clzll((long long)a);
-  a <<= lz & 63;
-  // leading bit at 63: 53 bits rounded to nearest, the implicit one adds 1 to the exponent field
-  const unsigned long long r = (a >> 11) + ((a >> 10) & 1ull);
-  unsigned long long b = ((unsigned long long)(unsigned)(emax + 4 - lz) << 52) + r;
-  b = v == 0 ? 0ull : (b | ((unsigned long long)v & 0x8000000000000000ull));
-  return __longlong_as_double((long long)b);
-}
-
 // 2-D float64 residual in 32 x 8 tiles: the quantities every point shares
 // with its neighbours -- |u|^2 + 2 mu (mu the implicit chemical potential: the
 // unknown, or ln rho + 2 c_e rho), rho^k u, rho^k v -- are formed once per
@@ -2236,28 +2303,52 @@ __global__ void __launch_bounds__(TPB, 4) k_resid64_tile(Fields64 F, Resid64Out 
 
 // Per-point quantities every point shares with its neighbours in the
 // float64 residual (used in 3-D): X[0] = |u|^2, X[1 + d] = rho^k u_d, and for
-// CDFT X[4] = ln rho + 2 c_e rho.
+// CDFT X[4] = ln rho + 2 c_e rho.  mag: the largest magnitudes (high words) of
+// the whole grid's u, rho^k, mu (PFC: the unknown; CDFT: X[4]) and, PFC, kappa
+// and rho, which scale the residual's fixed-point sums; zero before the pass.
 struct Shared64 {
   double* x[5];
+  unsigned* mag;
 };
+constexpr int X64_NM = 5;
 
+// The shared quantities of one point with iterate gv, and its magnitudes.
 template <int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_shared64(Fields64 F, Shared64 X, int N, double ce) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= N) return;
-  const double rk = F.rho[idx];
-  double u[DIM];
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) u[d] = F.g[1 + d][idx];
-  const double r = F.g[0][idx];
+__device__ __forceinline__ void shared64_point(const Shared64& X, const double* gv, double rk, double ce, int idx,
+                                               unsigned (&m)[X64_NM]) {
+  using LY = Layout<KIND, DIM>;
   double q = 0;
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
-    q += u[d] * u[d];
-    X.x[1 + d][idx] = rk * u[d];
+    q += gv[1 + d] * gv[1 + d];
+    X.x[1 + d][idx] = rk * gv[1 + d];
+    m[0] = max(m[0], fix_mag(gv[1 + d]));
   }
   X.x[0][idx] = q;
-  if constexpr (KIND == KCDFT) X.x[4][idx] = log(r) + 2.0 * ce * r;
+  m[1] = fix_mag(rk);
+  if constexpr (KIND == KPFC) {
+    m[2] = fix_mag(gv[LY::IMU]);
+    m[3] = fix_mag(gv[LY::IKA]);
+    m[4] = fix_mag(gv[0]);
+  } else {
+    const double mu = log(gv[0]) + 2.0 * ce * gv[0];
+    X.x[4][idx] = mu;
+    m[2] = fix_mag(mu);
+  }
+}
+
+template <int KIND, int DIM>
+__global__ void __launch_bounds__(TPB) k_shared64(Fields64 F, Shared64 X, int N, double ce) {
+  using LY = Layout<KIND, DIM>;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned m[X64_NM] = {0u, 0u, 0u, 0u, 0u};
+  if (idx < N) {
+    double gv[LY::NU];
+#pragma unroll
+    for (int q = 0; q < LY::NU; ++q) gv[q] = F.g[q][idx];
+    shared64_point<KIND, DIM>(X, gv, F.rho[idx], ce, idx, m);
+  }
+  grid_max(m, X.mag);
 }
 
 // After a cycle (3-D): the float64 update g += e of update64_point (with its
@@ -2269,82 +2360,107 @@ __global__ void __launch_bounds__(TPB) k_update_shared64(Fields64 F, Resid64Out 
                                                          double delta) {
   using LY = Layout<KIND, DIM>;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= N) return;
-  double gv[LY::NU];
-  T ev[LY::NU];  // all loads before the first store
+  unsigned m[X64_NM] = {0u, 0u, 0u, 0u, 0u};
+  if (idx < N) {
+    double gv[LY::NU];
+    T ev[LY::NU];  // all loads before the first store
 #pragma unroll
-  for (int q = 0; q < LY::NU; ++q) {
-    gv[q] = F.g[q][idx];
-    ev[q] = static_cast<const T*>(O.e0[q])[idx];
+    for (int q = 0; q < LY::NU; ++q) {
+      gv[q] = F.g[q][idx];
+      ev[q] = static_cast<const T*>(O.e0[q])[idx];
+    }
+    const double rk = F.rho[idx];
+#pragma unroll
+    for (int q = 0; q < LY::NU; ++q) gv[q] += from_t<T>(ev[q]);
+    gv[0] = (delta > 0.0) ? sqrt(gv[0] * gv[0] + delta * delta) : fabs(gv[0]);
+    if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
+#pragma unroll
+    for (int q = 0; q < LY::NU; ++q) F.g[q][idx] = gv[q];
+    shared64_point<KIND, DIM>(X, gv, rk, ce, idx, m);
   }
-  const double rk = F.rho[idx];
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) gv[q] += from_t<T>(ev[q]);
-  gv[0] = (delta > 0.0) ? sqrt(gv[0] * gv[0] + delta * delta) : fabs(gv[0]);
-  if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) F.g[q][idx] = gv[q];
-  double q2 = 0;
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) {
-    q2 += gv[1 + d] * gv[1 + d];
-    X.x[1 + d][idx] = rk * gv[1 + d];
-  }
-  X.x[0][idx] = q2;
-  if constexpr (KIND == KCDFT) X.x[4][idx] = log(gv[0]) + 2.0 * ce * gv[0];
+  grid_max(m, X.mag);
 }
 
-// Float64 residual reading the shared quantities of k_shared64.
-template <int KIND, int DIM, typename T>
-__global__ void __launch_bounds__(TPB) k_resid64_x(Fields64 F, Shared64 X, Resid64Out O, Geo G, Step64 K,
-                                                   Phys<double> P, double* partials) {
+// Float64 residual reading the shared quantities of k_shared64.  Bound by the
+// float64 pipe: ~28 instructions a point in 3-D with the neighbour sums in
+// fixed point (scaled by the grid's magnitudes), 81 without.
+template <int KIND, int DIM, typename T, bool FIX>
+__device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64& X, const Resid64Out& O, const Geo& G,
+                                               const Step64& K, const Phys<double>& P, double* partials,
+                                               const int (&em)[X64_NM]) {
   using LY = Layout<KIND, DIM>;
+  constexpr bool PFC = KIND == KPFC;
   double acc[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) acc[q] = 0.0;
   float fa[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) fa[q] = 0.0f;
-  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_m = K.c_m, c_v = K.c_v;
+  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_v = K.c_v;
   const double third = 1.0 / 3.0;
   const double* const* g = F.g;
-  const double* M = (KIND == KPFC) ? g[LY::IMU] : X.x[4];
+  const double* M = PFC ? g[LY::IMU] : X.x[4];
+  const int e_b = max(2 * em[0] - 1023 + 3, em[2] + 1) + 1;  // |u|^2 + 2 mu
+  const int e_ru = max(em[0] + em[1] - 1023 + 1, FIX_EMIN);  // rho^k u
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < G.N; idx += gridDim.x * blockDim.x) {
     int i, j, k;
     coords(idx, G, i, j, k);
     const Nb n = neighbours(i, j, k, G);
-    const double rkc = F.rho[n.c];
-    double N[LY::NU];
-    double div = 0;
+    auto lap = [&](const double* a, double c, int e) {  // h^2 Lap
+      if constexpr (FIX) {
+        long long s = 0;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) div += X.x[1 + d][n.p[d]] - X.x[1 + d][n.m[d]];
-    N[0] = g[0][n.c] + c_div * div;
-    double uc[3], w[3], wx[3];
+        for (int d = 0; d < DIM; ++d) s += to_fix(a[n.m[d]], e) + to_fix(a[n.p[d]], e);
+        return from_fix(s - 2 * DIM * to_fix(c, e), e);
+      } else {
+        return nbsum<double, DIM>(a, n) - 2.0 * DIM * c;
+      }
+    };
+    double dv, dq[DIM];  // 2h div(rho^k u), differences of |u|^2 + 2 mu
+    if constexpr (FIX) {
+      long long s = 0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        s += to_fix(X.x[1 + d][n.p[d]], e_ru) - to_fix(X.x[1 + d][n.m[d]], e_ru);
+        dq[d] = from_fix((to_fix(X.x[0][n.p[d]], e_b) - to_fix(X.x[0][n.m[d]], e_b)) +
+                             2 * (to_fix(M[n.p[d]], e_b) - to_fix(M[n.m[d]], e_b)),
+                         e_b);
+      }
+      dv = from_fix(s, e_ru);
+    } else {
+      dv = 0;
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        dv += X.x[1 + d][n.p[d]] - X.x[1 + d][n.m[d]];
+        dq[d] = (X.x[0][n.p[d]] - X.x[0][n.m[d]]) + 2.0 * (M[n.p[d]] - M[n.m[d]]);
+      }
+    }
+    const double rkc = F.rho[n.c], g0c = g[0][n.c];
+    double uc[3], w[3], S[LY::NU], rv[LY::NU];  // all loads before the first store
 #pragma unroll
     for (int d = 0; d < DIM; ++d) uc[d] = g[1 + d][n.c];
 #pragma unroll
-    for (int d = 0; d < LY::NOM; ++d) w[d] = F.om[d][n.c];
-    cross<double, DIM>(w, uc, wx);
+    for (int d = 0; d < LY::NOM; ++d) w[d] = c_w * F.om[d][n.c];
+#pragma unroll
+    for (int q = 0; q < LY::NU; ++q) S[q] = F.S[q][idx];
+    rv[0] = fma(-c_div, dv, S[0] - g0c);
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-      N[1 + a] = rkc * (uc[a] + c_w * wx[a] + c_q * (X.x[0][n.p[a]] - X.x[0][n.m[a]]) + c_m * (M[n.p[a]] - M[n.m[a]]))
-               - c_v * (nbsum<double, DIM>(g[1 + a], n) - 2.0 * DIM * uc[a]);
+      // u + c_w (omega x u) + c_q d(|u|^2 + 2 mu)
+      double br;
+      if constexpr (DIM == 2)
+        br = a == 0 ? fma(-w[0], uc[1], uc[0]) : fma(w[0], uc[0], uc[1]);
+      else
+        br = fma(w[(a + 1) % 3], uc[(a + 2) % 3], fma(-w[(a + 2) % 3], uc[(a + 1) % 3], uc[a]));
+      br = fma(c_q, dq[a], br);
+      rv[1 + a] = fma(c_v, lap(g[1 + a], uc[a], em[0]), fma(-rkc, br, S[1 + a]));
     }
-    if constexpr (KIND == KPFC) {
-      const double rc = g[0][n.c];
-      const double psi = rc - 1.5;
-      const double kc = g[LY::IKA][n.c];
-      // h^2 Lap_h kappa and h^2 Lap_h rho; the 1/h^2 scale and the cubic (Horner form)
-      // go into fused multiply-adds (fewer float64 instructions, the same rows)
-      const double dk = nbsum<double, DIM>(g[LY::IKA], n) - 2.0 * DIM * kc;
-      const double dr = nbsum<double, DIM>(g[0], n) - 2.0 * DIM * rc;
-      N[LY::IMU] = fma(-ih2, dk, g[LY::IMU][n.c] - psi * fma(psi * psi, third, P.alpha));
-      N[LY::IKA] = fma(-ih2, dr, kc);
+    if constexpr (PFC) {
+      const double psi = g0c - 1.5, kc = g[LY::IKA][n.c];
+      rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap(g[LY::IKA], kc, em[3]),
+                                     fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][n.c]));
+      rv[LY::IKA] = S[LY::IKA] - fma(-ih2, lap(g[0], g0c, em[4]), kc);
     }
-    double rv[LY::NU];  // all loads (S, rho) before the first store
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) rv[q] = F.S[q][idx] - N[q];
-    const double g0c = g[0][idx];
 #pragma unroll
     for (int q = 0; q < LY::NU; ++q) {
       const double r = rv[q];
@@ -2359,6 +2475,20 @@ __global__ void __launch_bounds__(TPB) k_resid64_x(Fields64 F, Shared64 X, Resid
     }
   }
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, blockIdx.x);
+}
+
+template <int KIND, int DIM, typename T>
+__global__ void __launch_bounds__(TPB, 4) k_resid64_x(Fields64 F, Shared64 X, Resid64Out O, Geo G, Step64 K,
+                                                   Phys<double> P, double* partials) {
+  int em[X64_NM];
+  bool fix = true;
+#pragma unroll
+  for (int a = 0; a < X64_NM; ++a) {
+    em[a] = max((int)(X.mag[a] >> 20), FIX_EMIN);
+    fix = fix && em[a] <= FIX_EMAX;
+  }
+  if (fix) resid64_x_body<KIND, DIM, T, true>(F, X, O, G, K, P, partials, em);
+  else resid64_x_body<KIND, DIM, T, false>(F, X, O, G, K, P, partials, em);
 }
 
 template <int KIND, int DIM, typename T>
@@ -2530,6 +2660,24 @@ __global__ void __launch_bounds__(TPB) k_closure(Fields64 F, Geo G, Step64 K, Ph
                                                  const Ctl* ctl) {
   if (ctl->status != FM_OK) return;
   closure_point<DIM>(F, G, K, P, out, blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// The same (3-D) from the products rho^k u_d that the last residual's first
+// pass left in X for the converged velocity.
+template <int DIM>
+__global__ void __launch_bounds__(TPB) k_closure_x(Fields64 F, Shared64 X, Geo G, Step64 K, Phys<double> P, double* out,
+                                                   const Ctl* ctl) {
+  if (ctl->status != FM_OK) return;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= G.N) return;
+  int i, j, k;
+  coords(idx, G, i, j, k);
+  const Nb n = neighbours(i, j, k, G);
+  double div = 0;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) div += X.x[1 + d][n.p[d]] - X.x[1 + d][n.m[d]];
+  const double r = F.S[0][idx] - K.c_div * div;
+  out[idx] = (P.delta > 0.0) ? sqrt(r * r + P.delta * P.delta) : fabs(r);
 }
 
 // New time level: rho <- closure result, u <- converged velocity (if the

@@ -693,7 +693,14 @@ struct Solver {
     }
     Fields64 F = make_fields(st);
     const Step64 K = make_step64(P, 1.0 / h);
-    k_prepare<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
+    if constexpr (DIM == 3) {
+      FM_CUDA(cudaMemsetAsync(st->mag, 0, 2 * sizeof(unsigned), s));
+      k_prepare_mag<DIM><<<st->nblk, TPB, 0, s>>>(F, G.N, st->mag);
+      FM_LAUNCHED();
+      k_prepare_fix<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P, st->mag);
+    } else {
+      k_prepare<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
+    }
     FM_LAUNCHED();
     if (KIND == KPFC) {
       k_prepare_mu<DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
@@ -726,6 +733,13 @@ struct Solver {
     return O;
   }
 
+  static Shared64 shared64(fm_state* st) {
+    Shared64 X;
+    for (int q = 0; q < 5; ++q) X.x[q] = st->x64[q];
+    X.mag = st->mag;
+    return X;
+  }
+
   // Float64 residual: 2-D tiled kernel; 3-D shared quantities then residual.
   // update (3-D, after a cycle): the float64 update g += e is made by the
   // shared-quantity pass (2-D makes it in k_update64 before this).
@@ -736,8 +750,8 @@ struct Solver {
       k_resid64_tile<KIND, T><<<st->nblk, TPB, 0, s>>>(F, O, G, make_step64(P, 1.0 / h), P, st->partials);
       FM_LAUNCHED();
     } else {
-      Shared64 X;
-      for (int q = 0; q < 5; ++q) X.x[q] = st->x64[q];
+      const Shared64 X = shared64(st);
+      FM_CUDA(cudaMemsetAsync(st->mag, 0, X64_NM * sizeof(unsigned), s));
       if (update)
         k_update_shared64<KIND, DIM, T><<<nblocks(G.N), TPB, 0, s>>>(F, O, X, G.N, P.ce, st->prm.delta);
       else
@@ -1198,8 +1212,11 @@ struct Solver {
     Fields64 F = make_fields(st);
     Phys<double> P64 = make_phys<double>(st);
     const Ctl* ctl = (const Ctl*)st->ctl;
-    k_closure<DIM><<<nblocks(G.N), TPB, 0, st->stream>>>(F, G, make_step64(P64, 1.0 / st->lv[0].h), P64, st->tmp,
-                                                         ctl);
+    const Step64 K = make_step64(P64, 1.0 / st->lv[0].h);
+    if constexpr (DIM == 3)
+      k_closure_x<DIM><<<nblocks(G.N), TPB, 0, st->stream>>>(F, shared64(st), G, K, P64, st->tmp, ctl);
+    else
+      k_closure<DIM><<<nblocks(G.N), TPB, 0, st->stream>>>(F, G, K, P64, st->tmp, ctl);
     FM_LAUNCHED();
     Vel3W vw{{st->vel[0], st->vel[1], st->vel[2]}};
     Vel3 gv{{st->g[1], st->g[2], DIM == 3 ? st->g[3] : nullptr}};
@@ -1310,6 +1327,7 @@ static size_t carve(fm_state* st, char* base) {
   st->partials = (double*)C.take((size_t)st->nblk * 8 * d8);
   st->dscal = (double*)C.take(64 * d8);
   st->ctl = C.take(64);
+  st->mag = (unsigned*)C.take(8 * sizeof(unsigned));
   for (int l = 0; l < st->nlev; ++l) {
     LevelBufs& B = st->lv[l];
     const size_t N = B.g.N;
