@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(TPB) k_ch_closure(Fields64 F, Geo G, Step64 K,
     div += gv(F.rho, n.p[d], G.N, 0, W) * gv(F.g[1 + d], n.p[d], G.N, d + 1, W) -
            gv(F.rho, n.m[d], G.N, 0, W) * gv(F.g[1 + d], n.m[d], G.N, d + 1, W);
   const double r = F.S[0][idx] - K.c_div * div;
-  out[idx] = delta > 0.0 ? sqrt(r * r + delta * delta) : fabs(r);
+  out[idx] = delta > 0.0 ? proj_rho(r, delta) : fabs(r);
 }
 
 // Energy densities of the PFC functional with the Neumann Laplacian, and KE.

@@ -102,7 +102,7 @@ struct RoleUpdate {
       for (int d = 0; d < DIM; ++d) div += r[2 * d + 1] * u[2 * d + 1] - r[2 * d] * u[2 * d];
       double er = f0 - K.c_div * div;
       const double x = crc + er;
-      if (x <= K.proj) er = sqrt(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
+      if (x <= K.proj) er = proj_rho(x, P.delta) - crc;  // Sec. 6 projection
       if constexpr (KIND == KPFC) {
         const double psi = crc - 1.5;
         g.cub = er * (psi * psi + psi * er + er * er * (1.0 / 3.0)) + P.alpha * er;
@@ -496,7 +496,7 @@ struct ClCycle {
       double ev = L.rec[p * D::NR + q] + w * acc;
       if (q == 0 && P.delta > 0.0) {
         const double c = a.cr(idx), x = c + ev;
-        if (x <= proj_threshold<double>(P.delta)) ev = sqrt(x * x + P.delta * P.delta) - c;
+        if (x <= proj_threshold<double>(P.delta)) ev = proj_rho(x, P.delta) - c;
       }
       L.rec[p * D::NR + q] = ev;
       if constexpr (KIND == KCDFT) {

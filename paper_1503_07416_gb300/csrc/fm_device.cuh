@@ -48,6 +48,15 @@ __host__ __device__ __forceinline__ T proj_threshold(T delta) {
   return delta * (sizeof(T) == 4 ? T(8192) : T(134217728));  // 2^13 ~ sqrt(2/2^-24), 2^27 ~ sqrt(2/2^-53)
 }
 
+// The positive projection sqrt(x^2 + delta^2).  In float64 a call, not inlined:
+// inlined, the compiler turns the branches around it into selects and every
+// point pays the square root's ~9 instructions on the float64 pipe, though
+// hardly any takes it (the 3-D update and first pass of the residual: 103 us at
+// 128^3 inlined, 65 us so).
+static __device__ __noinline__ double proj_call(double x, double delta) { return sqrt(x * x + delta * delta); }
+__device__ __forceinline__ double proj_rho(double x, double delta) { return proj_call(x, delta); }
+__device__ __forceinline__ float proj_rho(float x, float delta) { return sqrtf(x * x + delta * delta); }
+
 template <typename T, int DIM>
 __host__ __device__ __forceinline__ PtK<T> make_ptk(const Phys<T>& P, T h) {
   PtK<T> K;
@@ -109,7 +118,7 @@ __device__ __forceinline__ void smooth_point_a(const A& a, const Phys<T>& P, con
   T er = a.f(0, fc) - K.c_div * div;
   {
     const T x = crc + er;
-    if (x <= K.proj) er = sqrt_t(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
+    if (x <= K.proj) er = proj_rho(x, P.delta) - crc;  // Sec. 6 projection
   }
   T eg[LY::NU];
   eg[0] = er;
@@ -324,7 +333,7 @@ __device__ __forceinline__ void prolong_point(const Lvl<T>& F, const Lvl<T>& C, 
   if (P.delta > T(0)) {
     const T c = F.cr[idx];
     const T x = c + ev[0];
-    if (x <= proj_threshold<T>(P.delta)) ev[0] = sqrt_t(x * x + P.delta * P.delta) - c;
+    if (x <= proj_threshold<T>(P.delta)) ev[0] = proj_rho(x, P.delta) - c;
   }
 #pragma unroll
   for (int q = 0; q < NU; ++q) F.e[q][idx] = ev[q];
@@ -2372,7 +2381,7 @@ __global__ void __launch_bounds__(TPB) k_update_shared64(Fields64 F, Resid64Out 
     const double rk = F.rho[idx];
 #pragma unroll
     for (int q = 0; q < LY::NU; ++q) gv[q] += from_t<T>(ev[q]);
-    gv[0] = (delta > 0.0) ? sqrt(gv[0] * gv[0] + delta * delta) : fabs(gv[0]);
+    gv[0] = (delta > 0.0) ? proj_rho(gv[0], delta) : fabs(gv[0]);
     if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
 #pragma unroll
     for (int q = 0; q < LY::NU; ++q) F.g[q][idx] = gv[q];
@@ -2511,7 +2520,7 @@ __device__ __forceinline__ void update64_point(const Fields64& F, const Resid64O
   }
 #pragma unroll
   for (int q = 0; q < NU; ++q) gv[q] += from_t<T>(ev[q]);
-  gv[0] = (delta > 0.0) ? sqrt(gv[0] * gv[0] + delta * delta) : fabs(gv[0]);
+  gv[0] = (delta > 0.0) ? proj_rho(gv[0], delta) : fabs(gv[0]);
   if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
 #pragma unroll
   for (int q = 0; q < NU; ++q) F.g[q][idx] = gv[q];
@@ -2652,7 +2661,7 @@ __device__ __forceinline__ void closure_point(const Fields64& F, const Geo& G, c
   for (int d = 0; d < DIM; ++d)
     div += F.rho[n.p[d]] * F.g[1 + d][n.p[d]] - F.rho[n.m[d]] * F.g[1 + d][n.m[d]];
   const double r = F.S[0][idx] - K.c_div * div;
-  out[idx] = (P.delta > 0.0) ? sqrt(r * r + P.delta * P.delta) : fabs(r);
+  out[idx] = (P.delta > 0.0) ? proj_rho(r, P.delta) : fabs(r);
 }
 
 template <int DIM>
@@ -2677,7 +2686,7 @@ __global__ void __launch_bounds__(TPB) k_closure_x(Fields64 F, Shared64 X, Geo G
 #pragma unroll
   for (int d = 0; d < DIM; ++d) div += X.x[1 + d][n.p[d]] - X.x[1 + d][n.m[d]];
   const double r = F.S[0][idx] - K.c_div * div;
-  out[idx] = (P.delta > 0.0) ? sqrt(r * r + P.delta * P.delta) : fabs(r);
+  out[idx] = (P.delta > 0.0) ? proj_rho(r, P.delta) : fabs(r);
 }
 
 // New time level: rho <- closure result, u <- converged velocity (if the

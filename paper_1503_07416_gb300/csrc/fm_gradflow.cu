@@ -111,7 +111,7 @@ __device__ __forceinline__ void gf_smooth_point(const A& a, const Phys<T>& P, co
     T er = b1 - K.a * em;
     {
       const T x = crc + er;
-      if (x <= K.proj) er = sqrt_t(x * x + P.delta * P.delta) - crc;  // Sec. 6 projection
+      if (x <= K.proj) er = proj_rho(x, P.delta) - crc;  // Sec. 6 projection
     }
     const T ek = b3 - K.c * er;
     a.set_e(0, c, (T(1) - w) * er + w * eo0);
@@ -127,7 +127,7 @@ __device__ __forceinline__ void gf_smooth_point(const A& a, const Phys<T>& P, co
     T en = eo - F / dF;
     {
       const T x = crc + en;
-      if (x <= K.proj) en = sqrt_t(x * x + P.delta * P.delta) - crc;
+      if (x <= K.proj) en = proj_rho(x, P.delta) - crc;
     }
     a.set_e(0, c, (T(1) - w) * en + w * eo);
   }
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(TPB) k_gf_closure(GF64 F, Geo G, double ih2, d
     lap = (nb - 2.0 * DIM * mc) * ih2;
   }
   const double r = F.rho[idx] + s * lap;
-  out[idx] = (delta > 0.0) ? sqrt(r * r + delta * delta) : fabs(r);
+  out[idx] = (delta > 0.0) ? proj_rho(r, delta) : fabs(r);
 }
 
 __global__ void __launch_bounds__(TPB) k_gf_commit(double* rho, const double* rnew, int N, const Ctl* ctl) {
