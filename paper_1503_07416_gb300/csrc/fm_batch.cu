@@ -214,12 +214,15 @@ __global__ void __launch_bounds__(TPB) kb_resid_restrict2(const WorkItem* items,
   if (!inst_active(ctl, inst)) return;
   __shared__ Lvl<T> F, Cc;
   __shared__ T sr[Layout<KIND, 2>::NU * RR_FN];
+  __shared__ PtK<T> K[2];
   smem_copy(&F, &D[inst].lv[level]);
   smem_copy(&Cc, &D[inst].lv[level + 1]);
   __syncthreads();
+  if (threadIdx.x < 2) K[threadIdx.x] = make_ptk<T, 2>(P[inst], threadIdx.x ? Cc.h : F.h);
+  __syncthreads();
   lvl_swap_er(F, fswap);
   const int ntx = items[k_].aux;
-  resid_restrict2_tile<T, KIND>(F, Cc, P[inst], (lb % ntx) * RR_TX, (lb / ntx) * RR_TY, sr);
+  resid_restrict2_tile<T, KIND>(F, Cc, P[inst], K[0], K[1], (lb % ntx) * RR_TX, (lb / ntx) * RR_TY, sr);
 }
 
 template <typename T, int NU>

@@ -21,6 +21,20 @@ constexpr int TPB = 256;
 
 static inline int nblocks(long long work) { return (int)((work + TPB - 1) / TPB); }
 
+// Threads of a block of a per-point kernel over `work` points in precision T.
+// float64 kernels are bound by the multiprocessors' float64 pipes, so their
+// work is cut finely enough to load all of them alike (a 40 x 48 x 56 colour
+// pass in blocks of 256 puts two blocks on 58 of 152 multiprocessors and one
+// on the others: 27.0 us a pass, 19.3 us in blocks of 64; its 20 x 24 x 28 level
+// 14.8 us, 9.3 us in blocks of 32); float32 ones take small blocks where large
+// ones would leave multiprocessors without one.
+template <typename T>
+static inline int point_tpb(long long work, int sms) {
+  if (sizeof(T) == 8) return work <= 64LL * sms ? 32 : 64;
+  return work < (long long)TPB * sms ? 64 : TPB;
+}
+static inline int blocks_of(long long work, int tpb) { return (int)((work + tpb - 1) / tpb); }
+
 // --------------------------------------------------------------------------
 // Smoother point update (correction form)
 // --------------------------------------------------------------------------
@@ -69,6 +83,44 @@ __host__ __device__ __forceinline__ PtK<T> make_ptk(const Phys<T>& P, T h) {
   K.c_b = T(0.5) * P.sigma * P.s;
   K.proj = proj_threshold<T>(P.delta);
   return K;
+}
+
+// M(e) = N(c + e) - N(c) at one point, all components (App. G operator N in
+// correction form about the coefficient iterate c); K: the constants of the
+// spacing M is taken at.
+template <typename T, int KIND, int DIM>
+__device__ __forceinline__ void applyM(const Lvl<T>& L, const Phys<T>& P, const PtK<T>& K, const Nb& n,
+                                       T* const* E, T* M) {
+  using LY = Layout<KIND, DIM>;
+  const T rkc = L.rk[n.c];
+  T div = 0;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d)
+    div += L.rk[n.p[d]] * E[1 + d][n.p[d]] - L.rk[n.m[d]] * E[1 + d][n.m[d]];
+  M[0] = E[0][n.c] + K.c_div * div;
+
+  T ec[3], w[3], wx[3];
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) ec[d] = E[1 + d][n.c];
+#pragma unroll
+  for (int d = 0; d < LY::NOM; ++d) w[d] = K.c_b * L.om[d][n.c];
+  cross<T, DIM>(w, ec, wx);
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) {
+    const T dq = qcorr<T, DIM>(E, L.cv, n.p[a]) - qcorr<T, DIM>(E, L.cv, n.m[a]);
+    const T dm = mcorr<T, KIND, DIM>(E, L.cr, n.p[a], P.ce) - mcorr<T, KIND, DIM>(E, L.cr, n.m[a], P.ce);
+    M[1 + a] = rkc * (ec[a] + wx[a] + K.c_sih * (T(0.25) * dq + T(0.5) * dm))
+             - K.c_v * (nbsum<T, DIM>(E[1 + a], n) - T(2 * DIM) * ec[a]);
+  }
+  if constexpr (KIND == KPFC) {
+    const T er = E[0][n.c];
+    const T psi = L.cr[n.c] - T(1.5);
+    const T ek = E[LY::IKA][n.c];
+    const T lapk = (nbsum<T, DIM>(E[LY::IKA], n) - T(2 * DIM) * ek) * K.ih2;
+    const T lapr = (nbsum<T, DIM>(E[0], n) - T(2 * DIM) * er) * K.ih2;
+    M[LY::IMU] = E[LY::IMU][n.c] - er * (psi * psi + psi * er + er * er * T(1.0 / 3.0)) - P.alpha * er - lapk;
+    M[LY::IKA] = ek - lapr;
+  }
 }
 
 // Reciprocal of the point block's velocity determinant: the float32 smoother
@@ -222,7 +274,7 @@ __device__ __forceinline__ void smooth_point(const Lvl<T>& L, const Phys<T>& P, 
 // single-block small-level V-cycle)
 // --------------------------------------------------------------------------
 template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void resid_point(const Lvl<T>& L, const Phys<T>& P, int idx) {
+__device__ __forceinline__ void resid_point(const Lvl<T>& L, const Phys<T>& P, const PtK<T>& K, int idx) {
   using LY = Layout<KIND, DIM>;
   int i, j, k;
   coords(idx, L.g, i, j, k);
@@ -232,7 +284,7 @@ __device__ __forceinline__ void resid_point(const Lvl<T>& L, const Phys<T>& P, i
   // compiler knows, so interleaving would serialise them
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) fv[q] = L.f[q][idx];
-  applyM<T, KIND, DIM>(L, P, n, L.e, M);
+  applyM<T, KIND, DIM>(L, P, K, n, L.e, M);
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) L.r[q][idx] = fv[q] - M[q];
 }
@@ -282,13 +334,13 @@ __device__ __forceinline__ void restrict_point(const Lvl<T>& F, const Lvl<T>& C,
 
 // f_C += M_C(eh_C)
 template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void coarse_rhs_point(const Lvl<T>& L, const Phys<T>& P, int idx) {
+__device__ __forceinline__ void coarse_rhs_point(const Lvl<T>& L, const Phys<T>& P, const PtK<T>& K, int idx) {
   using LY = Layout<KIND, DIM>;
   int i, j, k;
   coords(idx, L.g, i, j, k);
   const Nb n = neighbours(i, j, k, L.g);
   T M[LY::NU];
-  applyM<T, KIND, DIM>(L, P, n, L.eh, M);
+  applyM<T, KIND, DIM>(L, P, K, n, L.eh, M);
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) L.f[q][idx] += M[q];
 }
@@ -344,19 +396,22 @@ __device__ __forceinline__ void prolong_point(const Lvl<T>& F, const Lvl<T>& C, 
 // M_C(eh) at the coarse point is evaluated on the fine arrays at the fine
 // indices 2I and 2I +- 2 with the coarse spacing.
 template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void coarse_m_on_fine(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int idx);
+__device__ __forceinline__ void coarse_m_on_fine(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P,
+                                                 const PtK<T>& KC, int idx);
 
 template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void restrict_rhs_point(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int idx) {
+__device__ __forceinline__ void restrict_rhs_point(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P,
+                                                   const PtK<T>& KC, int idx) {
   using LY = Layout<KIND, DIM>;
   restrict_point<T, LY::NU, DIM>(F, C, idx);
-  coarse_m_on_fine<T, KIND, DIM>(F, C, P, idx);
+  coarse_m_on_fine<T, KIND, DIM>(F, C, P, KC, idx);
 }
 
 // f_C += M_C(eh_C) at coarse point idx, evaluated on the fine arrays (see
 // restrict_rhs_point).
 template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void coarse_m_on_fine(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int idx) {
+__device__ __forceinline__ void coarse_m_on_fine(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P,
+                                                 const PtK<T>& KC, int idx) {
   using LY = Layout<KIND, DIM>;
   int I, J, K;
   coords(idx, C.g, I, J, K);
@@ -376,21 +431,19 @@ __device__ __forceinline__ void coarse_m_on_fine(const Lvl<T>& F, const Lvl<T>& 
   } else {
     n.m[2] = n.p[2] = n.c;
   }
-  Lvl<T> V = F;
-  V.h = C.h;
   T M[LY::NU];
   T fv[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) fv[q] = C.f[q][idx];
-  applyM<T, KIND, DIM>(V, P, n, F.e, M);
+  applyM<T, KIND, DIM>(F, P, KC, n, F.e, M);
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) C.f[q][idx] = fv[q] + M[q];
 }
 
 template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_restrict_rhs(Lvl<T> F, Lvl<T> C, Phys<T> P) {
+__global__ void __launch_bounds__(TPB) k_restrict_rhs(Lvl<T> F, Lvl<T> C, Phys<T> P, PtK<T> KC) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < C.g.N) restrict_rhs_point<T, KIND, DIM>(F, C, P, idx);
+  if (idx < C.g.N) restrict_rhs_point<T, KIND, DIM>(F, C, P, KC, idx);
 }
 
 // 2-D, one launch in place of k_resid + k_restrict_rhs: a block takes a
@@ -404,8 +457,8 @@ constexpr int RR_FN = (2 * RR_TX + 1) * (2 * RR_TY + 1);  // fine points per til
 
 // Coarse tile (I0, J0); sr: shared memory for NU x RR_FN values.
 template <typename T, int KIND>
-__device__ __forceinline__ void resid_restrict2_tile(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int I0,
-                                                     int J0, T* sr) {
+__device__ __forceinline__ void resid_restrict2_tile(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P,
+                                                     const PtK<T>& KF, const PtK<T>& KC, int I0, int J0, T* sr) {
   constexpr int NU = Layout<KIND, 2>::NU;
   constexpr int FW = 2 * RR_TX + 1, FN = RR_FN;
   for (int t = threadIdx.x; t < FN; t += blockDim.x) {
@@ -413,7 +466,7 @@ __device__ __forceinline__ void resid_restrict2_tile(const Lvl<T>& F, const Lvl<
     const int x = wrapi(2 * I0 - 1 + lx, F.g.nx), y = wrapi(2 * J0 - 1 + ly, F.g.ny);
     const Nb n = neighbours(x, y, 0, F.g);
     T M[NU];
-    applyM<T, KIND, 2>(F, P, n, F.e, M);
+    applyM<T, KIND, 2>(F, P, KF, n, F.e, M);
 #pragma unroll
     for (int q = 0; q < NU; ++q) sr[q * FN + t] = F.f[q][n.c] - M[q];
   }
@@ -439,23 +492,24 @@ __device__ __forceinline__ void resid_restrict2_tile(const Lvl<T>& F, const Lvl<
       C.e[q][cidx] = ev[q];
       C.eh[q][cidx] = ev[q];
     }
-    coarse_m_on_fine<T, KIND, 2>(F, C, P, cidx);
+    coarse_m_on_fine<T, KIND, 2>(F, C, P, KC, cidx);
   }
 }
 
 template <typename T, int KIND>
-__global__ void __launch_bounds__(TPB) k_resid_restrict2(Lvl<T> F, Lvl<T> C, Phys<T> P, int ntx) {
+__global__ void __launch_bounds__(TPB) k_resid_restrict2(Lvl<T> F, Lvl<T> C, Phys<T> P, PtK<T> KF, PtK<T> KC,
+                                                         int ntx) {
   __shared__ T sr[Layout<KIND, 2>::NU * RR_FN];
-  resid_restrict2_tile<T, KIND>(F, C, P, (blockIdx.x % ntx) * RR_TX, (blockIdx.x / ntx) * RR_TY, sr);
+  resid_restrict2_tile<T, KIND>(F, C, P, KF, KC, (blockIdx.x % ntx) * RR_TX, (blockIdx.x / ntx) * RR_TY, sr);
 }
 
 template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_smooth(Lvl<T> L, Phys<T> P, int color) {
+__global__ void __launch_bounds__(TPB) k_smooth(Lvl<T> L, Phys<T> P, PtK<T> K, int color) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int i, j, k;
   if (!colour_point(t, color, L.g, i, j, k)) return;
   const Nb n = neighbours(i, j, k, L.g);
-  smooth_point<T, KIND, DIM>(L, P, make_ptk<T, DIM>(P, L.h), n);
+  smooth_point<T, KIND, DIM>(L, P, K, n);
 }
 
 // Level accessor whose neighbours' CDFT chemical-potential parts come from M.
@@ -481,12 +535,11 @@ struct McAcc64 {
 // read only by the launch after the one that wrote it, so values and order
 // are those of k_smooth.
 template <int DIM, bool USE_M>
-__global__ void __launch_bounds__(TPB) k_smooth_cdft64_mc(Lvl<double> L, Phys<double> P, int color, double* M) {
+__global__ void __launch_bounds__(TPB) k_smooth_cdft64_mc(Lvl<double> L, Phys<double> P, PtK<double> K, int color, double* M) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int i, j, k;
   if (!colour_point(t, color, L.g, i, j, k)) return;
   const Nb n = neighbours(i, j, k, L.g);
-  const PtK<double> K = make_ptk<double, DIM>(P, L.h);
   if constexpr (USE_M) {
     const McAcc64 a{L, M};
     smooth_point_a<double, KCDFT, DIM>(a, P, K, n, n.c);
@@ -501,19 +554,19 @@ __global__ void __launch_bounds__(TPB) k_smooth_cdft64_mc(Lvl<double> L, Phys<do
 // cached loads, and more warps in flight hide that latency.  The 3-D
 // autotuner times it against k_smooth per level (it spills in float64).
 template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB, 6) k_smooth_occ(Lvl<T> L, Phys<T> P, int color) {
+__global__ void __launch_bounds__(TPB, 6) k_smooth_occ(Lvl<T> L, Phys<T> P, PtK<T> K, int color) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int i, j, k;
   if (!colour_point(t, color, L.g, i, j, k)) return;
   const Nb n = neighbours(i, j, k, L.g);
-  smooth_point<T, KIND, DIM>(L, P, make_ptk<T, DIM>(P, L.h), n);
+  smooth_point<T, KIND, DIM>(L, P, K, n);
 }
 
 // One colour of a sweep over the rows [row0, row0 + nrows) of a 3-D level
 // (a row is one (j, k); rows past the last wrap to the first), bounded to six
 // blocks per SM like k_smooth_occ.  Used to sweep the level in z-chunks.
 template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB, 6) k_smooth_rows(Lvl<T> L, Phys<T> P, int color, int row0, int nrows) {
+__global__ void __launch_bounds__(TPB, 6) k_smooth_rows(Lvl<T> L, Phys<T> P, PtK<T> K, int color, int row0, int nrows) {
   const int half = L.g.nx >> 1;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)nrows * half) return;
@@ -523,7 +576,7 @@ __global__ void __launch_bounds__(TPB, 6) k_smooth_rows(Lvl<T> L, Phys<T> P, int
   const int j = rowid % L.g.ny, k = rowid / L.g.ny;
   const int i = 2 * (int)(t % half) + ((j + k + color) & 1);
   const Nb n = neighbours(i, j, k, L.g);
-  smooth_point<T, KIND, DIM>(L, P, make_ptk<T, DIM>(P, L.h), n);
+  smooth_point<T, KIND, DIM>(L, P, K, n);
 }
 
 // 3-D sweep variants: 0 k_smooth, 1 k_smooth_occ, 2 the same sweep in
@@ -554,21 +607,9 @@ static inline int z_chunk_planes(const Geo& g) {
 }
 
 template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_resid(Lvl<T> L, Phys<T> P) {
+__global__ void __launch_bounds__(TPB) k_resid(Lvl<T> L, Phys<T> P, PtK<T> K) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < L.g.N) resid_point<T, KIND, DIM>(L, P, idx);
-}
-
-template <typename T, int NU, int DIM>
-__global__ void __launch_bounds__(TPB) k_restrict(Lvl<T> F, Lvl<T> C) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < C.g.N) restrict_point<T, NU, DIM>(F, C, idx);
-}
-
-template <typename T, int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_coarse_rhs(Lvl<T> L, Phys<T> P) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < L.g.N) coarse_rhs_point<T, KIND, DIM>(L, P, idx);
+  if (idx < L.g.N) resid_point<T, KIND, DIM>(L, P, K, idx);
 }
 
 template <typename T, int NU, int DIM>
@@ -1343,11 +1384,12 @@ __device__ __forceinline__ void vcycle_small_body(const SmallLv<T>& S, const Phy
     const Lvl<T>& F = S.lv[l];
     const Lvl<T>& C = S.lv[l + 1];
     block_smooth<T, KIND, DIM>(F, P, nu1);
-    for (int idx = threadIdx.x; idx < F.g.N; idx += blockDim.x) resid_point<T, KIND, DIM>(F, P, idx);
+    const PtK<T> K = make_ptk<T, DIM>(P, F.h), KC = make_ptk<T, DIM>(P, C.h);
+    for (int idx = threadIdx.x; idx < F.g.N; idx += blockDim.x) resid_point<T, KIND, DIM>(F, P, K, idx);
     __syncthreads();
     for (int idx = threadIdx.x; idx < C.g.N; idx += blockDim.x) restrict_point<T, LY::NU, DIM>(F, C, idx);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < C.g.N; idx += blockDim.x) coarse_rhs_point<T, KIND, DIM>(C, P, idx);
+    for (int idx = threadIdx.x; idx < C.g.N; idx += blockDim.x) coarse_rhs_point<T, KIND, DIM>(C, P, KC, idx);
     __syncthreads();
   }
   block_smooth<T, KIND, DIM>(S.lv[nl - 1], P, ncoarse);
@@ -1420,11 +1462,12 @@ __device__ __forceinline__ void group_down(const Lvl<T>& F, const Lvl<T>& C, con
   const int tid = WARP ? (threadIdx.x & 31) : threadIdx.x;
   const int nth = WARP ? 32 : blockDim.x;
   group_smooth<T, KIND, DIM, WARP>(F, P, nu1);
-  for (int idx = tid; idx < F.g.N; idx += nth) resid_point<T, KIND, DIM>(F, P, idx);
+  const PtK<T> K = make_ptk<T, DIM>(P, F.h), KC = make_ptk<T, DIM>(P, C.h);
+  for (int idx = tid; idx < F.g.N; idx += nth) resid_point<T, KIND, DIM>(F, P, K, idx);
   group_sync<T, KIND, DIM, WARP>();
   for (int idx = tid; idx < C.g.N; idx += nth) restrict_point<T, LY::NU, DIM>(F, C, idx);
   group_sync<T, KIND, DIM, WARP>();
-  for (int idx = tid; idx < C.g.N; idx += nth) coarse_rhs_point<T, KIND, DIM>(C, P, idx);
+  for (int idx = tid; idx < C.g.N; idx += nth) coarse_rhs_point<T, KIND, DIM>(C, P, KC, idx);
   group_sync<T, KIND, DIM, WARP>();
 }
 

@@ -225,12 +225,6 @@ __global__ void __launch_bounds__(TPB) k_gf_coarse_rhs(Lvl<T> C, Phys<T> P) {
   for (int q = 0; q < NU; ++q) C.f[q][idx] = fv[q] + M[q];
 }
 
-template <typename T, int NU, int DIM>
-__global__ void __launch_bounds__(TPB) k_gf_prolong(Lvl<T> F, Lvl<T> C, Phys<T> P) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < F.g.N) prolong_point<T, NU, DIM>(F, C, P, idx);
-}
-
 // ---------------------------------------------------------------------------
 // float64 kernels of the finest level
 // ---------------------------------------------------------------------------
@@ -481,7 +475,8 @@ struct GFSolver {
     FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
     const int rc = vcycle2(st, l + 1, P, &c_in_r);
     if (rc) return rc;
-    k_gf_prolong<T, NU, 2><<<nblocks(F.g.N), TPB, 0, s>>>(F, fz_view(C, c_in_r), P);
+    const int tp = point_tpb<T>(F.g.N, st->sms);
+    k_prolong<T, NU, 2><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, fz_view(C, c_in_r), P);
     FM_LAUNCHED();
     FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
     return FM_OK;
@@ -503,7 +498,8 @@ struct GFSolver {
     FM_LAUNCHED();
     rc = vcycle(st, l + 1, P);
     if (rc) return rc;
-    k_gf_prolong<T, NU, DIM><<<nblocks(F.g.N), TPB, 0, s>>>(F, C, P);
+    const int tp = point_tpb<T>(F.g.N, st->sms);
+    k_prolong<T, NU, DIM><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, C, P);
     FM_LAUNCHED();
     return smooth(st, F, P, st->prm.nu2);
   }

@@ -148,45 +148,4 @@ __device__ __forceinline__ T mcorr(T* const* E, const T* cr, int idx, T ce) {
   }
 }
 
-// M(e) = N(c + e) - N(c) at one point, all components (App. G operator N in
-// correction form about the coefficient iterate c).
-template <typename T, int KIND, int DIM>
-__device__ __forceinline__ void applyM(const Lvl<T>& L, const Phys<T>& P, const Nb& n,
-                                       T* const* E, T* M) {
-  using LY = Layout<KIND, DIM>;
-  const T ih = T(1) / L.h;
-  const T ih2 = ih * ih;
-  const T rkc = L.rk[n.c];
-  T div = 0;
-#pragma unroll
-  for (int d = 0; d < DIM; ++d)
-    div += L.rk[n.p[d]] * E[1 + d][n.p[d]] - L.rk[n.m[d]] * E[1 + d][n.m[d]];
-  M[0] = E[0][n.c] + P.s * T(0.25) * ih * div;
-
-  T ec[3], w[3], wx[3];
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) ec[d] = E[1 + d][n.c];
-#pragma unroll
-  for (int d = 0; d < LY::NOM; ++d) w[d] = L.om[d][n.c];
-  cross<T, DIM>(w, ec, wx);
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) {
-    const T dq = qcorr<T, DIM>(E, L.cv, n.p[a]) - qcorr<T, DIM>(E, L.cv, n.m[a]);
-    const T dm = mcorr<T, KIND, DIM>(E, L.cr, n.p[a], P.ce) - mcorr<T, KIND, DIM>(E, L.cr, n.m[a], P.ce);
-    const T lapa = (nbsum<T, DIM>(E[1 + a], n) - T(2 * DIM) * ec[a]) * ih2;
-    M[1 + a] = rkc * ec[a] + T(0.5) * P.sigma * P.s * rkc * wx[a]
-             + P.s * rkc * ih * (T(0.25) * dq + T(0.5) * dm)
-             - T(0.5) * P.s * P.gamma * lapa;
-  }
-  if constexpr (KIND == KPFC) {
-    const T er = E[0][n.c];
-    const T psi = L.cr[n.c] - T(1.5);
-    const T ek = E[LY::IKA][n.c];
-    const T lapk = (nbsum<T, DIM>(E[LY::IKA], n) - T(2 * DIM) * ek) * ih2;
-    const T lapr = (nbsum<T, DIM>(E[0], n) - T(2 * DIM) * er) * ih2;
-    M[LY::IMU] = E[LY::IMU][n.c] - er * (psi * psi + psi * er + er * er * T(1.0 / 3.0)) - P.alpha * er - lapk;
-    M[LY::IKA] = ek - lapr;
-  }
-}
-
 }  // namespace fm

@@ -486,6 +486,8 @@ struct Solver {
   using LY = Layout<KIND, DIM>;
   static constexpr int NVEL = DIM;  // velocity arrays of the state (copied by step_host)
 
+  static PtK<T> ptk(const Lvl<T>& L, const Phys<T>& P) { return make_ptk<T, DIM>(P, L.h); }
+
   static int inject_all(fm_state* st, bool coefficients_only) {
     if (st->nlev < 2) return FM_OK;
     InjAll<T> A;
@@ -535,13 +537,13 @@ struct Solver {
     const int nch = nz / Z;
     for (int c = 0; c < nch; ++c) {
       int rows = Z * ny;
-      k_smooth_rows<T, KIND, DIM><<<nblocks((long long)rows * half), TPB, 0, s>>>(L, P, 0, c * Z * ny, rows);
+      k_smooth_rows<T, KIND, DIM><<<nblocks((long long)rows * half), TPB, 0, s>>>(L, P, ptk(L, P), 0, c * Z * ny, rows);
       FM_LAUNCHED();
       const int b0 = c == 0 ? 1 : c * Z - 1;
       const int b1 = c == nch - 1 ? nz + 1 : (c + 1) * Z - 1;  // nz + 1: through nz - 1 and plane 0
       rows = (b1 - b0) * ny;
       if (rows > 0) {
-        k_smooth_rows<T, KIND, DIM><<<nblocks((long long)rows * half), TPB, 0, s>>>(L, P, 1, b0 * ny, rows);
+        k_smooth_rows<T, KIND, DIM><<<nblocks((long long)rows * half), TPB, 0, s>>>(L, P, ptk(L, P), 1, b0 * ny, rows);
         FM_LAUNCHED();
       }
     }
@@ -550,7 +552,7 @@ struct Solver {
 
   // Launch one sweep (a red and a black colour pass) of variant v (3-D) on level L.
   static int launch_colour_pair(fm_state* st, int v, const Lvl<T>& L, const Phys<T>& P) {
-    const int half = L.g.N / 2;
+    const int half = L.g.N / 2, tpb = point_tpb<T>(half, st->sms);
     if (v >= SM3_ZM) {
       if constexpr (DIM == 3) {
         const int rc = launch_zm3<T, KIND>(st, v, L, P, st->stream, 0);
@@ -565,9 +567,9 @@ struct Solver {
     }
     for (int color = 0; color < 2; ++color) {
       if (v == 1)
-        k_smooth_occ<T, KIND, DIM><<<nblocks(half), TPB, 0, st->stream>>>(L, P, color);
+        k_smooth_occ<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, st->stream>>>(L, P, ptk(L, P), color);
       else
-        k_smooth<T, KIND, DIM><<<nblocks(half), TPB, 0, st->stream>>>(L, P, color);
+        k_smooth<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, st->stream>>>(L, P, ptk(L, P), color);
       FM_LAUNCHED();
     }
     return FM_OK;
@@ -848,7 +850,7 @@ struct Solver {
   // around each launch.
   static int run_sweeps(fm_state* st, const Lvl<T>& L, int v, const Phys<T>& P, int iters, int* in_r, bool prof) {
     cudaStream_t s = st->stream;
-    const int half = L.g.N / 2;
+    const int half = L.g.N / 2, tpb = point_tpb<T>(half, st->sms);
     const int nfused = (DIM == 2 && v >= 0) ? (iters & ~1) : 0;
     const int per = v >= 0 ? sweeps_per_launch(v) : 1;
     if (DIM == 2 && v == RB_COOP && !coop_applies<T, KIND>(L)) v = -1;  // odd rows: two-colour launches
@@ -912,9 +914,9 @@ struct Solver {
             if (rc) return rc;
           }
         } else if (DIM == 3 && v == 1) {  // 3-D: v is the colour-sweep variant
-          k_smooth_occ<T, KIND, DIM><<<nblocks(half), TPB, 0, s>>>(*in_r ? swap_er(L) : L, P, color);
+          k_smooth_occ<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, s>>>(*in_r ? swap_er(L) : L, P, ptk(L, P), color);
         } else {
-          k_smooth<T, KIND, DIM><<<nblocks(half), TPB, 0, s>>>(*in_r ? swap_er(L) : L, P, color);
+          k_smooth<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, s>>>(*in_r ? swap_er(L) : L, P, ptk(L, P), color);
         }
         FM_LAUNCHED();
         if (prof && st->npev + 2 <= MAXEV) {
@@ -1117,6 +1119,7 @@ struct Solver {
       // operations per multiprocessor and clock)
       const Lvl<double> L64 = make_lvl_bufs<double>(st->lv64[l]);
       const int half = L64.g.N / 2;
+      const PtK<double> K64 = make_ptk<double, DIM>(P64, L64.h);
       // CDFT: the chemical-potential part of the points a launch updates is
       // kept in M (the level's float64 r[0], unused by these sweeps) for the
       // next launch
@@ -1125,11 +1128,11 @@ struct Solver {
         for (int color = 0; color < 2; ++color) {
           if constexpr (KIND == KCDFT) {
             if (it == 0 && color == 0)
-              k_smooth_cdft64_mc<DIM, false><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, color, M);
+              k_smooth_cdft64_mc<DIM, false><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color, M);
             else
-              k_smooth_cdft64_mc<DIM, true><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, color, M);
+              k_smooth_cdft64_mc<DIM, true><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color, M);
           } else {
-            k_smooth<double, KIND, DIM><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, color);
+            k_smooth<double, KIND, DIM><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color);
           }
           FM_LAUNCHED();
         }
@@ -1167,18 +1170,20 @@ struct Solver {
     Lvl<T> C = make_lvl<T>(st, l + 1);
     if constexpr (DIM == 2) {
       const int ntx = (C.g.nx + RR_TX - 1) / RR_TX, nty = (C.g.ny + RR_TY - 1) / RR_TY;
-      k_resid_restrict2<T, KIND><<<ntx * nty, TPB, 0, s>>>(F, C, P, ntx);
+      k_resid_restrict2<T, KIND><<<ntx * nty, TPB, 0, s>>>(F, C, P, ptk(F, P), ptk(C, P), ntx);
       FM_LAUNCHED();
     } else {
-      k_resid<T, KIND, DIM><<<nblocks(F.g.N), TPB, 0, s>>>(F, P);
+      const int tf = point_tpb<T>(F.g.N, st->sms), tc = point_tpb<T>(C.g.N, st->sms);
+      k_resid<T, KIND, DIM><<<blocks_of(F.g.N, tf), tf, 0, s>>>(F, P, ptk(F, P));
       FM_LAUNCHED();
-      k_restrict_rhs<T, KIND, DIM><<<nblocks(C.g.N), TPB, 0, s>>>(F, C, P);
+      k_restrict_rhs<T, KIND, DIM><<<blocks_of(C.g.N, tc), tc, 0, s>>>(F, C, P, ptk(C, P));
       FM_LAUNCHED();
     }
     int c_in_r = 0;
     rc = vcycle(st, l + 1, P, &c_in_r);
     if (rc) return rc;
-    k_prolong<T, LY::NU, DIM><<<nblocks(F.g.N), TPB, 0, s>>>(F, c_in_r ? swap_er(C) : C, P);
+    const int tp = point_tpb<T>(F.g.N, st->sms);
+    k_prolong<T, LY::NU, DIM><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, c_in_r ? swap_er(C) : C, P);
     FM_LAUNCHED();
     rc = smooth(st, l, P, st->prm.nu2, &in_r);
     if (rc) return rc;
