@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(TPB) kb_prolong(const WorkItem* items, int nit
   __syncthreads();
   lvl_swap_er(F, fswap);
   const int idx = lb * TPB + threadIdx.x;
-  if (idx < F.g.N) prolong_point<T, NU, 2>(F, Cc, P[inst], idx);
+  if (idx < Cc.g.N) prolong_cell<T, NU, 2>(F, Cc, P[inst], idx);
 }
 
 // one block per instance
@@ -540,7 +540,7 @@ struct Batch {
         const int ctx = (gc.nx + RR_TX - 1) / RR_TX, cty = (gc.ny + RR_TY - 1) / RR_TY;
         cr.push_back({i, ctx * cty});  // coarse tiles of the fused residual + restriction
         craux.push_back(ctx);
-        pr.push_back({i, nblocks(g.N)});
+        pr.push_back({i, nblocks(gc.N)});  // a thread per coarse point
       }
       for (int sh = 0; sh < 9; ++sh) b->w_smooth[sh][l] = add_list(b, ts[sh], &aux[sh]);
       b->w_resid[l] = add_list(b, rs);

@@ -612,10 +612,75 @@ __global__ void __launch_bounds__(TPB) k_resid(Lvl<T> L, Phys<T> P, PtK<T> K) {
   if (idx < L.g.N) resid_point<T, KIND, DIM>(L, P, K, idx);
 }
 
+// e_F += P(e_C - eh_C) (see prolong_point) for the 2^DIM fine points at and
+// after coarse point idx: the coarse differences of its 2^DIM parents are
+// formed once for all of them (2-D: 3 operations a value and component instead
+// of 5.4 point by point, and 2 loads of the coarse level instead of 4.5).
 template <typename T, int NU, int DIM>
-__global__ void __launch_bounds__(TPB) k_prolong(Lvl<T> F, Lvl<T> C, Phys<T> P) {
+__device__ __forceinline__ void prolong_cell(const Lvl<T>& F, const Lvl<T>& C, const Phys<T>& P, int idx) {
+  constexpr int NP = 1 << DIM;
+  int I, J, K;
+  coords(idx, C.g, I, J, K);
+  const int I1 = I + 1 == C.g.nx ? 0 : I + 1, J1 = J + 1 == C.g.ny ? 0 : J + 1, K1 = K + 1 == C.g.nz ? 0 : K + 1;
+  int ci[NP], fi[NP / 2];  // parents; first of each pair of fine points along x
+#pragma unroll
+  for (int p = 0; p < NP; ++p)
+    ci[p] = (((p & 4) ? K1 : K) * C.g.ny + ((p & 2) ? J1 : J)) * C.g.nx + ((p & 1) ? I1 : I);
+#pragma unroll
+  for (int p = 0; p < NP / 2; ++p)
+    fi[p] = ((DIM == 3 ? 2 * K + (p >> 1) : 0) * F.g.ny + 2 * J + (p & 1)) * F.g.nx + 2 * I;
+  const bool proj = P.delta > T(0);
+  T fe[NU][NP];  // loaded before the first store; the coarse level is read-only here
+#pragma unroll
+  for (int q = 0; q < NU; ++q)
+#pragma unroll
+    for (int p = 0; p < NP / 2; ++p) {
+      fe[q][2 * p] = F.e[q][fi[p]];
+      fe[q][2 * p + 1] = F.e[q][fi[p] + 1];
+    }
+#pragma unroll
+  for (int q = 0; q < NU; ++q) {
+    T d[NP];
+    T(&ev)[NP] = fe[q];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) d[p] = __ldg(C.e[q] + ci[p]) - __ldg(C.eh[q] + ci[p]);
+    // sums over the parents of each offset: along x, then y, then z
+    T s[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) s[p] = (p & 1) ? d[p - 1] + d[p] : d[p];
+#pragma unroll
+    for (int w = 2; w < NP; w *= 2) {
+      T t[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) t[p] = (p & w) ? s[p - w] + s[p] : s[p];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) s[p] = t[p];
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const T w = ((p & 1) ? T(0.5) : T(1)) * ((p & 2) ? T(0.5) : T(1)) * ((p & 4) ? T(0.5) : T(1));
+      ev[p] += w * s[p];
+    }
+    if (q == 0 && proj) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const T c = F.cr[fi[p >> 1] + (p & 1)], x = c + ev[p];
+        if (x <= proj_threshold<T>(P.delta)) ev[p] = proj_rho(x, P.delta) - c;
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < NP / 2; ++p) {
+      F.e[q][fi[p]] = ev[2 * p];
+      F.e[q][fi[p] + 1] = ev[2 * p + 1];
+    }
+  }
+}
+
+template <typename T, int NU, int DIM>
+__global__ void __launch_bounds__(TPB) k_prolong(const __grid_constant__ Lvl<T> F, const __grid_constant__ Lvl<T> C,
+                                                 Phys<T> P) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < F.g.N) prolong_point<T, NU, DIM>(F, C, P, idx);
+  if (idx < C.g.N) prolong_cell<T, NU, DIM>(F, C, P, idx);
 }
 
 // Fused red-black sweep of a 2-D level in TX x TY tiles.  The tile and a

@@ -475,8 +475,8 @@ struct GFSolver {
     FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
     const int rc = vcycle2(st, l + 1, P, &c_in_r);
     if (rc) return rc;
-    const int tp = point_tpb<T>(F.g.N, st->sms);
-    k_prolong<T, NU, 2><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, fz_view(C, c_in_r), P);
+    const int tp = point_tpb<T>(C.g.N, st->sms);
+    k_prolong<T, NU, 2><<<blocks_of(C.g.N, tp), tp, 0, s>>>(F, fz_view(C, c_in_r), P);
     FM_LAUNCHED();
     FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
     return FM_OK;
@@ -498,8 +498,8 @@ struct GFSolver {
     FM_LAUNCHED();
     rc = vcycle(st, l + 1, P);
     if (rc) return rc;
-    const int tp = point_tpb<T>(F.g.N, st->sms);
-    k_prolong<T, NU, DIM><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, C, P);
+    const int tp = point_tpb<T>(C.g.N, st->sms);
+    k_prolong<T, NU, DIM><<<blocks_of(C.g.N, tp), tp, 0, s>>>(F, C, P);
     FM_LAUNCHED();
     return smooth(st, F, P, st->prm.nu2);
   }

@@ -1182,8 +1182,8 @@ struct Solver {
     int c_in_r = 0;
     rc = vcycle(st, l + 1, P, &c_in_r);
     if (rc) return rc;
-    const int tp = point_tpb<T>(F.g.N, st->sms);
-    k_prolong<T, LY::NU, DIM><<<blocks_of(F.g.N, tp), tp, 0, s>>>(F, c_in_r ? swap_er(C) : C, P);
+    const int tp = point_tpb<T>(C.g.N, st->sms);
+    k_prolong<T, LY::NU, DIM><<<blocks_of(C.g.N, tp), tp, 0, s>>>(F, c_in_r ? swap_er(C) : C, P);
     FM_LAUNCHED();
     rc = smooth(st, l, P, st->prm.nu2, &in_r);
     if (rc) return rc;
