@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(rb_threads(TX, TY), rb_minb<T>(TX, TY)) kb_smo
                                                              int ntiles, int dir) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* buf0 = reinterpret_cast<T*>(smraw);
-  constexpr int BUFSTRIDE = rb_arrays<KIND, SF>() * RBGeom<TX, TY, NS>::SN;
+  constexpr int BUFSTRIDE = rb_slots<KIND, SF>() * RBGeom<TX, TY, NS>::SN;
   __shared__ Lvl<T> Gs[2];
   __shared__ int s_inst[2], s_x0[2], s_y0[2];
   int t = blockIdx.x;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(rb_threads(TX, TY), rb_minb<T>(TX, TY)) kb_smo
     fetch(t, 0);
     cp_async_wait_all();
     __syncthreads();
-    if (s_inst[0] >= 0) rb2d_compute<T, KIND, TX, TY, SF, NS>(Gs[0], P[s_inst[0]], 0, s_x0[0], s_y0[0], dir);
+    if (s_inst[0] >= 0) rb2d_compute<T, KIND, TX, TY, SF, NS>(Gs[0], P[s_inst[0]], make_ptk<T, 2>(P[s_inst[0]], Gs[0].h), 0, s_x0[0], s_y0[0], dir);
   } else {
     fetch(t, 0);
     for (int k = 0;; ++k) {
@@ -133,7 +133,8 @@ __global__ void __launch_bounds__(rb_threads(TX, TY), rb_minb<T>(TX, TY)) kb_smo
       __syncthreads();
       const int slot = k & 1;
       if (s_inst[slot] >= 0)
-        rb2d_compute<T, KIND, TX, TY, SF, NS>(Gs[slot], P[s_inst[slot]], slot * BUFSTRIDE, s_x0[slot], s_y0[slot],
+        rb2d_compute<T, KIND, TX, TY, SF, NS>(Gs[slot], P[s_inst[slot]], make_ptk<T, 2>(P[s_inst[slot]], Gs[slot].h),
+                                          slot * BUFSTRIDE, s_x0[slot], s_y0[slot],
                                           dir);
       __syncthreads();
       if (!next) break;
@@ -278,6 +279,16 @@ __global__ void __launch_bounds__(TPB) kb_prepare_mu(const WorkItem* items, int 
                                                      const Phys<double>* P64, const Step64* K64) {
   FM_BATCH_HEAD();
   prepare_mu_point<2>(D[inst].F, D[inst].g0, K64[inst], P64[inst], lb * TPB + threadIdx.x);
+}
+
+// FP64 path: the inverse determinants of level `level` of all instances (work
+// items: the level's points, as for kb_copy_back).
+__global__ void __launch_bounds__(TPB) kb_inverse(const WorkItem* items, int nitems, const InstDev<double>* D,
+                                                  const Phys<double>* P64, int level) {
+  FM_BATCH_HEAD();
+  const Lvl<double>& L = D[inst].lv[level];
+  const int idx = lb * TPB + threadIdx.x;
+  if (idx < L.g.N) iv_point<2>(L, make_ptk<double, 2>(P64[inst], L.h), idx);
 }
 
 template <typename T, int KIND>
@@ -799,6 +810,14 @@ struct Batch {
     if (wi.n) {
       kb_inject<T><<<wi.nblocks, TPB, 0, s>>>(it(b, wi), wi.n, D, b->ctl, 0, 0);
       FMB_LAUNCHED();
+    }
+    if constexpr (sizeof(T) == 8) {
+      for (int l = 0; l < b->maxdepth; ++l) {  // (the one-block levels form theirs point by point)
+        const WList& wl = b->w_resid[l];
+        if (!wl.n) continue;
+        kb_inverse<<<wl.nblocks, TPB, 0, s>>>(it(b, wl), wl.n, D, b->P64, l);
+        FMB_LAUNCHED();
+      }
     }
     return resid_norm(b, 0, hdl);
   }

@@ -24,6 +24,9 @@ struct CoopAcc {
   __device__ __forceinline__ T f(int q, int i) const { return __ldg(L.f[q] + i); }
   __device__ __forceinline__ T om(int d, int i) const { return __ldg(L.om[d] + i); }
 };
+struct CoopAccIv : CoopAcc<double> {
+  __device__ __forceinline__ double iv(int i) const { return __ldg(L.iv + i); }
+};
 
 // Grid-wide barrier number k (1, 2, ...) of a launch whose blocks are all
 // resident (cooperative launch): every block adds one arrival to bar[0] and
@@ -75,10 +78,13 @@ __device__ __forceinline__ void grid_barrier_leave(unsigned* bar) {
 // barrier wait runs out returns without leaving (*fault is set; the step
 // reports FM_ETIMEOUT).
 template <typename T, int KIND>
-__global__ void __launch_bounds__(TPB) k_smooth_coop(const __grid_constant__ Lvl<T> L, Phys<T> P, int nsweeps,
+__global__ void __launch_bounds__(TPB) k_smooth_coop(const __grid_constant__ Lvl<T> L, Phys<T> P, PtK<T> K, int nsweeps,
                                                      unsigned* bar, int* fault) {
-  const PtK<T> K = make_ptk<T, 2>(P, L.h);
-  const CoopAcc<T> a{L};
+  using Acc = std::conditional_t<sizeof(T) == 8, CoopAccIv, CoopAcc<T>>;
+  const Acc a = [&] {
+    if constexpr (sizeof(T) == 8) return CoopAccIv{{L}};
+    else return CoopAcc<T>{L};
+  }();
   const int half = L.g.N >> 1;
   const int stride = gridDim.x * blockDim.x;
   const int npass = 2 * nsweeps;

@@ -36,6 +36,7 @@ struct Lvl {
   T* r[MAXU];        // residual
   T* eh[MAXU];       // injected correction (coarse levels)
   const T* rk;       // rho^k
+  const T* iv;       // float64, FP64 path: inverse determinant of the velocity block (or null)
   const T* om[3];    // omega^k
   const T* cr;       // coefficient iterate: rho
   const T* cv[3];    // coefficient iterate: velocity
@@ -101,8 +102,6 @@ __device__ __forceinline__ bool colour_point(int t, int color, const Geo& g, int
 
 __device__ __forceinline__ float log1p_t(float x) { return log1pf(x); }
 __device__ __forceinline__ double log1p_t(double x) { return log1p(x); }
-__device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
 
 template <typename T, int DIM>
 __device__ __forceinline__ T nbsum(const T* a, const Nb& n) {

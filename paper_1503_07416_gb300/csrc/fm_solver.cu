@@ -143,7 +143,8 @@ static int launch_rb_v(fm_state* st, const Lvl<T>& L, const Phys<T>& P, cudaStre
   const int ntiles = ntx * ((L.g.ny + TY - 1) / TY);
   int grid = ntiles;
   if (PIPE && grid > per_sm * st->sms) grid = per_sm * st->sms;
-  k_smooth_rb2d<T, KIND, TX, TY, SF, PIPE, NS><<<grid, rb_threads(TX, TY), smem, s>>>(L, P, ntx, ntiles, dir);
+  k_smooth_rb2d<T, KIND, TX, TY, SF, PIPE, NS><<<grid, rb_threads(TX, TY), smem, s>>>(L, P, make_ptk<T, 2>(P, L.h), ntx,
+                                                                                            ntiles, dir);
   return FM_OK;
 }
 
@@ -215,7 +216,7 @@ static int launch_rb_tma(fm_state* st, const Lvl<T>& L, const Phys<T>& P, cudaSt
   const int ntx = (L.g.nx + TX - 1) / TX;
   const int ntiles = ntx * ((L.g.ny + TY - 1) / TY);
   k_smooth_rb2d_tma<T, KIND, TX, TY, NS><<<ntiles, rb_threads(TX, TY), smem, s>>>(
-      L, P, ntx, ntiles, dir, maps, &static_cast<Ctl*>(st->ctl)->fault);
+      L, P, make_ptk<T, 2>(P, L.h), ntx, ntiles, dir, maps, &static_cast<Ctl*>(st->ctl)->fault);
   return FM_OK;
 }
 
@@ -385,7 +386,7 @@ static int launch_coop(fm_state* st, const Lvl<T>& L, const Phys<T>& P, cudaStre
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   Ctl* ctl = static_cast<Ctl*>(st->ctl);
-  if (cudaLaunchKernelEx(&cfg, k_smooth_coop<T, KIND>, L, P, nsweeps, &ctl->gbar[0], &ctl->fault) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, k_smooth_coop<T, KIND>, L, P, make_ptk<T, 2>(P, L.h), nsweeps, &ctl->gbar[0], &ctl->fault) != cudaSuccess) {
     cudaGetLastError();
     return FM_ECUDA;
   }
@@ -708,7 +709,26 @@ struct Solver {
       k_prepare_mu<DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
       FM_LAUNCHED();
     }
-    return inject_all(st, false);
+    const int rc = inject_all(st, false);
+    if (rc) return rc;
+    if constexpr (sizeof(T) == 8) return inverses(st);
+    return FM_OK;
+  }
+
+  // FP64 path: the inverse determinants of the velocity blocks of every level.
+  static int inverses(fm_state* st) {
+    IvAll A;
+    memset(&A, 0, sizeof(A));
+    A.nl = st->nlev;
+    const Phys<double> P = make_phys<double>(st);
+    for (int l = 0; l < st->nlev; ++l) {
+      A.lv[l] = make_lvl<double>(st, l);
+      A.K[l] = make_ptk<double, DIM>(P, A.lv[l].h);
+      A.off[l + 1] = A.off[l] + st->lv[l].g.N;
+    }
+    k_inverse<DIM><<<blocks_of(A.off[st->nlev], 64), 64, 0, st->stream>>>(A);
+    FM_LAUNCHED();
+    return FM_OK;
   }
 
   static int prepare(fm_state* st) {
@@ -1343,6 +1363,9 @@ static size_t carve(fm_state* st, char* base) {
       B.eh[q] = (q < st->nu && l > 0) ? C.take(N * es) : nullptr;
     }
     const bool alias = (l == 0 && st->prm.precision == FM_FP64);
+    B.iv = (st->prm.precision == FM_FP64 && st->model == FM_HYDRO && st->prm.walls == FM_WALLS_NONE)
+               ? C.take(N * d8)
+               : nullptr;
     const int nvel = st->model == FM_HYDRO ? st->dim : 0;  // velocity coefficients
     if (alias) {
       B.rk = st->rho;

@@ -18,6 +18,7 @@ struct LevelBufs {
   void* f[MAXU];
   void* r[MAXU];
   void* eh[MAXU];
+  void* iv;        // float64, FP64 path: inverse determinant of the velocity block (or null)
   void* rk;        // precision-T rho^k (level 0 of the FP64 path: aliases st.rho)
   void* om[3];
   void* cr;        // precision-T coefficient iterate (level 0 FP64: aliases st.g)
