@@ -1951,7 +1951,8 @@ struct Fields64 {
 // are exact, the result is rounded once, and each value carries 6 bits more
 // than the largest float64, so the error is below that of the float64 sum
 // wherever a point's values are within a factor 16 of the set's largest.
-constexpr int FIX_EMIN = 128, FIX_EMAX = 1423;  // clamp below; above (2^400), or non-finite: plain float64
+constexpr int FIX_EMIN = 640, FIX_EMAX = 1423;  // clamp below (2^-383: products keep their exponents);
+                                                // above (2^400), or non-finite: plain float64
 
 __device__ __forceinline__ unsigned fix_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 __device__ __forceinline__ int fix_exp(double x) { return (int)(fix_mag(x) >> 20) - 1023; }  // floor(log2 |x|)
@@ -2376,6 +2377,10 @@ __device__ __forceinline__ void resid64_body(const Fields64& F, const Resid64Out
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
 }
 
+// The product of two values in fixed point (exponents ea, eb), in fixed point
+// with exponent ea + eb - 1023 + 2.
+__device__ __forceinline__ long long mul_fix(long long a, long long b) { return __mul64hi(a << 4, b); }
+
 // 2-D float64 residual in 32 x 8 tiles: the quantities every point shares
 // with its neighbours -- |u|^2 + 2 mu (mu the implicit chemical potential: the
 // unknown, or ln rho + 2 c_e rho), rho^k u, rho^k v -- are formed once per
@@ -2386,12 +2391,13 @@ __device__ __forceinline__ void resid64_body(const Fields64& F, const Resid64Out
 // Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 as in
 // resid64_body (same per-block accumulation order on every run).
 //
-// Bound by the float64 pipe: ~25 float64 instructions a point with the
-// neighbour sums in fixed point, 51 without.  The scales come from a first
+// Bound by the float64 pipe: ~18 float64 instructions a point with the
+// neighbour sums and the products they take in fixed point, 51 without.  The scales come from a first
 // pass over the tile's magnitudes (exponents only; its loads find the second
 // pass's in L1, which costs less than holding seven values a point in
-// registers over the barrier: 28.6 us a launch at 512^2 so, 24.9 now, 36.8 with
-// float64 sums; 24 instance ensemble, 11 M points, 12.1 -> 10.8 ms a step).
+// registers over the barrier: 28.6 us a launch at 512^2 so, 24.9 this way, 23.4
+// with integer products too, 36.8 with float64 sums and products; ensemble of
+// 24 instances, 7.8 M points: 12.1 -> 10.8 ms a step).
 // Against quad precision the rows' errors are at most what they were (rho
 // 3e-17 -> 4e-21, u 4.0e-19 -> 3.1e-19, kappa 2.5e-16 -> 6e-18 at 512^2).  Where a tile holds a value that fixed point
 // does not take (non-finite, beyond 2^400) its sums are float64.
@@ -2470,8 +2476,9 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
             em[1] <= FIX_EMAX;
       e_mu = max(em[2] + 2 + fix_exp(P.ce), 1023 + 32 - __clz(lg)) + 1;
     }
-    const int e_b = max(2 * em[0] - 1023 + 2, e_mu + 1) + 1;  // |u|^2 + 2 mu
-    const int e_ru = max(em[0] + em[1] - 1023 + 1, FIX_EMIN);
+    // rho^k u and |u|^2 + 2 mu (|u|^2 shifted down to the sum's scale)
+    const int e_ru = em[0] + em[1] - 1023 + 2, e_q = 2 * em[0] - 1023 + 2;
+    const int e_b = max(e_q + 1, e_mu + 1) + 1, sh_q = min(e_b - e_q, 63);
     for (int t = threadIdx.x; t < R64_SN; t += TPB) {
       const int gi = cell(t);
       const double u = g[1][gi], v = g[2][gi], rk = F.rho[gi];
@@ -2482,17 +2489,17 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
         const double r = g[0][gi];
         m = log(r) + 2.0 * P.ce * r;
       }
-      const double q = u * u + v * v, ru = rk * u, rv = rk * v;
       if (fix) {
-        sX[0][t] = to_fix(q, e_b) + 2 * to_fix(m, e_b);
-        sX[1][t] = to_fix(ru, e_ru);
-        sX[2][t] = to_fix(rv, e_ru);
-        sX[3][t] = to_fix(u, em[0]);
-        sX[4][t] = to_fix(v, em[0]);
+        const long long uf = to_fix(u, em[0]), vf = to_fix(v, em[0]), rf = to_fix(rk, em[1]);
+        sX[0][t] = ((mul_fix(uf, uf) + mul_fix(vf, vf)) >> sh_q) + 2 * to_fix(m, e_b);
+        sX[1][t] = mul_fix(uf, rf);
+        sX[2][t] = mul_fix(vf, rf);
+        sX[3][t] = uf;
+        sX[4][t] = vf;
       } else {
-        sX[0][t] = __double_as_longlong(q + 2.0 * m);
-        sX[1][t] = __double_as_longlong(ru);
-        sX[2][t] = __double_as_longlong(rv);
+        sX[0][t] = __double_as_longlong(u * u + v * v + 2.0 * m);
+        sX[1][t] = __double_as_longlong(rk * u);
+        sX[2][t] = __double_as_longlong(rk * v);
         sX[3][t] = __double_as_longlong(u);
         sX[4][t] = __double_as_longlong(v);
       }
@@ -2513,7 +2520,7 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
         const int xm = c - 1, xp = c + 1, ym = c - R64_SW, yp = c + R64_SW;
         double S[LY::NU];
 #pragma unroll
-        for (int q = 0; q < LY::NU; ++q) S[q] = F.S[q][idx];
+        for (int q = 0; q < (PFC ? LY::IKA : LY::NU); ++q) S[q] = F.S[q][idx];
         const double rkc = F.rho[idx], uc = g[1][idx], vc = g[2][idx], g0c = g[0][idx];
         const double w = F.om[0][idx];
         // 2h div(rho^k u), differences of |u|^2 + 2 mu, h^2 Lap of u, v (kappa, rho)
@@ -2542,7 +2549,7 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
         if constexpr (PFC) {
           const double psi = g0c - 1.5;
           rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap[2], fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][idx]));
-          rv[LY::IKA] = S[LY::IKA] - fma(-ih2, lap[3], g[LY::IKA][idx]);
+          rv[LY::IKA] = fma(ih2, lap[3], -g[LY::IKA][idx]);  // S_kappa = 0
         }
 #pragma unroll
         for (int q = 0; q < LY::NU; ++q) {
@@ -2710,7 +2717,7 @@ __device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64
 #pragma unroll
     for (int d = 0; d < LY::NOM; ++d) w[d] = c_w * F.om[d][n.c];
 #pragma unroll
-    for (int q = 0; q < LY::NU; ++q) S[q] = F.S[q][idx];
+    for (int q = 0; q < (PFC ? LY::IKA : LY::NU); ++q) S[q] = F.S[q][idx];
     rv[0] = fma(-c_div, dv, S[0] - g0c);
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
@@ -2727,7 +2734,7 @@ __device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64
       const double psi = g0c - 1.5, kc = g[LY::IKA][n.c];
       rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap(g[LY::IKA], kc, em[3]),
                                      fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][n.c]));
-      rv[LY::IKA] = S[LY::IKA] - fma(-ih2, lap(g[0], g0c, em[4]), kc);
+      rv[LY::IKA] = fma(ih2, lap(g[0], g0c, em[4]), -kc);  // S_kappa = 0
     }
 #pragma unroll
     for (int q = 0; q < LY::NU; ++q) {
@@ -2846,30 +2853,41 @@ static __global__ void k_hist_advance(Ctl* ctl) {
 // Block-level body: thread 0 returns whether the instance continues.
 //
 // One block between two launches of every cycle, so its latency counts in
-// full, and on GB300 that is the length of its chain of float64 instructions:
-// warp q sums component q (its partials in four running sums a lane, then
-// shuffles), thread 0 takes one square root, of the largest weighted sum
+// full, and on GB300 that is the length of its chains of loads and of float64
+// instructions: all partials are loaded at once, warp q sums component q of
+// the threads' sums, thread 0 takes one square root, of the largest weighted sum
 // (sqrt is monotone, so it is the largest of the square roots), and the
 // control block is read before the sums are known.
 template <int NQ>
 __device__ __forceinline__ bool norm_ctl_body(const double* partials, int nblk, double w, Ctl* ctl, double tol,
                                               int max_cycles, int in_body) {
   static_assert(NQ <= TPB / 32, "one warp per component");
-  __shared__ double sm[NQ];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NT = TPB / NQ * NQ;  // threads that sum: thread t takes component t % NQ of every NT-th value
+  __shared__ double part[NT], sm[NQ];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int fault = 0, nonpos = 0, done = 0;
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     fault = ctl->fault;
     nonpos = ctl->nonpos;
     done = ctl->cycles;
   }
-  if (warp < NQ) {
+  if (tid < NT) {
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = lane; b < nblk; b += 128)
+    const int n = nblk * NQ;
+    for (int b = tid; b < n; b += 16 * NT) {
+      double x[16];  // all loads in flight together
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (b + 32 * k < nblk) v[k] += partials[(b + 32 * k) * NQ + warp];
-    double x = (v[0] + v[1]) + (v[2] + v[3]);
+      for (int k = 0; k < 16; ++k) x[k] = b + k * NT < n ? partials[b + k * NT] : 0.0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (b + (k & ~3) * NT < n) v[k & 3] += x[k];
+    }
+    part[tid] = n > 2 * NT ? (v[0] + v[1]) + (v[2] + v[3]) : v[0] + v[1];
+  }
+  __syncthreads();
+  if (warp < NQ) {
+    double x = 0.0;
+    for (int k = lane; k < NT / NQ; k += 32) x += part[k * NQ + warp];
     for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
     if (lane == 0) sm[warp] = w * x;
   }
