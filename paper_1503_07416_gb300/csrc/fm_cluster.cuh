@@ -10,11 +10,10 @@
 //    where the device does not offer 16), 64 points to a block on the largest
 //    level, one warp of each colour;
 //  * the rows of the update are split over warps, hence partitions: one warp
-//    takes rho, kappa and mu (CDFT: rho and its chemical-potential part), one
-//    the neighbour sums of kappa and mu, one each velocity row; they exchange
-//    what they need of one another in shared memory.  The longest chain is
-//    then ~22 instead of ~90 instructions a pass; the transfers take one
-//    thread per point and component;
+//    takes rho (CDFT: and its chemical-potential part), one kappa and mu, one
+//    each velocity row; they exchange what they need of one another in shared
+//    memory.  The longest chain is then ~23 instead of ~90 instructions a pass;
+//    the transfers take one thread per point and component;
 //  * the inverse of the velocity block, which depends only on rho^k and
 //    omega^k, is formed once per launch.
 // A block keeps the records of its points (correction; CDFT: also its
@@ -27,9 +26,9 @@
 // with the integer conversions, so no conversion launch is needed.
 //
 // Measured (32^2 and 16^2 levels, V(2,2), 4 coarse sweeps, kernel time): PFC
-// 46 us, CDFT 58 us; one block on one multiprocessor (the form before) 221 and
+// 42 us, CDFT 58 us; one block on one multiprocessor (the form before) 221 and
 // 396 us; points split over the cluster but a whole point update a thread, 92
-// and 96 us.
+// and 96 us; kappa and mu finished by the rho role, 46 us.
 #pragma once
 
 #include "fm_device.cuh"
@@ -46,8 +45,9 @@ struct ClDim {
   static constexpr int NU = LY::NU;
   static constexpr int NR = NU + (KIND == KCDFT ? 1 : 0);  // doubles of a point's record: e, cdft_mc(e)
   static constexpr int NCO = 2 + DIM + LY::NOM;            // coefficients: rho^k, rho, u (DIM), omega^k (NOM)
-  static constexpr int NV = DIM == 2 ? 2 : 9;              // the velocity block's inverse: a I + b J, or a matrix
-  static constexpr int R = 1 + DIM + (KIND == KPFC ? 1 : 0);  // roles: rho (kappa, mu), velocities, PFC sums
+  static constexpr int NI = DIM == 2 ? 2 : 9;              // the velocity block's inverse: a I + b J, or a matrix
+  static constexpr int NV = NI + 1;                        // and s rho^k / (4 h)
+  static constexpr int R = 1 + DIM + (KIND == KPFC ? 1 : 0);  // roles: rho, velocities, PFC: kappa and mu
   static constexpr int SETS = CL_TPB / 32 / R;             // warps of each role in a block
 };
 
@@ -61,17 +61,18 @@ struct RolePt {
   int ni[2 * DIM];
   const double* nr[2 * DIM];  // m, p of each direction
 };
-// What role 0 carries from the first half of an update to the second.
+// What the rho role (a: rho) and the kappa and mu role (a, b: their neighbour
+// sums) carry from the first half of an update to the second.
 struct RoleRegs {
-  double er, cub;
+  double a, b;
 };
 
 // smooth_point_a's update of the point t in slot p of a pass, split over the
 // roles; a block barrier between the halves.  An accessor A gives rk(i),
 // cr(i), cv(d, i), f(q, i), the point's own record recp(i) and velocity-block
 // inverse ivp(i), keep_mc(i, e0, ce), and xch(k, p): value k of slot p in the
-// exchange area (0 .. DIM - 1 velocity right-hand sides, DIM and DIM + 1 the
-// kappa and mu sums).  Every value of another point is loaded before the first
+// exchange area (0 .. DIM - 1 velocity right-hand sides, DIM the new rho,
+// DIM + 1 its part of mu).  Every value of another point is loaded before the first
 // use, so that remote reads overlap.
 template <int KIND, int DIM>
 struct RoleUpdate {
@@ -105,9 +106,10 @@ struct RoleUpdate {
       if (x <= K.proj) er = proj_rho(x, P.delta) - crc;  // Sec. 6 projection
       if constexpr (KIND == KPFC) {
         const double psi = crc - 1.5;
-        g.cub = er * (psi * psi + psi * er + er * er * (1.0 / 3.0)) + P.alpha * er;
+        a.xch(DIM, p) = er;
+        a.xch(DIM + 1, p) = er * (psi * psi + psi * er + er * er * (1.0 / 3.0)) + P.alpha * er;
       }
-      g.er = er;
+      g.a = er;
     } else if (role == AUX) {
       if constexpr (KIND == KPFC) {
         double v[2 * DIM], k2[2 * DIM];
@@ -116,8 +118,8 @@ struct RoleUpdate {
           v[k] = t.nr[k][0];
           k2[k] = t.nr[k][LY::IKA];
         }
-        a.xch(DIM, p) = a.f(LY::IKA, t.idx) + sum(v) * K.ih2;
-        a.xch(DIM + 1, p) = a.f(LY::IMU, t.idx) + sum(k2) * K.ih2;
+        g.a = a.f(LY::IKA, t.idx) + sum(v) * K.ih2;
+        g.b = a.f(LY::IMU, t.idx) + sum(k2) * K.ih2;
       }
     } else {
 #pragma unroll
@@ -135,14 +137,14 @@ struct RoleUpdate {
               c[k][b] = a.cv(b, t.ni[2 * d + k]);
             }
           }
-          const double fd = a.f(1 + d, t.idx), cs = K.c_sih * a.rk(t.idx);
+          const double fd = a.f(1 + d, t.idx), cs = a.ivp(t.idx)[D::NI];
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             q[k] = 0;
 #pragma unroll
             for (int b = 0; b < DIM; ++b) q[k] += u[k][b] * (2.0 * c[k][b] + u[k][b]);
           }
-          a.xch(d, p) = fd - cs * (0.25 * (q[1] - q[0]) + 0.5 * (m[1] - m[0])) + K.c_v * sum(v);
+          a.xch(d, p) = fd - cs * ((q[1] - q[0]) + 2.0 * (m[1] - m[0])) + K.c_v * sum(v);
         }
     }
   }
@@ -153,16 +155,17 @@ struct RoleUpdate {
     const double w = P.w;
     double* eo = a.recp(t.idx);
     if (role == 0) {
+      const double er = (1.0 - w) * g.a + w * eo[0];
+      eo[0] = er;
+      if constexpr (KIND == KCDFT) a.keep_mc(t.idx, er, P.ce);
+    } else if (role == AUX) {
       if constexpr (KIND == KPFC) {
         const double c4 = 2.0 * DIM * K.ih2;
-        const double ek = a.xch(DIM, p) - c4 * g.er;
-        const double em = a.xch(DIM + 1, p) + g.cub - c4 * ek;
+        const double ek = g.a - c4 * a.xch(DIM, p);
+        const double em = g.b + a.xch(DIM + 1, p) - c4 * ek;
         eo[LY::IKA] = (1.0 - w) * ek + w * eo[LY::IKA];
         eo[LY::IMU] = (1.0 - w) * em + w * eo[LY::IMU];
       }
-      const double er = (1.0 - w) * g.er + w * eo[0];
-      eo[0] = er;
-      if constexpr (KIND == KCDFT) a.keep_mc(t.idx, er, P.ce);
     } else if (role <= DIM) {
       const double* v = a.ivp(t.idx);
       double eg;
@@ -175,7 +178,8 @@ struct RoleUpdate {
   }
 };
 
-// The inverse of the velocity block at a point (see smooth_point_a).
+// The inverse of the velocity block at a point (see smooth_point_a), and s
+// rho^k / (4 h) after it.
 template <int DIM>
 __device__ __forceinline__ void invert_block(const PtK<double>& K, double rk, const double* om, double* v) {
   const double Ad = rk + K.c_ad, bs = K.c_b * rk;
@@ -183,7 +187,9 @@ __device__ __forceinline__ void invert_block(const PtK<double>& K, double rk, co
     const double b = bs * om[0], inv = 1.0 / (Ad * Ad + b * b);
     v[0] = Ad * inv;
     v[1] = b * inv;
+    v[2] = 0.25 * K.c_sih * rk;
   } else {
+    v[9] = 0.25 * K.c_sih * rk;
     const double b[3] = {bs * om[0], bs * om[1], bs * om[2]};
     const double inv = 1.0 / (Ad * (Ad * Ad + b[0] * b[0] + b[1] * b[1] + b[2] * b[2]));
 #pragma unroll
