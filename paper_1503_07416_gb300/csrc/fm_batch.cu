@@ -271,7 +271,7 @@ template <typename T, int KIND>
 __global__ void __launch_bounds__(TPB) kb_prepare(const WorkItem* items, int nitems, const InstDev<T>* D,
                                                   const Phys<double>* P64, const Step64* K64) {
   FM_BATCH_HEAD();
-  prepare_point<KIND, 2>(D[inst].F, D[inst].g0, K64[inst], P64[inst], lb * TPB + threadIdx.x);
+  prepare_tile<KIND>(D[inst].F, D[inst].g0, K64[inst], P64[inst], lb);  // a tile a block
 }
 
 template <typename T>
@@ -385,7 +385,7 @@ struct fm_batch {
   Ctl* hctl;
   // work lists
   std::vector<WorkItem> hitems;
-  WList w_fine, w_resid64, w_inject;
+  WList w_fine, w_prep, w_resid64, w_inject;
   WList w_smooth[3 + 6][MAXLEV];  // per tile shape (32x16, 64x8, 32x32), then per marching variant
   WList w_resid[MAXLEV], w_rr[MAXLEV], w_prolong[MAXLEV];
   int rbv[MAXLEV];           // chosen fused-sweep variant per level
@@ -518,6 +518,9 @@ struct Batch {
     v.clear();
     for (int i = 0; i < b->count; ++i) v.push_back({i, nblocks(b->inst[i]->lv[0].g.N)});
     b->w_fine = add_list(b, v);
+    v.clear();
+    for (int i = 0; i < b->count; ++i) v.push_back({i, prep_tiles(b->inst[i]->lv[0].g.nx, b->inst[i]->lv[0].g.ny)});
+    b->w_prep = add_list(b, v);
     v.clear();
     for (int i = 0; i < b->count; ++i) v.push_back({i, b->inst[i]->nblk});
     b->w_resid64 = add_list(b, v);
@@ -799,8 +802,8 @@ struct Batch {
     }
     kb_set_active<<<(b->count + 255) / 256, 256, 0, s>>>(b->ctl, b->count);  // clears the flags
     FMB_LAUNCHED();
-    const WList& w = b->w_fine;
-    kb_prepare<T, KIND><<<w.nblocks, TPB, 0, s>>>(it(b, w), w.n, D, b->P64, b->K64);
+    const WList &w = b->w_fine, &wp = b->w_prep;
+    kb_prepare<T, KIND><<<wp.nblocks, TPB, 0, s>>>(it(b, wp), wp.n, D, b->P64, b->K64);
     FMB_LAUNCHED();
     if (KIND == KPFC) {
       kb_prepare_mu<T><<<w.nblocks, TPB, 0, s>>>(it(b, w), w.n, D, b->P64, b->K64);

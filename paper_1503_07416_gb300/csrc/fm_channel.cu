@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(TPB) k_ch_prepare_mu(Fields64 F, Geo G, Step64
 }
 
 // r = S - N(g) in float64 with the wall ghosts; the level-0 set-up of a
-// cycle and the block partial sums of r^2 (as resid64_body).
+// cycle and the block partial sums of r^2.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_ch_resid64(Fields64 F, Resid64Out O, Geo G, Step64 K, Phys<double> P,
                                                     Walls64 W, double* partials) {

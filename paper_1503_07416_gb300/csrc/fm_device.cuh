@@ -2072,9 +2072,139 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
   }
 }
 
-template <int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_prepare(Fields64 F, Geo G, Step64 K, Phys<double> P) {
-  prepare_point<KIND, DIM>(F, G, K, P, blockIdx.x * blockDim.x + threadIdx.x);
+// The product of two values in fixed point (exponents ea, eb), in fixed point
+// with exponent ea + eb - 1023 + 2.
+__device__ __forceinline__ long long mul_fix(long long a, long long b) { return __mul64hi(a << 4, b); }
+
+// Largest of the block's values m into sm (zero before; a barrier on each side).
+template <int NM>
+__device__ __forceinline__ void block_max(const unsigned (&m)[NM], unsigned* sm) {
+  __syncthreads();
+#pragma unroll
+  for (int a = 0; a < NM; ++a) {
+    const unsigned x = __reduce_max_sync(0xffffffffu, m[a]);
+    if ((threadIdx.x & 31) == 0) atomicMax(&sm[a], x);
+  }
+  __syncthreads();
+}
+
+// prepare_point on a 32 x 8 tile (tile `tile` of the grid's, one a block): u, v,
+// rho^k u, rho^k v (PFC: rho^k) of the tile and its one-point halo in fixed point
+// in shared memory, scaled by the tile's magnitudes as in the residual's tile.
+// 11 float64 instructions a point (PFC) instead of 37 on the pipe that bounded
+// it: 11.0 us at 512^2, 20.0 point by point.  Beyond FIX_EMAX the same body runs
+// in float64 (as a select in every value it cost a 512^2 film step 0.4%).
+constexpr int PT_TX = 32, PT_TY = 8, PT_SW = PT_TX + 2, PT_SN = PT_SW * (PT_TY + 2);
+__host__ __device__ constexpr int prep_tiles(int nx, int ny) {
+  return ((nx + PT_TX - 1) / PT_TX) * ((ny + PT_TY - 1) / PT_TY);
+}
+
+template <int KIND>
+__device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, const Step64& K, const Phys<double>& P,
+                                             int tile) {
+  using LY = Layout<KIND, 2>;
+  constexpr bool PFC = KIND == KPFC;
+  constexpr int NA = PFC ? 5 : 4;
+  __shared__ long long sX[NA][PT_SN];
+  __shared__ unsigned sMax[2];
+  const int nx = G.nx, ny = G.ny;
+  const int ntx = (nx + PT_TX - 1) / PT_TX;
+  const int x0 = (tile % ntx) * PT_TX, y0 = (tile / ntx) * PT_TY;
+  auto load = [&](int t, double& u, double& v, double& r) {
+    const int ly = t / PT_SW, lx = t - ly * PT_SW;
+    const int gi = wrapi(y0 + ly - 1, ny) * nx + wrapi(x0 + lx - 1, nx);
+    u = F.vel[0][gi];
+    v = F.vel[1][gi];
+    r = F.rho[gi];
+  };
+  if (threadIdx.x < 2) sMax[threadIdx.x] = 0u;
+  unsigned mag[2] = {0u, 0u};
+  for (int t = threadIdx.x; t < PT_SN; t += TPB) {
+    double u, v, r;
+    load(t, u, v, r);
+    mag[0] = max(mag[0], max(fix_mag(u), fix_mag(v)));
+    mag[1] = max(mag[1], fix_mag(r));
+  }
+  block_max(mag, sMax);
+  const int eu = max((int)(sMax[0] >> 20), FIX_EMIN), er = max((int)(sMax[1] >> 20), FIX_EMIN);
+  const int i = x0 + (threadIdx.x & 31), j = y0 + (threadIdx.x >> 5);
+  const bool own = i < nx && j < ny;
+  const int idx = own ? j * nx + i : 0;
+  // FIX: the staged values in fixed point; else (non-finite or huge ones) their float64 bits
+  auto finish = [&](auto fixed) {
+    constexpr bool FIX = decltype(fixed)::value;
+    auto fix = [](double x, int e) { return FIX ? to_fix(x, e) : __double_as_longlong(x); };
+    const int e_ru = eu + er - 1023 + 2;
+    for (int t = threadIdx.x; t < PT_SN; t += TPB) {
+      double ud, vd, rd;
+      load(t, ud, vd, rd);
+      const long long u = fix(ud, eu), v = fix(vd, eu), r = fix(rd, er);
+      sX[0][t] = u;
+      sX[1][t] = v;
+      sX[2][t] = FIX ? mul_fix(u, r) : __double_as_longlong(ud * rd);
+      sX[3][t] = FIX ? mul_fix(v, r) : __double_as_longlong(vd * rd);
+      if constexpr (PFC) sX[4][t] = r;
+    }
+    __syncthreads();
+    if (!own) return;
+    const int c = ((threadIdx.x >> 5) + 1) * PT_SW + (threadIdx.x & 31) + 1;
+    const int xm = c - 1, xp = c + 1, ym = c - PT_SW, yp = c + PT_SW;
+    // (a_{xp} - a_{xm}) + sg (b_{yp} - b_{ym}), and h^2 Lap
+    auto dif = [&](int a, int b, int sg, int e) {
+      if (FIX) return from_fix((sX[a][xp] - sX[a][xm]) + sg * (sX[b][yp] - sX[b][ym]), e);
+      auto x = [&](int q, int k) { return __longlong_as_double(sX[q][k]); };
+      return (x(a, xp) - x(a, xm)) + sg * (x(b, yp) - x(b, ym));
+    };
+    auto lap = [&](int a, int e) {
+      if (FIX) return from_fix((sX[a][xm] + sX[a][xp]) + (sX[a][ym] + sX[a][yp]) - (sX[a][c] << 2), e);
+      auto x = [&](int k) { return __longlong_as_double(sX[a][k]); };
+      return (x(xm) + x(xp) + x(ym) + x(yp)) - 4.0 * x(c);
+    };
+    const double w = K.hih * dif(1, 0, -1, eu);
+    const double div = dif(2, 3, 1, e_ru);
+    const double rk = F.rho[idx], uc[2] = {F.vel[0][idx], F.vel[1][idx]};
+    if constexpr (!PFC) {
+      if (F.nonpos && rk <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
+    }
+    const double cw = K.c_w * w;
+    double sv[2] = {fma(K.c_v, lap(0, eu), rk * fma(cw, uc[1], uc[0])),
+                    fma(K.c_v, lap(1, eu), rk * fma(-cw, uc[0], uc[1]))};
+    if constexpr (!PFC) {
+      const Nb n = neighbours(i, j, 0, G);
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const double Ep = 2.0 * P.ce * F.rho[n.p[a]] + F.conv[n.p[a]];
+        const double Em = 2.0 * P.ce * F.rho[n.m[a]] + F.conv[n.m[a]];
+        sv[a] += K.c_m * rk * (Ep - Em);
+      }
+    }
+    const double lapr = PFC ? lap(NA - 1, er) * K.ih2 : 0.0;
+    const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
+    F.S[0][idx] = fma(-K.c_div, div, rk);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      F.S[1 + a][idx] = sv[a];
+      if (!keep) F.g[1 + a][idx] = uc[a];
+    }
+    if (!keep) F.g[0][idx] = rk;
+    if constexpr (PFC) {
+      F.S[LY::IMU][idx] = 2.0 * lapr;
+      F.S[LY::IKA][idx] = 0.0;
+      if (!keep) F.g[LY::IKA][idx] = lapr;
+    }
+    F.om[0][idx] = w;
+    if (F.rk32) {
+      F.rk32[idx] = narrow_rn(rk);
+      F.om32[0][idx] = narrow_rn(w);
+    }
+  };
+  if (max(eu, er) <= FIX_EMAX) finish(std::true_type{});
+  else finish(std::false_type{});
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(TPB) k_prepare_tile(Fields64 F, Geo G, Step64 K, Phys<double> P) {
+  prepare_tile<KIND>(F, G, K, P, blockIdx.x);
 }
 
 // Largest of every thread's values into mag, one atomic a block and value.
@@ -2093,9 +2223,9 @@ __device__ __forceinline__ void grid_max(const unsigned (&m)[NM], unsigned* mag)
 }
 
 // 3-D: the largest magnitudes (high words) of the velocity and the density
-// into mag[0 .. 1] (zero before), and k_prepare with its neighbour sums scaled
-// by them.  k_prepare is bound by the float64 pipe, 60 instructions a point in
-// 3-D, 27 in fixed point; the extra pass reads four arrays.
+// into mag[0 .. 1] (zero before), and prepare_point with its neighbour sums
+// scaled by them: bound by the float64 pipe, 27 instructions a point, 60 with
+// the sums in float64; the extra pass reads four arrays.
 template <int DIM>
 __global__ void __launch_bounds__(TPB) k_prepare_mag(Fields64 F, int N, unsigned* mag) {
   unsigned m[2] = {0u, 0u};
@@ -2292,95 +2422,6 @@ struct Resid64Out {
   double* r64[MAXU];  // optional float64 residual output
 };
 
-// r = S - N(g) in float64 (App. G operator N, full form), block partials of r^2.
-// Block `lb` of `nb` blocks: strided loop over the points, partial sums of
-// r^2 into partials[lb][q].
-template <int KIND, int DIM, typename T>
-__device__ __forceinline__ void resid64_body(const Fields64& F, const Resid64Out& O, const Geo& G, const Step64& K,
-                                             const Phys<double>& P, double* partials, int lb, int nb) {
-  using LY = Layout<KIND, DIM>;
-  double acc[LY::NU];
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) acc[q] = 0.0;
-  float fa[LY::NU];
-#pragma unroll
-  for (int q = 0; q < LY::NU; ++q) fa[q] = 0.0f;
-  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_m = K.c_m, c_v = K.c_v;
-  const double third = 1.0 / 3.0;
-  for (int idx = lb * blockDim.x + threadIdx.x; idx < G.N; idx += nb * blockDim.x) {
-    int i, j, k;
-    coords(idx, G, i, j, k);
-    const Nb n = neighbours(i, j, k, G);
-    const double* const* g = F.g;
-    const double rkc = F.rho[n.c];
-    double N[LY::NU];
-    double div = 0;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d)
-      div += F.rho[n.p[d]] * g[1 + d][n.p[d]] - F.rho[n.m[d]] * g[1 + d][n.m[d]];
-    N[0] = g[0][n.c] + c_div * div;
-    double uc[3], w[3], wx[3];
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) uc[d] = g[1 + d][n.c];
-#pragma unroll
-    for (int d = 0; d < LY::NOM; ++d) w[d] = F.om[d][n.c];
-    cross<double, DIM>(w, uc, wx);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      double qp = 0, qm = 0;
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        const double up = g[1 + d][n.p[a]], um = g[1 + d][n.m[a]];
-        qp += up * up;
-        qm += um * um;
-      }
-      double mp, mm;
-      if constexpr (KIND == KPFC) {
-        mp = g[LY::IMU][n.p[a]];
-        mm = g[LY::IMU][n.m[a]];
-      } else {
-        const double rp = g[0][n.p[a]], rm = g[0][n.m[a]];
-        mp = log(rp) + 2.0 * P.ce * rp;
-        mm = log(rm) + 2.0 * P.ce * rm;
-      }
-      N[1 + a] = rkc * (uc[a] + c_w * wx[a] + c_q * (qp - qm) + c_m * (mp - mm))
-               - c_v * (nbsum<double, DIM>(g[1 + a], n) - 2.0 * DIM * uc[a]);
-    }
-    if constexpr (KIND == KPFC) {
-      const double rc = g[0][n.c];
-      const double psi = rc - 1.5;
-      const double kc = g[LY::IKA][n.c];
-      // h^2 Lap_h kappa and h^2 Lap_h rho; the 1/h^2 scale and the cubic (Horner form)
-      // go into fused multiply-adds (fewer float64 instructions, the same rows)
-      const double dk = nbsum<double, DIM>(g[LY::IKA], n) - 2.0 * DIM * kc;
-      const double dr = nbsum<double, DIM>(g[0], n) - 2.0 * DIM * rc;
-      N[LY::IMU] = fma(-ih2, dk, g[LY::IMU][n.c] - psi * fma(psi * psi, third, P.alpha));
-      N[LY::IKA] = fma(-ih2, dr, kc);
-    }
-    double rv[LY::NU];  // all loads (S, rho) before the first store
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) rv[q] = F.S[q][idx] - N[q];
-    const double g0c = g[0][idx];
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) {
-      const double r = rv[q];
-      norm_add<T>(O.f0[q], r, acc[q], fa[q], idx);
-      if (O.e0[q]) static_cast<T*>(O.e0[q])[idx] = T(0);
-      if (O.r64[q]) O.r64[q][idx] = r;
-    }
-    if (O.cr32) {
-      O.cr32[idx] = narrow_rn(g0c);
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) O.cv32[d][idx] = narrow_rn(uc[d]);
-    }
-  }
-  norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
-}
-
-// The product of two values in fixed point (exponents ea, eb), in fixed point
-// with exponent ea + eb - 1023 + 2.
-__device__ __forceinline__ long long mul_fix(long long a, long long b) { return __mul64hi(a << 4, b); }
-
 // 2-D float64 residual in 32 x 8 tiles: the quantities every point shares
 // with its neighbours -- |u|^2 + 2 mu (mu the implicit chemical potential: the
 // unknown, or ln rho + 2 c_e rho), rho^k u, rho^k v -- are formed once per
@@ -2388,8 +2429,8 @@ __device__ __forceinline__ long long mul_fix(long long a, long long b) { return 
 // kappa and rho) beside them, all in fixed point; then N is evaluated on the
 // tile.  |u|^2 and 2 mu are one quantity because the coefficient of the
 // chemical potential's gradient, s/(2h), is twice the kinetic one, s/(4h).
-// Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 as in
-// resid64_body (same per-block accumulation order on every run).
+// Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 per block
+// (the same accumulation order on every run).
 //
 // Bound by the float64 pipe: ~18 float64 instructions a point with the
 // neighbour sums and the products they take in fixed point, 51 without.  The scales come from a first
@@ -2452,13 +2493,7 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
         mag[3] = max(mag[3], r > 0.0 ? 0x7ff00000u - min(fix_mag(r), 0x7ff00000u) : 0x7ff00000u);
       }
     }
-    __syncthreads();  // sMax is zero, the tile before is finished
-#pragma unroll
-    for (int a = 0; a < NM; ++a) {
-      const unsigned m = __reduce_max_sync(0xffffffffu, mag[a]);
-      if ((threadIdx.x & 31) == 0) atomicMax(&sMax[a], m);
-    }
-    __syncthreads();
+    block_max(mag, sMax);  // (sMax is zero; its first barrier: the tile before is finished)
     int em[NM];
     bool fix = true;
 #pragma unroll
@@ -2764,12 +2799,6 @@ __global__ void __launch_bounds__(TPB, 4) k_resid64_x(Fields64 F, Shared64 X, Re
   }
   if (fix) resid64_x_body<KIND, DIM, T, true>(F, X, O, G, K, P, partials, em);
   else resid64_x_body<KIND, DIM, T, false>(F, X, O, G, K, P, partials, em);
-}
-
-template <int KIND, int DIM, typename T>
-__global__ void __launch_bounds__(TPB) k_resid64(Fields64 F, Resid64Out O, Geo G, Step64 K,
-                                                 Phys<double> P, double* partials) {
-  resid64_body<KIND, DIM, T>(F, O, G, K, P, partials, blockIdx.x, gridDim.x);
 }
 
 // g += e (float64), then the projection of Sec. 6 on rho.

@@ -702,7 +702,7 @@ struct Solver {
       FM_LAUNCHED();
       k_prepare_fix<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P, st->mag);
     } else {
-      k_prepare<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
+      k_prepare_tile<KIND><<<prep_tiles(G.nx, G.ny), TPB, 0, s>>>(F, G, K, P);
     }
     FM_LAUNCHED();
     if (KIND == KPFC) {
