@@ -2088,6 +2088,26 @@ __device__ __forceinline__ void block_max(const unsigned (&m)[NM], unsigned* sm)
   __syncthreads();
 }
 
+// Walls at y = 0 and y = ny h moving along x (the channel): in the tile kernels
+// the halo row beyond a wall holds the ghosts of App. E.2, scalars mirrored, the
+// normal velocity odd, the tangential one 2 U - u.
+struct Walls64 {
+  double ub, ut;
+};
+template <bool WALLS>
+__device__ __forceinline__ int tile_row(int y, int ny) {
+  return WALLS ? min(max(y, 0), ny - 1) : wrapi(y, ny);
+}
+template <bool WALLS>
+__device__ __forceinline__ void ghost_velocity(double& u, double& v, int y, int ny, const Walls64& W) {
+  if constexpr (WALLS) {
+    if (y < 0 || y >= ny) {
+      u = 2.0 * (y < 0 ? W.ub : W.ut) - u;
+      v = -v;
+    }
+  }
+}
+
 // prepare_point on a 32 x 8 tile (tile `tile` of the grid's, one a block): u, v,
 // rho^k u, rho^k v (PFC: rho^k) of the tile and its one-point halo in fixed point
 // in shared memory, scaled by the tile's magnitudes as in the residual's tile.
@@ -2099,9 +2119,9 @@ __host__ __device__ constexpr int prep_tiles(int nx, int ny) {
   return ((nx + PT_TX - 1) / PT_TX) * ((ny + PT_TY - 1) / PT_TY);
 }
 
-template <int KIND>
+template <int KIND, bool WALLS = false>
 __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, const Step64& K, const Phys<double>& P,
-                                             int tile) {
+                                             int tile, const Walls64& W = Walls64{}) {
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
   constexpr int NA = PFC ? 5 : 4;
@@ -2111,11 +2131,12 @@ __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, co
   const int ntx = (nx + PT_TX - 1) / PT_TX;
   const int x0 = (tile % ntx) * PT_TX, y0 = (tile / ntx) * PT_TY;
   auto load = [&](int t, double& u, double& v, double& r) {
-    const int ly = t / PT_SW, lx = t - ly * PT_SW;
-    const int gi = wrapi(y0 + ly - 1, ny) * nx + wrapi(x0 + lx - 1, nx);
+    const int ly = t / PT_SW, lx = t - ly * PT_SW, y = y0 + ly - 1;
+    const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
     u = F.vel[0][gi];
     v = F.vel[1][gi];
     r = F.rho[gi];
+    ghost_velocity<WALLS>(u, v, y, ny, W);
   };
   if (threadIdx.x < 2) sMax[threadIdx.x] = 0u;
   unsigned mag[2] = {0u, 0u};
@@ -2445,10 +2466,11 @@ struct Resid64Out {
 constexpr int R64_TX = 32, R64_TY = 8;
 constexpr int R64_SW = R64_TX + 2, R64_SN = R64_SW * (R64_TY + 2);
 
-template <int KIND, typename T>
+template <int KIND, typename T, bool WALLS = false>
 __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid64Out& O, const Geo& G,
                                                   const Step64& K,
-                                                  const Phys<double>& P, double* partials, int lb, int nb) {
+                                                  const Phys<double>& P, double* partials, int lb, int nb,
+                                                  const Walls64& W = Walls64{}) {
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
   // staged: |u|^2 + 2 mu, rho^k u, rho^k v, u, v (PFC: kappa, rho)
@@ -2472,16 +2494,22 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
   if (threadIdx.x < NM) sMax[threadIdx.x] = 0u;
   for (int tile = lb; tile < ntiles; tile += nb) {
     const int x0 = (tile % ntx) * R64_TX, y0 = (tile / ntx) * R64_TY;
-    auto cell = [&](int t) {
-      const int ly = t / R64_SW, lx = t - ly * R64_SW;
-      return wrapi(y0 + ly - 1, ny) * nx + wrapi(x0 + lx - 1, nx);
+    // grid index of staged cell t and the velocity there (a ghost beyond a wall)
+    auto cell = [&](int t, double& u, double& v) {
+      const int ly = t / R64_SW, lx = t - ly * R64_SW, y = y0 + ly - 1;
+      const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
+      u = g[1][gi];
+      v = g[2][gi];
+      ghost_velocity<WALLS>(u, v, y, ny, W);
+      return gi;
     };
     unsigned mag[NM];
 #pragma unroll
     for (int a = 0; a < NM; ++a) mag[a] = 0u;
     for (int t = threadIdx.x; t < R64_SN; t += TPB) {
-      const int gi = cell(t);
-      mag[0] = max(mag[0], max(fix_mag(g[1][gi]), fix_mag(g[2][gi])));
+      double u, v;
+      const int gi = cell(t, u, v);
+      mag[0] = max(mag[0], max(fix_mag(u), fix_mag(v)));
       mag[1] = max(mag[1], fix_mag(F.rho[gi]));
       if constexpr (PFC) {
         mag[2] = max(mag[2], fix_mag(g[LY::IMU][gi]));
@@ -2515,9 +2543,9 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
     const int e_ru = em[0] + em[1] - 1023 + 2, e_q = 2 * em[0] - 1023 + 2;
     const int e_b = max(e_q + 1, e_mu + 1) + 1, sh_q = min(e_b - e_q, 63);
     for (int t = threadIdx.x; t < R64_SN; t += TPB) {
-      const int gi = cell(t);
-      const double u = g[1][gi], v = g[2][gi], rk = F.rho[gi];
-      double m;
+      double u, v, m;
+      const int gi = cell(t, u, v);
+      const double rk = F.rho[gi];
       if constexpr (PFC) {
         m = g[LY::IMU][gi];
       } else {

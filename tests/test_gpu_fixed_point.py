@@ -40,7 +40,7 @@ def _close(got, want):
 # planes that do not fill the last block
 GRIDS = [("pfc", (36, 20)), ("pfc", (2, 70)), ("pfc", (70, 2)), ("pfc", (130, 72)), ("pfc", (10, 6, 14)),
          ("pfc", (64, 4, 2)), ("cdft", (64, 32)), ("cdft", (16, 8, 32))]
-CASES = [(k, n, m) for k, n in GRIDS for m in ("periodic",)]
+CASES = [(k, n, m) for k, n in GRIDS for m in ("periodic", "walls", "gradflow") if m == "periodic" or len(n) == 2 and k == "pfc"]
 
 
 @pytest.mark.parametrize("vel_of", ["ordinary", "zero", "spike"])
