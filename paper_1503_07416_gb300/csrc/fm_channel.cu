@@ -169,38 +169,44 @@ __device__ __forceinline__ void ch_restrict(const Lvl<T>& F, const Lvl<T>& C, in
   }
 }
 
-// Coefficients of the finest level injected into every coarser level, one
-// launch: a level's value is the mean of the two fine cells of the level
+// Coefficients of the finest level injected into every coarser level at once: a
+// level's value is the mean of the two fine cells of the level
 // above at x = 2I, so level l takes the pairwise means over 2^l rows, eight
 // rows loaded at a time.
+struct InjRows {
+  template <typename T>
+  static __device__ __forceinline__ void point(const InjAll<T>& A, int t) {
+    if (t >= A.off[A.nl]) return;
+    int l = 1;
+    while (t >= A.off[l + 1]) ++l;
+    const int idx = t - A.off[l], I = idx % A.g[l].nx, J = idx / A.g[l].nx;
+    const int nx = A.g0.nx, nb = (1 << l) >= 8 ? (1 << l) / 8 : 1, step = (1 << l) >= 8 ? 8 : 1 << l;
+    for (int q = 0; q < A.nsrc; ++q) {
+      const T* src = A.src[q] + (size_t)(J << l) * nx + (I << l);
+      T part[MAXLEV];  // part[k]: the mean of 8 2^k rows waiting for its pair
+      T v = T(0);
+      for (int b = 0; b < nb; ++b, src += (size_t)8 * nx) {
+        T r[8];
+  #pragma unroll
+        for (int k = 0; k < 8; ++k) r[k] = k < step ? src[(size_t)k * nx] : T(0);
+  #pragma unroll
+        for (int w = 1; w < 8; w *= 2)
+          if (w < step)
+  #pragma unroll
+            for (int k = 0; k < 8; k += 2 * w) r[k] = T(0.5) * (r[k] + r[k + w]);
+        v = r[0];
+        int k = 0;
+        for (int n = b; n & 1; n >>= 1, ++k) v = T(0.5) * (part[k] + v);
+        part[k] = v;
+      }
+      A.dst[l][q][idx] = v;
+    }
+  }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_ch_inject_all(const __grid_constant__ InjAll<T> A) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= A.off[A.nl]) return;
-  int l = 1;
-  while (t >= A.off[l + 1]) ++l;
-  const int idx = t - A.off[l], I = idx % A.g[l].nx, J = idx / A.g[l].nx;
-  const int nx = A.g0.nx, nb = (1 << l) >= 8 ? (1 << l) / 8 : 1, step = (1 << l) >= 8 ? 8 : 1 << l;
-  for (int q = 0; q < A.nsrc; ++q) {
-    const T* src = A.src[q] + (size_t)(J << l) * nx + (I << l);
-    T part[MAXLEV];  // part[k]: the mean of 8 2^k rows waiting for its pair
-    T v = T(0);
-    for (int b = 0; b < nb; ++b, src += (size_t)8 * nx) {
-      T r[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) r[k] = k < step ? src[(size_t)k * nx] : T(0);
-#pragma unroll
-      for (int w = 1; w < 8; w *= 2)
-        if (w < step)
-#pragma unroll
-          for (int k = 0; k < 8; k += 2 * w) r[k] = T(0.5) * (r[k] + r[k + w]);
-      v = r[0];
-      int k = 0;
-      for (int n = b; n & 1; n >>= 1, ++k) v = T(0.5) * (part[k] + v);
-      part[k] = v;
-    }
-    A.dst[l][q][idx] = v;
-  }
+  InjRows::point(A, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Fine cell idx: e_F += P(e_C - eh_C): x linear between nodes, y linear
@@ -380,8 +386,7 @@ struct ChannelSolver {
 
   // rho^k and omega^k (which = 0) or the coefficient iterate rho, u, v
   // (which = 1) of the finest level down the hierarchy.
-  static int inject(fm_state* st, int which) {
-    if (st->nlev < 2) return FM_OK;
+  static InjAll<T> injection(fm_state* st, int which) {
     InjAll<T> A;
     memset(&A, 0, sizeof(A));
     A.nl = st->nlev;
@@ -397,9 +402,7 @@ struct ChannelSolver {
       A.g[l] = B.g;
       A.off[l + 1] = l == 0 ? 0 : A.off[l] + B.g.N;
     }
-    k_ch_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
-    FM_LAUNCHED();
-    return FM_OK;
+    return A;
   }
 
   static int enqueue_prepare(fm_state* st) {
@@ -409,7 +412,12 @@ struct ChannelSolver {
     FM_LAUNCHED();
     k_ch_prepare_mu<<<nblocks(G.N), TPB, 0, st->stream>>>(F, G, step64(st), st->fn.alpha, walls64(st));
     FM_LAUNCHED();
-    return inject(st, 0);
+    if (st->nlev > 1) {
+      const InjAll<T> A = injection(st, 0);
+      k_ch_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
+      FM_LAUNCHED();
+    }
+    return FM_OK;
   }
 
   static int launch_resid64(fm_state* st, const Resid64Out& O) {
@@ -423,8 +431,9 @@ struct ChannelSolver {
     int rc = launch_resid64(st, out0(st, true, nullptr));
     if (rc) return rc;
     const double h = st->lv[0].h;
-    k_norm_ctl<LY::NU><<<1, TPB, 0, st->stream>>>(st->partials, st->nblk, h * h, (Ctl*)st->ctl, st->prm.tol,
-                                                  st->prm.max_cycles, in_body, hdl, use_handle);
+    const InjAll<T> A = injection(st, 1);
+    k_norm_ctl<LY::NU, InjRows, T><<<1 + nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(
+        st->partials, st->nblk, h * h, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -461,10 +470,8 @@ struct ChannelSolver {
   }
 
   static int enqueue_body(fm_state* st, cudaGraphConditionalHandle hdl, int use_handle) {
-    int rc = inject(st, 1);
-    if (rc) return rc;
     int in_r = 0;
-    rc = vcycle(st, 0, make_phys<T>(st), &in_r);
+    int rc = vcycle(st, 0, make_phys<T>(st), &in_r);
     if (rc) return rc;
     const Geo G = st->lv[0].g;
     Resid64Out O = out0(st, true, nullptr);

@@ -1814,6 +1814,13 @@ __global__ void __launch_bounds__(TPB) k_inject_all(InjAll<T> A) {
   inject_all_point<T>(A, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
+struct InjSample {
+  template <typename T>
+  static __device__ __forceinline__ void point(const InjAll<T>& A, int t) {
+    inject_all_point<T>(A, t);
+  }
+};
+
 // --------------------------------------------------------------------------
 // float64 kernels of the finest level
 // --------------------------------------------------------------------------
@@ -2974,9 +2981,20 @@ __device__ __forceinline__ bool norm_ctl_body(const double* partials, int nblk, 
   return false;
 }
 
-template <int NQ>
-__global__ void k_norm_ctl(const double* partials, int nblk, double w, Ctl* ctl, double tol, int max_cycles,
-                           int in_body, cudaGraphConditionalHandle handle, int use_handle) {
+// Block 0: the norm and the control update.  The other blocks: the coefficients
+// of the next cycle, which the residual launch has just written on the finest
+// level, down to the coarser ones (the last residual of a step writes them
+// unused).  The norm takes one block 5 us and waits on latency only, so the
+// injection beside it takes no time of its own (512^2: 5.0 us alone, 5.3 with
+// it); as a launch at the head of a cycle it took 3.4 us, channel 6.2.
+template <int NQ, typename INJ, typename T>
+__global__ void __launch_bounds__(TPB) k_norm_ctl(const double* partials, int nblk, double w, Ctl* ctl, double tol,
+                                                  int max_cycles, int in_body, cudaGraphConditionalHandle handle,
+                                                  int use_handle, const __grid_constant__ InjAll<T> A) {
+  if (blockIdx.x > 0) {
+    INJ::point(A, (blockIdx.x - 1) * TPB + threadIdx.x);
+    return;
+  }
   const bool cont = norm_ctl_body<NQ>(partials, nblk, w, ctl, tol, max_cycles, in_body);
   if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, cont ? 1u : 0u);
 }

@@ -521,13 +521,30 @@ struct GFSolver {
     return FM_OK;
   }
 
+  // The coefficient density of level 0 (precision T) down the hierarchy.
+  static InjAll<T> injection(fm_state* st) {
+    InjAll<T> A;
+    memset(&A, 0, sizeof(A));
+    A.nl = st->nlev;
+    A.g0 = st->lv[0].g;
+    A.nsrc = 1;
+    A.src[0] = (const T*)st->lv[0].cr;
+    for (int l = 1; l < st->nlev; ++l) {
+      A.g[l] = st->lv[l].g;
+      A.off[l + 1] = A.off[l] + st->lv[l].g.N;
+      A.dst[l][0] = (T*)st->lv[l].cr;
+    }
+    return A;
+  }
+
   static int enqueue_resid_norm(fm_state* st, int in_body, cudaGraphConditionalHandle hdl, int use_handle) {
     int rc = launch_resid64(st, out0(st, true, nullptr));
     if (rc) return rc;
     const double h = st->lv[0].h;
     const double w = DIM == 3 ? h * h * h : h * h;
-    k_norm_ctl<NU><<<1, TPB, 0, st->stream>>>(st->partials, st->nblk, w, (Ctl*)st->ctl, st->prm.tol,
-                                              st->prm.max_cycles, in_body, hdl, use_handle);
+    const InjAll<T> A = injection(st);
+    k_norm_ctl<NU, InjSample, T><<<1 + nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(
+        st->partials, st->nblk, w, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -596,30 +613,8 @@ struct GFSolver {
     return smooth(st, F, P, st->prm.nu2);
   }
 
-  // The coefficient density of level 0 (precision T) down the hierarchy.
-  static int inject_coefficient(fm_state* st) {
-    if (st->nlev < 2) return FM_OK;
-    InjAll<T> A;
-    memset(&A, 0, sizeof(A));
-    A.nl = st->nlev;
-    A.g0 = st->lv[0].g;
-    A.off[0] = A.off[1] = 0;
-    for (int l = 1; l < st->nlev; ++l) {
-      A.g[l] = st->lv[l].g;
-      A.off[l + 1] = A.off[l] + st->lv[l].g.N;
-    }
-    A.src[0] = (const T*)st->lv[0].cr;
-    for (int l = 1; l < st->nlev; ++l) A.dst[l][0] = (T*)st->lv[l].cr;
-    A.nsrc = 1;
-    k_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
-    FM_LAUNCHED();
-    return FM_OK;
-  }
-
   static int enqueue_body(fm_state* st, cudaGraphConditionalHandle hdl, int use_handle) {
-    int rc = inject_coefficient(st);
-    if (rc) return rc;
-    int in_r = 0;
+    int rc, in_r = 0;
     if constexpr (DIM == 2) rc = vcycle2(st, 0, make_phys<T>(st), &in_r);
     else rc = vcycle(st, 0, make_phys<T>(st));
     if (rc) return rc;

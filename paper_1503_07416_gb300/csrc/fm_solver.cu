@@ -489,39 +489,25 @@ struct Solver {
 
   static PtK<T> ptk(const Lvl<T>& L, const Phys<T>& P) { return make_ptk<T, DIM>(P, L.h); }
 
-  static int inject_all(fm_state* st, bool coefficients_only) {
-    if (st->nlev < 2) return FM_OK;
+  // rho^k and omega^k, or the coefficient iterate, of the finest level down
+  // the hierarchy.
+  static InjAll<T> injection(fm_state* st, bool iterate) {
     InjAll<T> A;
     memset(&A, 0, sizeof(A));
     A.nl = st->nlev;
     A.g0 = st->lv[0].g;
-    A.off[0] = A.off[1] = 0;
-    for (int l = 1; l < st->nlev; ++l) {
-      A.g[l] = st->lv[l].g;
-      A.off[l + 1] = A.off[l] + st->lv[l].g.N;
-    }
-    int q = 0;
-    if (coefficients_only) {
-      A.src[q] = (const T*)st->lv[0].cr;
-      for (int l = 1; l < st->nlev; ++l) A.dst[l][q] = (T*)st->lv[l].cr;
-      ++q;
-      for (int d = 0; d < DIM; ++d, ++q) {
-        A.src[q] = (const T*)st->lv[0].cv[d];
-        for (int l = 1; l < st->nlev; ++l) A.dst[l][q] = (T*)st->lv[l].cv[d];
+    A.nsrc = 1 + (iterate ? DIM : LY::NOM);
+    for (int l = 0; l < st->nlev; ++l) {
+      const LevelBufs& B = st->lv[l];
+      for (int q = 0; q < A.nsrc; ++q) {
+        T* v = (T*)(iterate ? (q ? B.cv[q - 1] : B.cr) : (q ? B.om[q - 1] : B.rk));
+        if (l == 0) A.src[q] = v;
+        else A.dst[l][q] = v;
       }
-    } else {
-      A.src[q] = (const T*)st->lv[0].rk;
-      for (int l = 1; l < st->nlev; ++l) A.dst[l][q] = (T*)st->lv[l].rk;
-      ++q;
-      for (int d = 0; d < LY::NOM; ++d, ++q) {
-        A.src[q] = (const T*)st->lv[0].om[d];
-        for (int l = 1; l < st->nlev; ++l) A.dst[l][q] = (T*)st->lv[l].om[d];
-      }
+      A.g[l] = B.g;
+      A.off[l + 1] = l == 0 ? 0 : A.off[l] + B.g.N;
     }
-    A.nsrc = q;
-    k_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
-    FM_LAUNCHED();
-    return FM_OK;
+    return A;
   }
 
   // Choose, per multi-kernel level, the fastest variant of the fused 2-D
@@ -709,8 +695,11 @@ struct Solver {
       k_prepare_mu<DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
       FM_LAUNCHED();
     }
-    const int rc = inject_all(st, false);
-    if (rc) return rc;
+    if (st->nlev > 1) {
+      const InjAll<T> A = injection(st, false);
+      k_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, s>>>(A);
+      FM_LAUNCHED();
+    }
     if constexpr (sizeof(T) == 8) return inverses(st);
     return FM_OK;
   }
@@ -786,8 +775,9 @@ struct Solver {
     return FM_OK;
   }
 
-  // float64 residual of the current iterate, the level-0 set-up of a cycle
-  // and the control-block update (in_body: this follows a cycle).
+  // float64 residual of the current iterate, the set-up of a cycle (level 0,
+  // and the coarser levels' coefficients) and the control-block update
+  // (in_body: this follows a cycle).
   static int enqueue_resid_norm(fm_state* st, int in_body, cudaGraphConditionalHandle hdl, int use_handle) {
     const Geo G = st->lv[0].g;
     const double h = st->lv[0].h;
@@ -798,8 +788,9 @@ struct Solver {
     int rc = launch_resid64(st, F, O, G, h, P, DIM == 3 && in_body);
     if (rc) return rc;
     const double w = (DIM == 3) ? h * h * h : h * h;
-    k_norm_ctl<LY::NU><<<1, TPB, 0, s>>>(st->partials, st->nblk, w, (Ctl*)st->ctl, st->prm.tol,
-                                         st->prm.max_cycles, in_body, hdl, use_handle);
+    const InjAll<T> A = injection(st, true);
+    k_norm_ctl<LY::NU, InjSample, T><<<1 + nblocks(A.off[st->nlev]), TPB, 0, s>>>(
+        st->partials, st->nblk, w, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -1212,11 +1203,9 @@ struct Solver {
   }
 
   static int enqueue_body(fm_state* st, cudaGraphConditionalHandle hdl, int use_handle) {
-    int rc = inject_all(st, true);
-    if (rc) return rc;
     Phys<T> P = make_phys<T>(st);
     int in_r = 0;
-    rc = vcycle(st, 0, P, &in_r);
+    int rc = vcycle(st, 0, P, &in_r);
     if (rc) return rc;
     if (in_r) {  // the float64 update reads the level-0 correction from e
       k_copy_back<T, LY::NU><<<nblocks(st->lv[0].g.N), TPB, 0, st->stream>>>(make_lvl<T>(st, 0));
