@@ -204,11 +204,6 @@ struct InjRows {
   }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_ch_inject_all(const __grid_constant__ InjAll<T> A) {
-  InjRows::point(A, blockIdx.x * blockDim.x + threadIdx.x);
-}
-
 // Fine cell idx: e_F += P(e_C - eh_C): x linear between nodes, y linear
 // between cell centres (3/4 the own coarse cell, 1/4 the next one towards the
 // fine cell), the coarse correction's ghost beyond a wall mirrored (scalars)
@@ -293,9 +288,17 @@ __global__ void __launch_bounds__(TPB) k_ch_prepare(Fields64 F, Geo G, Step64 K,
   prepare_tile<KPFC, true>(F, G, K, P, blockIdx.x, W);
 }
 
-// mu^0 = psi^3/3 + alpha psi + Lap_h kappa^0 + S_mu.
-__global__ void __launch_bounds__(TPB) k_ch_prepare_mu(Fields64 F, Geo G, Step64 K, double alpha, Walls64 W) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+// mu^0 = psi^3/3 + alpha psi + Lap_h kappa^0 + S_mu; the blocks after the last
+// point's: rho^k and omega^k down the levels.
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_ch_prepare_mu(Fields64 F, Geo G, Step64 K, double alpha, Walls64 W,
+                                                       const __grid_constant__ InjAll<T> A) {
+  const int nb = (G.N + TPB - 1) / TPB;
+  if ((int)blockIdx.x >= nb) {
+    InjRows::point(A, (blockIdx.x - nb) * TPB + threadIdx.x);
+    return;
+  }
+  const int idx = blockIdx.x * TPB + threadIdx.x;
   if (idx >= G.N) return;
   const int i = idx % G.nx, j = idx / G.nx;
   const Nb n = ch_neighbours(i, j, G);
@@ -410,13 +413,10 @@ struct ChannelSolver {
     const Fields64 F = make_fields(st);
     k_ch_prepare<<<prep_tiles(G.nx, G.ny), TPB, 0, st->stream>>>(F, G, step64(st), make_phys<double>(st), walls64(st));
     FM_LAUNCHED();
-    k_ch_prepare_mu<<<nblocks(G.N), TPB, 0, st->stream>>>(F, G, step64(st), st->fn.alpha, walls64(st));
+    const InjAll<T> A = injection(st, 0);
+    k_ch_prepare_mu<T><<<nblocks(G.N) + nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(F, G, step64(st), st->fn.alpha,
+                                                                                        walls64(st), A);
     FM_LAUNCHED();
-    if (st->nlev > 1) {
-      const InjAll<T> A = injection(st, 0);
-      k_ch_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(A);
-      FM_LAUNCHED();
-    }
     return FM_OK;
   }
 
@@ -490,7 +490,7 @@ struct ChannelSolver {
     FM_LAUNCHED();
     Vel3W vw{{st->vel[0], st->vel[1], nullptr}};
     Vel3 gv3{{st->g[1], st->g[2], nullptr}};
-    k_commit<2><<<nblocks(G.N), TPB, 0, st->stream>>>(st->rho, vw, st->tmp, gv3, G.N, ctl);
+    k_commit<2><<<nblocks(G.N), TPB, 0, st->stream>>>(st->rho, vw, st->tmp, gv3, G.N, (Ctl*)st->ctl);
     FM_LAUNCHED();
     FM_CUDA(cudaMemcpyAsync(st->hscal + 32, st->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st->stream));
     return FM_OK;

@@ -1,7 +1,7 @@
 // Device code of libfm shared by the single-instance driver (fm_solver.cu)
 // and the batched driver (fm_batch.cu): per-point operations of the FAS
 // cycle on the correction equation, the fused 2-D red-black tile sweep, the
-// single-block small-level V-cycle and the float64 kernels of the finest
+// float32 one-block V-cycle of the small levels and the float64 kernels of the finest
 // level, each as a device function with a thin kernel wrapper.
 #pragma once
 
@@ -2289,9 +2289,14 @@ __device__ __forceinline__ void prepare_mu_point(const Fields64& F, const Geo& G
   F.g[LY::IMU][idx] = psi * psi * psi * (1.0 / 3.0) + P.alpha * psi + lapk + F.S[LY::IMU][idx];
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(TPB) k_prepare_mu(Fields64 F, Geo G, Step64 K, Phys<double> P) {
-  prepare_mu_point<DIM>(F, G, K, P, blockIdx.x * blockDim.x + threadIdx.x);
+// The blocks after the last point's: rho^k and omega^k down the levels (as a
+// launch after this one 3.3 us at 512^2; here 0.2).
+template <int DIM, typename T>
+__global__ void __launch_bounds__(TPB) k_prepare_mu(Fields64 F, Geo G, Step64 K, Phys<double> P,
+                                                    const __grid_constant__ InjAll<T> A) {
+  const int nb = (G.N + TPB - 1) / TPB;
+  if ((int)blockIdx.x >= nb) inject_all_point<T>(A, (blockIdx.x - nb) * TPB + threadIdx.x);
+  else prepare_mu_point<DIM>(F, G, K, P, blockIdx.x * TPB + threadIdx.x);
 }
 
 // Fixed-order block sum of NQ per-thread values into partials[blk][q]: a
@@ -2905,12 +2910,6 @@ __global__ void __launch_bounds__(TPB) k_extrapolate(Ptr6 g, Ptr6 gp, int N, con
   }
 }
 
-// After the step's commit: one more converged iterate kept (at most 2), or
-// none after a failed step (its iterate is not a solution).
-static __global__ void k_hist_advance(Ctl* ctl) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) ctl->hist = ctl->status == FM_OK ? min(ctl->hist + 1, 2) : 0;
-}
-
 // Finishes the residual norm max_q sqrt(w * sum_q), updates the control
 // block (cycles += in_body) and, in graph mode, sets the WHILE condition:
 // continue while the norm is finite, above tol and cycles < max_cycles.
@@ -3056,10 +3055,14 @@ __device__ __forceinline__ void commit_point(double* rho, const Vel3W& vel, cons
   for (int d = 0; d < DIM; ++d) vel.p[d][idx] = v[d];
 }
 
+// hist (the extrapolated start): one more converged iterate kept (at most 2),
+// or none after a failed step (its iterate is not a solution).
 template <int DIM>
 __global__ void __launch_bounds__(TPB) k_commit(double* rho, Vel3W vel, const double* rnew, Vel3 gvel, int N,
-                                                const Ctl* ctl) {
-  if (ctl->status != FM_OK) return;
+                                                Ctl* ctl, bool hist = false) {
+  const bool ok = ctl->status == FM_OK;
+  if (hist && blockIdx.x == 0 && threadIdx.x == 0) ctl->hist = ok ? min(ctl->hist + 1, 2) : 0;
+  if (!ok) return;
   commit_point<DIM>(rho, vel, rnew, gvel, N, blockIdx.x * blockDim.x + threadIdx.x);
 }
 

@@ -18,7 +18,9 @@
 //    whole block (App. G.3); positive projection (Sec. 6) when rho <= 0.
 //  * Transfers: nodal full weighting of r, injection of e and of the
 //    coefficients, bilinear/trilinear prolongation of the coarse correction.
-//  * Coarsest grid: one thread block runs ncoarse red-black iterations.
+//  * Coarsest levels (at most 1,024 points): one launch runs their V-cycle, in
+//    float64 a cluster of blocks, in float32 one block; a larger coarsest level
+//    is smoothed by multi-block sweeps (float64 tiles in the mixed 2-D path).
 #include <cuda.h>
 #include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 #include <cuda_runtime.h>
@@ -691,13 +693,13 @@ struct Solver {
       k_prepare_tile<KIND><<<prep_tiles(G.nx, G.ny), TPB, 0, s>>>(F, G, K, P);
     }
     FM_LAUNCHED();
-    if (KIND == KPFC) {
-      k_prepare_mu<DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
+    const InjAll<T> A = injection(st, false);
+    const int ninj = nblocks(A.off[st->nlev]);
+    if constexpr (KIND == KPFC) {
+      k_prepare_mu<DIM, T><<<nblocks(G.N) + ninj, TPB, 0, s>>>(F, G, K, P, A);
       FM_LAUNCHED();
-    }
-    if (st->nlev > 1) {
-      const InjAll<T> A = injection(st, false);
-      k_inject_all<T><<<nblocks(A.off[st->nlev]), TPB, 0, s>>>(A);
+    } else if (ninj > 0) {
+      k_inject_all<T><<<ninj, TPB, 0, s>>>(A);
       FM_LAUNCHED();
     }
     if constexpr (sizeof(T) == 8) return inverses(st);
@@ -1234,12 +1236,9 @@ struct Solver {
     FM_LAUNCHED();
     Vel3W vw{{st->vel[0], st->vel[1], st->vel[2]}};
     Vel3 gv{{st->g[1], st->g[2], DIM == 3 ? st->g[3] : nullptr}};
-    k_commit<DIM><<<nblocks(G.N), TPB, 0, st->stream>>>(st->rho, vw, st->tmp, gv, G.N, ctl);
+    k_commit<DIM><<<nblocks(G.N), TPB, 0, st->stream>>>(st->rho, vw, st->tmp, gv, G.N, (Ctl*)st->ctl,
+                                                        st->prm.init == FM_INIT_EXTRAPOLATE);
     FM_LAUNCHED();
-    if (st->prm.init == FM_INIT_EXTRAPOLATE) {
-      k_hist_advance<<<1, 32, 0, st->stream>>>((Ctl*)st->ctl);
-      FM_LAUNCHED();
-    }
     FM_CUDA(cudaMemcpyAsync(st->hscal + 32, st->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st->stream));
     return FM_OK;
   }
@@ -1550,7 +1549,7 @@ int fm_create(const fm_grid* grid, const fm_params* prm, const fm_functional* fn
     const char* ef = getenv("FM_FUSED_RB");
     st->fused_rb = !(ef && ef[0] == '0');
   }
-  // A coarsest level that is the only level of the single-block part and
+  // A coarsest level that is the only level of the small part and
   // larger than SMALL_N points is smoothed by multi-block sweeps instead (the
   // fused sweeps in 2-D, a red and a black launch per sweep in 3-D or without
   // fusion); one block would run its points serially.
