@@ -153,6 +153,13 @@ struct HasMcv : std::false_type {};
 template <class A>
 struct HasMcv<A, std::void_t<decltype(std::declval<const A&>().mcv(0))>> : std::true_type {};
 
+// An accessor that also provides qcv(i), qcorr of point i's current correction
+// (the change of |u|^2), kept by the launch that last changed it.
+template <class A, class = void>
+struct HasQcv : std::false_type {};
+template <class A>
+struct HasQcv<A, std::void_t<decltype(std::declval<const A&>().qcv(0))>> : std::true_type {};
+
 // An accessor that also provides iv(i): the inverse determinant of point i's
 // velocity block, formed once a step (it depends on rho^k and omega^k only).
 template <class A, class = void>
@@ -171,7 +178,7 @@ __device__ __forceinline__ T block_det(T Ad, const T* b) {
 // Point-block update of one point, written against an accessor A that
 // provides e(q, i) / set_e(q, i, v), rk(i), cr(i), cv(d, i), f(q, fc) and
 // om(d, fc) (A is a level descriptor in any memory, or a shared-memory tile
-// with compile-time strides), and optionally mcv(i) and iv(i); K holds the level
+// with compile-time strides), and optionally mcv(i), qcv(i) and iv(i); K holds the level
 // constants.  Neighbours are at n.m / n.p; the right-hand side and omega^k
 // are read at index fc.
 template <typename T, int KIND, int DIM, class A>
@@ -208,13 +215,17 @@ __device__ __forceinline__ void smooth_point_a(const A& a, const Phys<T>& P, con
     return s;
   };
   auto qc = [&](int idx) {
-    T q = 0;
+    if constexpr (HasQcv<A>::value) {
+      return a.qcv(idx);
+    } else {
+      T q = 0;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-      const T e = a.e(1 + d, idx);
-      q += e * (T(2) * a.cv(d, idx) + e);
+      for (int d = 0; d < DIM; ++d) {
+        const T e = a.e(1 + d, idx);
+        q += e * (T(2) * a.cv(d, idx) + e);
+      }
+      return q;
     }
-    return q;
   };
   auto mc = [&](int idx) {
     if constexpr (KIND == KPFC) {
@@ -306,17 +317,11 @@ __device__ __forceinline__ void smooth_point(const Lvl<T>& L, const Phys<T>& P, 
   smooth_point_ex<T, KIND, DIM>(L, P, K, n, L.f, L.om, n.c);
 }
 
-// float64 levels of the FP64 path keep iv (L.iv); the float64 copies of the
-// mixed path's coarse levels do not.
 template <int KIND, int DIM>
 __device__ __forceinline__ void smooth_point_iv(const Lvl<double>& L, const Phys<double>& P, const PtK<double>& K,
                                                 const Nb& n) {
-  if (L.iv) {
-    LvlAccIv<double> a{{L, L.f, L.om}};
-    smooth_point_a<double, KIND, DIM>(a, P, K, n, n.c);
-  } else {
-    smooth_point<double, KIND, DIM>(L, P, K, n);
-  }
+  LvlAccIv<double> a{{L, L.f, L.om}};
+  smooth_point_a<double, KIND, DIM>(a, P, K, n, n.c);
 }
 
 // iv of the levels of a hierarchy (FP64 path), one launch a step: a division
@@ -612,45 +617,52 @@ __global__ void __launch_bounds__(TPB) k_smooth(Lvl<T> L, Phys<T> P, PtK<T> K, i
   int i, j, k;
   if (!colour_point(t, color, L.g, i, j, k)) return;
   const Nb n = neighbours(i, j, k, L.g);
-  if constexpr (sizeof(T) == 8) smooth_point_iv<KIND, DIM>(L, P, K, n);
-  else smooth_point<T, KIND, DIM>(L, P, K, n);
+  smooth_point<T, KIND, DIM>(L, P, K, n);
 }
 
-// Level accessor whose neighbours' CDFT chemical-potential parts come from M.
-struct McAcc64 {
-  const Lvl<double>& L;
+// Level accessor whose neighbours' |u|^2 parts come from Q (CDFT: and their
+// chemical-potential parts from M).
+struct KeepAcc : LvlAcc<double> {
+  const double* Q;
   const double* M;
-  __device__ __forceinline__ double e(int q, int i) const { return L.e[q][i]; }
-  __device__ __forceinline__ void set_e(int q, int i, double v) const { L.e[q][i] = v; }
-  __device__ __forceinline__ double rk(int i) const { return L.rk[i]; }
-  __device__ __forceinline__ double cr(int i) const { return L.cr[i]; }
-  __device__ __forceinline__ double cv(int d, int i) const { return L.cv[d][i]; }
-  __device__ __forceinline__ double f(int q, int i) const { return L.f[q][i]; }
-  __device__ __forceinline__ double om(int d, int i) const { return L.om[d][i]; }
+  __device__ __forceinline__ double qcv(int i) const { return Q[i]; }
   __device__ __forceinline__ double mcv(int i) const { return M[i]; }
 };
+struct KeepAccIv : KeepAcc {
+  __device__ __forceinline__ double iv(int i) const { return L.iv[i]; }
+};
 
-// A CDFT colour launch of the float64 coarsest-level sweeps that keeps
-// M[i] = cdft_mc of every point it updates: the next launch (the other
-// colour) reads its neighbours' values from M instead of evaluating the
-// logarithm at each of them (2 DIM evaluations a point on GB300's slow
-// float64 pipe become one).  The first launch of a solve (USE_M false)
-// evaluates its neighbours' values itself, as k_smooth does; M of a colour is
-// read only by the launch after the one that wrote it, so values and order
-// are those of k_smooth.
-template <int DIM, bool USE_M>
-__global__ void __launch_bounds__(TPB) k_smooth_cdft64_mc(Lvl<double> L, Phys<double> P, PtK<double> K, int color, double* M) {
+// A float64 colour launch that keeps, of every point it updates, what the next
+// launch (the other colour) would evaluate at each of its 2 DIM neighbours:
+// Q[i] = qcorr (4 float64 instructions in 2-D, 6 in 3-D) and, CDFT, M[i] =
+// cdft_mc (a logarithm and a division), on the pipe that bounds the launch.
+// The first launch of a run (USE false) evaluates its neighbours' values itself;
+// a colour's values are read only by the launch after the one that wrote them,
+// so values and order are those of k_smooth.  IV: the level keeps iv.  OCC: as
+// k_smooth_occ, but three blocks (80 registers: no spills, and few float64
+// warps fill the pipe).  Per launch of 53,760 points in 3-D: 15.8 us (the first
+// one 19.5), 18.2 without.
+template <int KIND, int DIM, bool USE, bool IV, bool OCC>
+__global__ void __launch_bounds__(TPB, OCC ? 3 : 1) k_smooth_keep(Lvl<double> L, Phys<double> P, PtK<double> K, int color,
+                                                                  double* Q, double* M) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int i, j, k;
   if (!colour_point(t, color, L.g, i, j, k)) return;
   const Nb n = neighbours(i, j, k, L.g);
-  if constexpr (USE_M) {
-    const McAcc64 a{L, M};
-    smooth_point_a<double, KCDFT, DIM>(a, P, K, n, n.c);
+  if constexpr (USE) {
+    using A = std::conditional_t<IV, KeepAccIv, KeepAcc>;
+    A a = [&] {
+      if constexpr (IV) return KeepAccIv{{{L, L.f, L.om}, Q, M}};
+      else return KeepAcc{{L, L.f, L.om}, Q, M};
+    }();
+    smooth_point_a<double, KIND, DIM>(a, P, K, n, n.c);
+  } else if constexpr (IV) {
+    smooth_point_iv<KIND, DIM>(L, P, K, n);
   } else {
-    smooth_point<double, KCDFT, DIM>(L, P, K, n);
+    smooth_point<double, KIND, DIM>(L, P, K, n);
   }
-  M[n.c] = cdft_mc<double>(L.e[0][n.c], L.cr[n.c], P.ce);
+  Q[n.c] = qcorr<double, DIM>(L.e, L.cv, n.c);
+  if constexpr (KIND == KCDFT) M[n.c] = cdft_mc<double>(L.e[0][n.c], L.cr[n.c], P.ce);
 }
 
 // The same colour sweep compiled for six resident blocks per SM (at most 40

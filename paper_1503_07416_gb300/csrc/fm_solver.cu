@@ -555,13 +555,35 @@ struct Solver {
       return Z ? chunked_sweep(st, L, P, Z, st->stream) : FM_EINVAL;  // no chunking at this size
     }
     for (int color = 0; color < 2; ++color) {
-      if (v == 1)
-        k_smooth_occ<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, st->stream>>>(L, P, ptk(L, P), color);
-      else
-        k_smooth<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, st->stream>>>(L, P, ptk(L, P), color);
+      colour_launch(v == 1, true, L, P, color, tpb, st->stream);
       FM_LAUNCHED();
     }
     return FM_OK;
+  }
+
+  // One colour of a sweep on level L, in place.  kept: the launch before was the
+  // other colour's (float64: what its points kept in the level's r, which
+  // in-place sweeps leave free).
+  static void colour_launch(bool occ, bool kept, const Lvl<T>& L, const Phys<T>& P, int color, int tpb, cudaStream_t s) {
+    const int nb = blocks_of(L.g.N / 2, tpb);
+    const PtK<T> K = ptk(L, P);
+    if constexpr (sizeof(T) == 8) {
+      auto go = [&](auto use, auto o) {
+        constexpr bool USE = decltype(use)::value, OCC = decltype(o)::value;
+        if (L.iv) k_smooth_keep<KIND, DIM, USE, true, OCC><<<nb, tpb, 0, s>>>(L, P, K, color, L.r[0], L.r[1]);
+        else k_smooth_keep<KIND, DIM, USE, false, OCC><<<nb, tpb, 0, s>>>(L, P, K, color, L.r[0], L.r[1]);
+      };
+      auto with = [&](auto use) {
+        if (occ) go(use, std::true_type{});
+        else go(use, std::false_type{});
+      };
+      if (kept) with(std::true_type{});
+      else with(std::false_type{});
+    } else if (occ) {
+      k_smooth_occ<T, KIND, DIM><<<nb, tpb, 0, s>>>(L, P, K, color);
+    } else {
+      k_smooth<T, KIND, DIM><<<nb, tpb, 0, s>>>(L, P, K, color);
+    }
   }
 
   // 3-D: time the colour-sweep variants per multi-kernel level (one warm-up
@@ -916,6 +938,7 @@ struct Solver {
       }
       v = 1;  // no chunking at this size
     }
+    bool kept = false;
     for (int it = 0; it < iters;) {
       const bool fused = it < nfused;
       const int nlaunch = fused ? 1 : 2;
@@ -926,10 +949,9 @@ struct Solver {
             const int rc = launch_rb<T, KIND>(st, v, L, P, s, *in_r);
             if (rc) return rc;
           }
-        } else if (DIM == 3 && v == 1) {  // 3-D: v is the colour-sweep variant
-          k_smooth_occ<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, s>>>(*in_r ? swap_er(L) : L, P, ptk(L, P), color);
-        } else {
-          k_smooth<T, KIND, DIM><<<blocks_of(half, tpb), tpb, 0, s>>>(*in_r ? swap_er(L) : L, P, ptk(L, P), color);
+        } else {  // 3-D: v is the colour-sweep variant
+          colour_launch(DIM == 3 && v == 1, kept, *in_r ? swap_er(L) : L, P, color, tpb, s);
+          kept = true;
         }
         FM_LAUNCHED();
         if (prof && st->npev + 2 <= MAXEV) {
@@ -1133,20 +1155,16 @@ struct Solver {
       const Lvl<double> L64 = make_lvl_bufs<double>(st->lv64[l]);
       const int half = L64.g.N / 2;
       const PtK<double> K64 = make_ptk<double, DIM>(P64, L64.h);
-      // CDFT: the chemical-potential part of the points a launch updates is
-      // kept in M (the level's float64 r[0], unused by these sweeps) for the
-      // next launch
-      double* M = static_cast<double*>(st->lv64[l].r[0]);
+      // (r is unused by these sweeps: what a launch's points keep for the next)
+      double *Q = L64.r[0], *M = L64.r[1];
       for (int it = 0; it < st->prm.ncoarse; ++it)
         for (int color = 0; color < 2; ++color) {
-          if constexpr (KIND == KCDFT) {
-            if (it == 0 && color == 0)
-              k_smooth_cdft64_mc<DIM, false><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color, M);
-            else
-              k_smooth_cdft64_mc<DIM, true><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color, M);
-          } else {
-            k_smooth<double, KIND, DIM><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color);
-          }
+          if (it == 0 && color == 0)
+            k_smooth_keep<KIND, DIM, false, false, false><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color,
+                                                                                                     Q, M);
+          else
+            k_smooth_keep<KIND, DIM, true, false, false><<<(half + 31) / 32, 32, 0, st->stream>>>(L64, P64, K64, color,
+                                                                                                    Q, M);
           FM_LAUNCHED();
         }
     }
