@@ -1968,29 +1968,31 @@ struct Fields64 {
 };
 
 // --------------------------------------------------------------------------
-// Exact neighbour sums in fixed point
+// Laplacians in fixed point
 // --------------------------------------------------------------------------
 // A multiprocessor retires one float64 warp instruction in 19 clocks on GB300
-// (measured) and some 40 integer ones in the same time, so the neighbour sums
-// and differences of the residual, half of its float64 instructions, are taken
-// in 64-bit integers: a set of values x (a staged tile of one quantity) whose
-// largest magnitude has the biased exponent emax is held as trunc(x 2^k), k
-// chosen so that the largest value has bit 58 set.  Sums of up to 16 of them
-// are exact, the result is rounded once, and each value carries 6 bits more
-// than the largest float64, so the error is below that of the float64 sum
-// wherever a point's values are within a factor 16 of the set's largest.
-constexpr int FIX_EMIN = 640, FIX_EMAX = 1423;  // clamp below (2^-383: products keep their exponents);
-                                                // above (2^400), or non-finite: plain float64
+// (measured) and some 40 integer ones in the same time, so the five- and
+// seven-point sums of the float64 kernels are taken in 64-bit integers.  The
+// values of one sum, whose largest magnitude has the biased exponent emax, are
+// held as trunc(x 2^k), k chosen so that the largest has bit 58 set: those down to
+// 2^-6 of it exactly, smaller ones to 2^-58 of it.  Up to 16 of them add without
+// an error and the result is rounded once, so a sum is at least as accurate as
+// the float64 one.  The scale is each sum's own: one shared by a tile or a grid
+// saves conversions, but keeps fewer bits than float64 wherever the values are far
+// below the largest of the set (a quiet region beside a fast one, a weak velocity
+// component beside a strong one).
+constexpr int FIX_EMIN = 64;                   // clamp below (2^-959): bits below 2^-1017 are dropped
+constexpr unsigned FIX_TOP = 2031u << 20;      // high words from here (2^1008, or non-finite): plain float64
 
 __device__ __forceinline__ unsigned fix_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-__device__ __forceinline__ int fix_exp(double x) { return (int)(fix_mag(x) >> 20) - 1023; }  // floor(log2 |x|)
+// (a zero or subnormal x is more than 63 bits below emax: its shift clamps to a zero)
 __device__ __forceinline__ long long to_fix(double x, int emax) {
   const unsigned hi = (unsigned)__double2hiint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  unsigned long long m =
+  const unsigned long long m =
       ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x)) << 6;
-  m = e == 0 ? 0ull : m >> min(emax - e, 63);
-  return (int)hi < 0 ? -(long long)m : (long long)m;
+  unsigned long long v;
+  asm("shr.b64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"((unsigned)(emax - (int)((hi >> 20) & 0x7ffu))));
+  return (int)hi < 0 ? -(long long)v : (long long)v;
 }
 __device__ __forceinline__ double from_fix(long long v, int emax) {
   unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
@@ -2002,13 +2004,52 @@ __device__ __forceinline__ double from_fix(long long v, int emax) {
   b = v == 0 ? 0ull : (b | ((unsigned long long)v & 0x8000000000000000ull));
   return __longlong_as_double((long long)b);
 }
+// Sum of v minus M c (M = 2 dim: h^2 Lap) into l; false where a value is beyond
+// fixed point.
+template <int M>
+__device__ __forceinline__ bool fix_lap(const double (&v)[M], double c, double& l) {
+  unsigned mag = fix_mag(c);
+#pragma unroll
+  for (int k = 0; k < M; ++k) mag = max(mag, fix_mag(v[k]));
+  const int e = max((int)(mag >> 20), FIX_EMIN);
+  long long s = -M * to_fix(c, e);
+#pragma unroll
+  for (int k = 0; k < M; ++k) s += to_fix(v[k], e);
+  l = from_fix(s, e);
+  return mag < FIX_TOP;
+}
+// h^2 Lap of a at n.  The float64 form is a call: inlined, the compiler turns the
+// branch into a select and every point pays its instructions.
+template <int DIM>
+static __device__ __noinline__ double lap_call(const double* a, Nb n) {
+  return nbsum<double, DIM>(a, n) - 2.0 * DIM * a[n.c];
+}
+template <int DIM>
+__device__ __forceinline__ double lap64(const double* a, const Nb& n) {
+  double v[2 * DIM], l;
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    v[2 * d] = __ldg(a + n.m[d]);  // (read-only where it is called)
+    v[2 * d + 1] = __ldg(a + n.p[d]);
+  }
+  return fix_lap(v, __ldg(a + n.c), l) ? l : lap_call<DIM>(a, n);
+}
+// The same at cell x of a staged array with rows of SW.
+template <int SW>
+static __device__ __noinline__ double lap_tile_call(const double* x) {
+  return (x[-1] + x[1] + x[-SW] + x[SW]) - 4.0 * x[0];
+}
+template <int SW>
+__device__ __forceinline__ double lap_tile(const double* x) {
+  const double v[4] = {x[-1], x[1], x[-SW], x[SW]};
+  double l;
+  return fix_lap(v, x[0], l) ? l : lap_tile_call<SW>(x);
+}
 
 // omega^k, S and the initial iterate g^0 (kappa^0 = Lap_h rho^k for PFC).
-// FIX: the neighbour sums in fixed point (eu, er: the exponents of the largest
-// velocity and density).
-template <int KIND, int DIM, bool FIX = false>
+template <int KIND, int DIM>
 __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, const Step64& K,
-                                              const Phys<double>& P, int idx, int eu = 0, int er = 0) {
+                                              const Phys<double>& P, int idx) {
   using LY = Layout<KIND, DIM>;
   if (idx >= G.N) return;
   int i, j, k;
@@ -2018,49 +2059,22 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
   const double* u = F.vel[0];
   const double* v = F.vel[1];
   double w[3];
-  // (b_{+i} - b_{-i}) - (a_{+j} - a_{-j})
-  auto rot = [&](const double* b, int i, const double* a, int j) {
-    if constexpr (FIX)
-      return from_fix((to_fix(b[n.p[i]], eu) - to_fix(b[n.m[i]], eu)) - (to_fix(a[n.p[j]], eu) - to_fix(a[n.m[j]], eu)),
-                      eu);
-    else
-      return (b[n.p[i]] - b[n.m[i]]) - (a[n.p[j]] - a[n.m[j]]);
-  };
-  auto lap = [&](const double* a, int e) {  // h^2 Lap
-    if constexpr (FIX) {
-      long long s = 0;
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) s += to_fix(a[n.m[d]], e) + to_fix(a[n.p[d]], e);
-      return from_fix(s - 2 * DIM * to_fix(a[n.c], e), e);
-    } else {
-      return nbsum<double, DIM>(a, n) - 2.0 * DIM * a[n.c];
-    }
-  };
   if constexpr (DIM == 2) {
-    w[0] = K.hih * rot(v, 0, u, 1);
+    w[0] = K.hih * ((v[n.p[0]] - v[n.m[0]]) - (u[n.p[1]] - u[n.m[1]]));
   } else {
     const double* ww = F.vel[2];
-    w[0] = K.hih * rot(ww, 1, v, 2);
-    w[1] = K.hih * rot(u, 2, ww, 0);
-    w[2] = K.hih * rot(v, 0, u, 1);
+    w[0] = K.hih * ((ww[n.p[1]] - ww[n.m[1]]) - (v[n.p[2]] - v[n.m[2]]));
+    w[1] = K.hih * ((u[n.p[2]] - u[n.m[2]]) - (ww[n.p[0]] - ww[n.m[0]]));
+    w[2] = K.hih * ((v[n.p[0]] - v[n.m[0]]) - (u[n.p[1]] - u[n.m[1]]));
   }
   const double rkc = F.rho[n.c];
   if constexpr (KIND == KCDFT) {
     if (F.nonpos && rkc <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
   }
   double div = 0;
-  if constexpr (FIX) {
-    const int e = max(eu + er - 1023 + 1, FIX_EMIN);
-    long long s = 0;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d)
-      s += to_fix(F.rho[n.p[d]] * F.vel[d][n.p[d]], e) - to_fix(F.rho[n.m[d]] * F.vel[d][n.m[d]], e);
-    div = from_fix(s, e);
-  } else {
-#pragma unroll
-    for (int d = 0; d < DIM; ++d)
-      div += F.rho[n.p[d]] * F.vel[d][n.p[d]] - F.rho[n.m[d]] * F.vel[d][n.m[d]];
-  }
+  for (int d = 0; d < DIM; ++d)
+    div += F.rho[n.p[d]] * F.vel[d][n.p[d]] - F.rho[n.m[d]] * F.vel[d][n.m[d]];
   const double c_w = K.c_w, c_v = K.c_v, c_e = K.c_m;
   const double s0 = rkc - K.c_div * div;
   double uc[3], wx[3], sv[3];  // all loads before the first store
@@ -2069,7 +2083,7 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
   cross<double, DIM>(w, uc, wx);
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    double sa = rkc * (uc[a] - c_w * wx[a]) + c_v * lap(F.vel[a], eu);
+    double sa = rkc * (uc[a] - c_w * wx[a]) + c_v * lap64<DIM>(F.vel[a], n);
     if constexpr (KIND == KCDFT) {
       const double Ep = 2.0 * P.ce * F.rho[n.p[a]] + F.conv[n.p[a]];
       const double Em = 2.0 * P.ce * F.rho[n.m[a]] + F.conv[n.m[a]];
@@ -2077,7 +2091,7 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
     }
     sv[a] = sa;
   }
-  const double lapr = (KIND == KPFC) ? lap(F.rho, er) * ih2 : 0.0;
+  const double lapr = (KIND == KPFC) ? lap64<DIM>(F.rho, n) * ih2 : 0.0;
   const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
   F.S[0][idx] = s0;
 #pragma unroll
@@ -2098,22 +2112,6 @@ __device__ __forceinline__ void prepare_point(const Fields64& F, const Geo& G, c
 #pragma unroll
     for (int d = 0; d < LY::NOM; ++d) F.om32[d][idx] = narrow_rn(w[d]);
   }
-}
-
-// The product of two values in fixed point (exponents ea, eb), in fixed point
-// with exponent ea + eb - 1023 + 2.
-__device__ __forceinline__ long long mul_fix(long long a, long long b) { return __mul64hi(a << 4, b); }
-
-// Largest of the block's values m into sm (zero before; a barrier on each side).
-template <int NM>
-__device__ __forceinline__ void block_max(const unsigned (&m)[NM], unsigned* sm) {
-  __syncthreads();
-#pragma unroll
-  for (int a = 0; a < NM; ++a) {
-    const unsigned x = __reduce_max_sync(0xffffffffu, m[a]);
-    if ((threadIdx.x & 31) == 0) atomicMax(&sm[a], x);
-  }
-  __syncthreads();
 }
 
 // Walls at y = 0 and y = ny h moving along x (the channel): in the tile kernels
@@ -2137,11 +2135,9 @@ __device__ __forceinline__ void ghost_velocity(double& u, double& v, int y, int 
 }
 
 // prepare_point on a 32 x 8 tile (tile `tile` of the grid's, one a block): u, v,
-// rho^k u, rho^k v (PFC: rho^k) of the tile and its one-point halo in fixed point
-// in shared memory, scaled by the tile's magnitudes as in the residual's tile.
-// 11 float64 instructions a point (PFC) instead of 37 on the pipe that bounded
-// it: 11.0 us at 512^2, 20.0 point by point.  Beyond FIX_EMAX the same body runs
-// in float64 (as a select in every value it cost a 512^2 film step 0.4%).
+// rho^k u, rho^k v (PFC: rho^k) of the tile and its one-point halo in shared
+// memory, so that the products are formed once a cell, and the Laplacians in
+// fixed point: 13.9 us at 512^2 (float64 sums 20.0, 20.8 point by point).
 constexpr int PT_TX = 32, PT_TY = 8, PT_SW = PT_TX + 2, PT_SN = PT_SW * (PT_TY + 2);
 __host__ __device__ constexpr int prep_tiles(int nx, int ny) {
   return ((nx + PT_TX - 1) / PT_TX) * ((ny + PT_TY - 1) / PT_TY);
@@ -2153,102 +2149,65 @@ __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, co
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
   constexpr int NA = PFC ? 5 : 4;
-  __shared__ long long sX[NA][PT_SN];
-  __shared__ unsigned sMax[2];
+  __shared__ double sX[NA][PT_SN];
   const int nx = G.nx, ny = G.ny;
   const int ntx = (nx + PT_TX - 1) / PT_TX;
   const int x0 = (tile % ntx) * PT_TX, y0 = (tile / ntx) * PT_TY;
-  auto load = [&](int t, double& u, double& v, double& r) {
+  for (int t = threadIdx.x; t < PT_SN; t += TPB) {
     const int ly = t / PT_SW, lx = t - ly * PT_SW, y = y0 + ly - 1;
     const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
-    u = F.vel[0][gi];
-    v = F.vel[1][gi];
-    r = F.rho[gi];
+    double u = F.vel[0][gi], v = F.vel[1][gi];
+    const double r = F.rho[gi];
     ghost_velocity<WALLS>(u, v, y, ny, W);
-  };
-  if (threadIdx.x < 2) sMax[threadIdx.x] = 0u;
-  unsigned mag[2] = {0u, 0u};
-  for (int t = threadIdx.x; t < PT_SN; t += TPB) {
-    double u, v, r;
-    load(t, u, v, r);
-    mag[0] = max(mag[0], max(fix_mag(u), fix_mag(v)));
-    mag[1] = max(mag[1], fix_mag(r));
+    sX[0][t] = u;
+    sX[1][t] = v;
+    sX[2][t] = r * u;
+    sX[3][t] = r * v;
+    if constexpr (PFC) sX[4][t] = r;
   }
-  block_max(mag, sMax);
-  const int eu = max((int)(sMax[0] >> 20), FIX_EMIN), er = max((int)(sMax[1] >> 20), FIX_EMIN);
+  __syncthreads();
   const int i = x0 + (threadIdx.x & 31), j = y0 + (threadIdx.x >> 5);
-  const bool own = i < nx && j < ny;
-  const int idx = own ? j * nx + i : 0;
-  // FIX: the staged values in fixed point; else (non-finite or huge ones) their float64 bits
-  auto finish = [&](auto fixed) {
-    constexpr bool FIX = decltype(fixed)::value;
-    auto fix = [](double x, int e) { return FIX ? to_fix(x, e) : __double_as_longlong(x); };
-    const int e_ru = eu + er - 1023 + 2;
-    for (int t = threadIdx.x; t < PT_SN; t += TPB) {
-      double ud, vd, rd;
-      load(t, ud, vd, rd);
-      const long long u = fix(ud, eu), v = fix(vd, eu), r = fix(rd, er);
-      sX[0][t] = u;
-      sX[1][t] = v;
-      sX[2][t] = FIX ? mul_fix(u, r) : __double_as_longlong(ud * rd);
-      sX[3][t] = FIX ? mul_fix(v, r) : __double_as_longlong(vd * rd);
-      if constexpr (PFC) sX[4][t] = r;
-    }
-    __syncthreads();
-    if (!own) return;
-    const int c = ((threadIdx.x >> 5) + 1) * PT_SW + (threadIdx.x & 31) + 1;
-    const int xm = c - 1, xp = c + 1, ym = c - PT_SW, yp = c + PT_SW;
-    // (a_{xp} - a_{xm}) + sg (b_{yp} - b_{ym}), and h^2 Lap
-    auto dif = [&](int a, int b, int sg, int e) {
-      if (FIX) return from_fix((sX[a][xp] - sX[a][xm]) + sg * (sX[b][yp] - sX[b][ym]), e);
-      auto x = [&](int q, int k) { return __longlong_as_double(sX[q][k]); };
-      return (x(a, xp) - x(a, xm)) + sg * (x(b, yp) - x(b, ym));
-    };
-    auto lap = [&](int a, int e) {
-      if (FIX) return from_fix((sX[a][xm] + sX[a][xp]) + (sX[a][ym] + sX[a][yp]) - (sX[a][c] << 2), e);
-      auto x = [&](int k) { return __longlong_as_double(sX[a][k]); };
-      return (x(xm) + x(xp) + x(ym) + x(yp)) - 4.0 * x(c);
-    };
-    const double w = K.hih * dif(1, 0, -1, eu);
-    const double div = dif(2, 3, 1, e_ru);
-    const double rk = F.rho[idx], uc[2] = {F.vel[0][idx], F.vel[1][idx]};
-    if constexpr (!PFC) {
-      if (F.nonpos && rk <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
-    }
-    const double cw = K.c_w * w;
-    double sv[2] = {fma(K.c_v, lap(0, eu), rk * fma(cw, uc[1], uc[0])),
-                    fma(K.c_v, lap(1, eu), rk * fma(-cw, uc[0], uc[1]))};
-    if constexpr (!PFC) {
-      const Nb n = neighbours(i, j, 0, G);
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const double Ep = 2.0 * P.ce * F.rho[n.p[a]] + F.conv[n.p[a]];
-        const double Em = 2.0 * P.ce * F.rho[n.m[a]] + F.conv[n.m[a]];
-        sv[a] += K.c_m * rk * (Ep - Em);
-      }
-    }
-    const double lapr = PFC ? lap(NA - 1, er) * K.ih2 : 0.0;
-    const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
-    F.S[0][idx] = fma(-K.c_div, div, rk);
+  if (i >= nx || j >= ny) return;
+  const int idx = j * nx + i;
+  const int c = ((threadIdx.x >> 5) + 1) * PT_SW + (threadIdx.x & 31) + 1;
+  const int xm = c - 1, xp = c + 1, ym = c - PT_SW, yp = c + PT_SW;
+  const double w = K.hih * ((sX[1][xp] - sX[1][xm]) - (sX[0][yp] - sX[0][ym]));
+  const double div = (sX[2][xp] - sX[2][xm]) + (sX[3][yp] - sX[3][ym]);
+  const double rk = F.rho[idx], uc[2] = {sX[0][c], sX[1][c]};
+  if constexpr (!PFC) {
+    if (F.nonpos && rk <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
+  }
+  const double cw = K.c_w * w;
+  double sv[2] = {fma(K.c_v, lap_tile<PT_SW>(sX[0] + c), rk * fma(cw, uc[1], uc[0])),
+                  fma(K.c_v, lap_tile<PT_SW>(sX[1] + c), rk * fma(-cw, uc[0], uc[1]))};
+  if constexpr (!PFC) {
+    const Nb n = neighbours(i, j, 0, G);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-      F.S[1 + a][idx] = sv[a];
-      if (!keep) F.g[1 + a][idx] = uc[a];
+      const double Ep = 2.0 * P.ce * F.rho[n.p[a]] + F.conv[n.p[a]];
+      const double Em = 2.0 * P.ce * F.rho[n.m[a]] + F.conv[n.m[a]];
+      sv[a] += K.c_m * rk * (Ep - Em);
     }
-    if (!keep) F.g[0][idx] = rk;
-    if constexpr (PFC) {
-      F.S[LY::IMU][idx] = 2.0 * lapr;
-      F.S[LY::IKA][idx] = 0.0;
-      if (!keep) F.g[LY::IKA][idx] = lapr;
-    }
-    F.om[0][idx] = w;
-    if (F.rk32) {
-      F.rk32[idx] = narrow_rn(rk);
-      F.om32[0][idx] = narrow_rn(w);
-    }
-  };
-  if (max(eu, er) <= FIX_EMAX) finish(std::true_type{});
-  else finish(std::false_type{});
+  }
+  const double lapr = PFC ? lap_tile<PT_SW>(sX[NA - 1] + c) * K.ih2 : 0.0;
+  const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
+  F.S[0][idx] = fma(-K.c_div, div, rk);
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    F.S[1 + a][idx] = sv[a];
+    if (!keep) F.g[1 + a][idx] = uc[a];
+  }
+  if (!keep) F.g[0][idx] = rk;
+  if constexpr (PFC) {
+    F.S[LY::IMU][idx] = 2.0 * lapr;
+    F.S[LY::IKA][idx] = 0.0;
+    if (!keep) F.g[LY::IKA][idx] = lapr;
+  }
+  F.om[0][idx] = w;
+  if (F.rk32) {
+    F.rk32[idx] = narrow_rn(rk);
+    F.om32[0][idx] = narrow_rn(w);
+  }
 }
 
 template <int KIND>
@@ -2256,42 +2215,11 @@ __global__ void __launch_bounds__(TPB) k_prepare_tile(Fields64 F, Geo G, Step64 
   prepare_tile<KIND>(F, G, K, P, blockIdx.x);
 }
 
-// Largest of every thread's values into mag, one atomic a block and value.
-template <int NM>
-__device__ __forceinline__ void grid_max(const unsigned (&m)[NM], unsigned* mag) {
-  __shared__ unsigned sm[NM];
-  if (threadIdx.x < NM) sm[threadIdx.x] = 0u;
-  __syncthreads();
-#pragma unroll
-  for (int a = 0; a < NM; ++a) {
-    const unsigned x = __reduce_max_sync(0xffffffffu, m[a]);
-    if ((threadIdx.x & 31) == 0) atomicMax(&sm[a], x);
-  }
-  __syncthreads();
-  if (threadIdx.x < NM) atomicMax(&mag[threadIdx.x], sm[threadIdx.x]);
-}
-
-// 3-D: the largest magnitudes (high words) of the velocity and the density
-// into mag[0 .. 1] (zero before), and prepare_point with its neighbour sums
-// scaled by them: bound by the float64 pipe, 27 instructions a point, 60 with
-// the sums in float64; the extra pass reads four arrays.
-template <int DIM>
-__global__ void __launch_bounds__(TPB) k_prepare_mag(Fields64 F, int N, unsigned* mag) {
-  unsigned m[2] = {0u, 0u};
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) m[0] = max(m[0], fix_mag(F.vel[d][idx]));
-    m[1] = max(m[1], fix_mag(F.rho[idx]));
-  }
-  grid_max(m, mag);
-}
-
+// 3-D: bound by the float64 pipe, 159 us at 128^3 with the Laplacians in fixed
+// point, 253 us in float64.
 template <int KIND, int DIM>
-__global__ void __launch_bounds__(TPB) k_prepare_fix(Fields64 F, Geo G, Step64 K, Phys<double> P, const unsigned* mag) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int eu = max((int)(mag[0] >> 20), FIX_EMIN), er = max((int)(mag[1] >> 20), FIX_EMIN);
-  if (max(eu, er) <= FIX_EMAX) prepare_point<KIND, DIM, true>(F, G, K, P, idx, eu, er);
-  else prepare_point<KIND, DIM>(F, G, K, P, idx);
+__global__ void __launch_bounds__(TPB, 4) k_prepare(Fields64 F, Geo G, Step64 K, Phys<double> P) {
+  prepare_point<KIND, DIM>(F, G, K, P, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // PFC: mu^0 = psi^3/3 + alpha psi + Lap_h kappa^0 + S_mu (value of the mu row at rho^k).
@@ -2477,25 +2405,23 @@ struct Resid64Out {
 };
 
 // 2-D float64 residual in 32 x 8 tiles: the quantities every point shares
-// with its neighbours -- |u|^2 + 2 mu (mu the implicit chemical potential: the
-// unknown, or ln rho + 2 c_e rho), rho^k u, rho^k v -- are formed once per
+// with its neighbours -- |u|^2, rho^k u, rho^k v and the implicit chemical
+// potential mu (the unknown, or ln rho + 2 c_e rho) -- are formed once per
 // point of the tile and its one-point halo in shared memory, with u, v (PFC:
-// kappa and rho) beside them, all in fixed point; then N is evaluated on the
-// tile.  |u|^2 and 2 mu are one quantity because the coefficient of the
-// chemical potential's gradient, s/(2h), is twice the kinetic one, s/(4h).
-// Block lb of nb walks tiles lb, lb + nb, ...; partial sums of r^2 per block
-// (the same accumulation order on every run).
+// kappa and rho) beside them; then N is evaluated on the tile, its Laplacians in
+// fixed point.  The differences of |u|^2 and 2 mu share a coefficient,
+// because the one of the chemical potential's gradient, s/(2h), is twice the
+// kinetic one, s/(4h).  Block lb of nb walks tiles lb, lb + nb, ...; partial
+// sums of r^2 per block (the same accumulation order on every run).
 //
-// Bound by the float64 pipe: ~18 float64 instructions a point with the
-// neighbour sums and the products they take in fixed point, 51 without.  The scales come from a first
-// pass over the tile's magnitudes (exponents only; its loads find the second
-// pass's in L1, which costs less than holding seven values a point in
-// registers over the barrier: 28.6 us a launch at 512^2 so, 24.9 this way, 23.4
-// with integer products too, 36.8 with float64 sums and products; ensemble of
-// 24 instances, 7.8 M points: 12.1 -> 10.8 ms a step).
-// Against quad precision the rows' errors are at most what they were (rho
-// 3e-17 -> 4e-21, u 4.0e-19 -> 3.1e-19, kappa 2.5e-16 -> 6e-18 at 512^2).  Where a tile holds a value that fixed point
-// does not take (non-finite, beyond 2^400) its sums are float64.
+// Bound by the float64 pipe and the integer one: 32 float64 instructions a point,
+// 51 with the Laplacians and the other sums in float64.  Only the Laplacians are
+// worth fixed point: a difference is one float64 instruction (19 clocks of a
+// multiprocessor), or two conversions and a rounding (~28).  The rows are formed
+// and stored one after the other: all of them at once spilled 44 registers.
+// 25.6 us a launch at 512^2 (float64 Laplacians 34.4; the form before 36.8), 83 us
+// at 1024^2 (122 before).  Bounded to three blocks a multiprocessor; to four
+// 26.3 and 82 us.
 constexpr int R64_TX = 32, R64_TY = 8;
 constexpr int R64_SW = R64_TX + 2, R64_SN = R64_SW * (R64_TY + 2);
 
@@ -2506,12 +2432,9 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
                                                   const Walls64& W = Walls64{}) {
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
-  // staged: |u|^2 + 2 mu, rho^k u, rho^k v, u, v (PFC: kappa, rho)
-  constexpr int NS = PFC ? 7 : 5;
-  // magnitudes: u and v, rho^k; PFC: mu, kappa, rho; CDFT: rho, the smallest rho
-  constexpr int NM = PFC ? 5 : 4;
-  __shared__ long long sX[NS][R64_SN];  // fixed point, or the bits of the float64 value
-  __shared__ unsigned sMax[NM];
+  // staged: u, v (PFC: kappa, rho), whose Laplacians are taken; |u|^2, mu, rho^k u, rho^k v
+  constexpr int NL = PFC ? 4 : 2, NS = NL + 4;
+  __shared__ double sX[NS][R64_SN];
   double acc[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) acc[q] = 0.0;
@@ -2524,202 +2447,101 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
   const int ntx = (nx + R64_TX - 1) / R64_TX;
   const int ntiles = ntx * ((ny + R64_TY - 1) / R64_TY);
   const double* const* g = F.g;
-  if (threadIdx.x < NM) sMax[threadIdx.x] = 0u;
   for (int tile = lb; tile < ntiles; tile += nb) {
     const int x0 = (tile % ntx) * R64_TX, y0 = (tile / ntx) * R64_TY;
-    // grid index of staged cell t and the velocity there (a ghost beyond a wall)
-    auto cell = [&](int t, double& u, double& v) {
+    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
       const int ly = t / R64_SW, lx = t - ly * R64_SW, y = y0 + ly - 1;
       const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
-      u = g[1][gi];
-      v = g[2][gi];
+      double u = g[1][gi], v = g[2][gi], m;
+      const double rk = F.rho[gi], r = g[0][gi];
       ghost_velocity<WALLS>(u, v, y, ny, W);
-      return gi;
-    };
-    unsigned mag[NM];
-#pragma unroll
-    for (int a = 0; a < NM; ++a) mag[a] = 0u;
-    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
-      double u, v;
-      const int gi = cell(t, u, v);
-      mag[0] = max(mag[0], max(fix_mag(u), fix_mag(v)));
-      mag[1] = max(mag[1], fix_mag(F.rho[gi]));
-      if constexpr (PFC) {
-        mag[2] = max(mag[2], fix_mag(g[LY::IMU][gi]));
-        mag[3] = max(mag[3], fix_mag(g[LY::IKA][gi]));
-        mag[4] = max(mag[4], fix_mag(g[0][gi]));
-      } else {
-        const double r = g[0][gi];
-        mag[2] = max(mag[2], fix_mag(r));
-        mag[3] = max(mag[3], r > 0.0 ? 0x7ff00000u - min(fix_mag(r), 0x7ff00000u) : 0x7ff00000u);
-      }
-    }
-    block_max(mag, sMax);  // (sMax is zero; its first barrier: the tile before is finished)
-    int em[NM];
-    bool fix = true;
-#pragma unroll
-    for (int a = 0; a < NM; ++a) {
-      em[a] = max((int)(sMax[a] >> 20), FIX_EMIN);
-      fix = fix && em[a] <= FIX_EMAX;
-    }
-    int e_mu = em[2];
-    if constexpr (!PFC) {
-      // |ln rho + 2 c_e rho|: |ln rho| from the exponents of the smallest and
-      // largest density; a density <= 0 (or subnormal) is left to float64
-      const int lo = 0x7ff - (int)(sMax[3] >> 20) - 1 - 1023, hi = (int)(sMax[2] >> 20) + 1 - 1023;
-      const int lg = max(max(lo < 0 ? -lo : lo, hi < 0 ? -hi : hi), 1);  // |ln rho| < lg
-      fix = (int)(sMax[3] >> 20) < 0x7fe && (int)(sMax[2] >> 20) <= FIX_EMAX && em[0] <= FIX_EMAX &&
-            em[1] <= FIX_EMAX;
-      e_mu = max(em[2] + 2 + fix_exp(P.ce), 1023 + 32 - __clz(lg)) + 1;
-    }
-    // rho^k u and |u|^2 + 2 mu (|u|^2 shifted down to the sum's scale)
-    const int e_ru = em[0] + em[1] - 1023 + 2, e_q = 2 * em[0] - 1023 + 2;
-    const int e_b = max(e_q + 1, e_mu + 1) + 1, sh_q = min(e_b - e_q, 63);
-    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
-      double u, v, m;
-      const int gi = cell(t, u, v);
-      const double rk = F.rho[gi];
       if constexpr (PFC) {
         m = g[LY::IMU][gi];
+        sX[2][t] = g[LY::IKA][gi];
+        sX[3][t] = r;
       } else {
-        const double r = g[0][gi];
         m = log(r) + 2.0 * P.ce * r;
       }
-      if (fix) {
-        const long long uf = to_fix(u, em[0]), vf = to_fix(v, em[0]), rf = to_fix(rk, em[1]);
-        sX[0][t] = ((mul_fix(uf, uf) + mul_fix(vf, vf)) >> sh_q) + 2 * to_fix(m, e_b);
-        sX[1][t] = mul_fix(uf, rf);
-        sX[2][t] = mul_fix(vf, rf);
-        sX[3][t] = uf;
-        sX[4][t] = vf;
-      } else {
-        sX[0][t] = __double_as_longlong(u * u + v * v + 2.0 * m);
-        sX[1][t] = __double_as_longlong(rk * u);
-        sX[2][t] = __double_as_longlong(rk * v);
-        sX[3][t] = __double_as_longlong(u);
-        sX[4][t] = __double_as_longlong(v);
-      }
+      sX[0][t] = u;
+      sX[1][t] = v;
+      sX[NL][t] = u * u + v * v;
+      sX[NL + 1][t] = m;
+      sX[NL + 2][t] = rk * u;
+      sX[NL + 3][t] = rk * v;
+    }
+    __syncthreads();
+    const int ty = threadIdx.x / R64_TX, tx = threadIdx.x - ty * R64_TX;
+    const int i = x0 + tx, j = y0 + ty;
+    if (i < nx && j < ny) {
+      const int idx = j * nx + i;
+      const int c = (ty + 1) * R64_SW + tx + 1;
+      const int xm = c - 1, xp = c + 1, ym = c - R64_SW, yp = c + R64_SW;
+      const double rkc = __ldg(F.rho + idx), w = __ldg(F.om[0] + idx);
+      const double uc = sX[0][c], vc = sX[1][c], g0c = PFC ? sX[NL - 1][c] : g[0][idx];
+      auto S = [&](int q) { return __ldg(F.S[q] + idx); };
+      auto dif = [&](int a, int p, int m) { return sX[a][p] - sX[a][m]; };
+      auto row = [&](int q, double r) {
+        norm_add<T>(O.f0[q], r, acc[q], fa[q], idx);
+        if (O.e0[q]) static_cast<T*>(O.e0[q])[idx] = T(0);
+        if (O.r64[q]) O.r64[q][idx] = r;
+      };
+      const double cw = c_w * w;
+      const double dqx = fma(2.0, dif(NL + 1, xp, xm), dif(NL, xp, xm));
+      const double dqy = fma(2.0, dif(NL + 1, yp, ym), dif(NL, yp, ym));
+      row(0, fma(-c_div, dif(NL + 2, xp, xm) + dif(NL + 3, yp, ym), S(0) - g0c));
+      row(1, fma(c_v, lap_tile<R64_SW>(sX[0] + c), fma(-rkc, fma(c_q, dqx, fma(-cw, vc, uc)), S(1))));
+      row(2, fma(c_v, lap_tile<R64_SW>(sX[1] + c), fma(-rkc, fma(c_q, dqy, fma(cw, uc, vc)), S(2))));
       if constexpr (PFC) {
-        const double ka = g[LY::IKA][gi], r = g[0][gi];
-        sX[NS - 2][t] = fix ? to_fix(ka, em[NM - 2]) : __double_as_longlong(ka);
-        sX[NS - 1][t] = fix ? to_fix(r, em[NM - 1]) : __double_as_longlong(r);
+        const double psi = g0c - 1.5;
+        row(LY::IMU, S(LY::IMU) - fma(-ih2, lap_tile<R64_SW>(sX[2] + c),
+                                      fma(-psi, fma(psi * psi, third, P.alpha), sX[NL + 1][c])));
+        row(LY::IKA, fma(ih2, lap_tile<R64_SW>(sX[3] + c), -sX[2][c]));  // S_kappa = 0
+      }
+      if (O.cr32) {
+        O.cr32[idx] = narrow_rn(g0c);
+        O.cv32[0][idx] = narrow_rn(uc);
+        O.cv32[1][idx] = narrow_rn(vc);
       }
     }
     __syncthreads();
-    if (threadIdx.x < NM) sMax[threadIdx.x] = 0u;
-    for (int t = threadIdx.x; t < R64_TX * R64_TY; t += TPB) {
-      const int ty = t / R64_TX, tx = t - ty * R64_TX;
-      const int i = x0 + tx, j = y0 + ty;
-      if (i < nx && j < ny) {
-        const int idx = j * nx + i;
-        const int c = (ty + 1) * R64_SW + tx + 1;
-        const int xm = c - 1, xp = c + 1, ym = c - R64_SW, yp = c + R64_SW;
-        double S[LY::NU];
-#pragma unroll
-        for (int q = 0; q < (PFC ? LY::IKA : LY::NU); ++q) S[q] = F.S[q][idx];
-        const double rkc = F.rho[idx], uc = g[1][idx], vc = g[2][idx], g0c = g[0][idx];
-        const double w = F.om[0][idx];
-        // 2h div(rho^k u), differences of |u|^2 + 2 mu, h^2 Lap of u, v (kappa, rho)
-        double dv, dq[2], lap[NS - 3];
-        if (fix) {
-          dv = from_fix((sX[1][xp] - sX[1][xm]) + (sX[2][yp] - sX[2][ym]), e_ru);
-          dq[0] = from_fix(sX[0][xp] - sX[0][xm], e_b);
-          dq[1] = from_fix(sX[0][yp] - sX[0][ym], e_b);
-#pragma unroll
-          for (int a = 3; a < NS; ++a)
-            lap[a - 3] = from_fix((sX[a][xm] + sX[a][xp]) + (sX[a][ym] + sX[a][yp]) - (sX[a][c] << 2),
-                                  em[a < 5 ? 0 : a - 2]);
-        } else {
-          auto x = [&](int a, int k) { return __longlong_as_double(sX[a][k]); };
-          dv = (x(1, xp) - x(1, xm)) + (x(2, yp) - x(2, ym));
-          dq[0] = x(0, xp) - x(0, xm);
-          dq[1] = x(0, yp) - x(0, ym);
-#pragma unroll
-          for (int a = 3; a < NS; ++a) lap[a - 3] = (x(a, xm) + x(a, xp) + x(a, ym) + x(a, yp)) - 4.0 * x(a, c);
-        }
-        double rv[LY::NU];
-        const double cw = c_w * w;
-        rv[0] = fma(-c_div, dv, S[0] - g0c);
-        rv[1] = fma(c_v, lap[0], fma(-rkc, fma(c_q, dq[0], fma(-cw, vc, uc)), S[1]));
-        rv[2] = fma(c_v, lap[1], fma(-rkc, fma(c_q, dq[1], fma(cw, uc, vc)), S[2]));
-        if constexpr (PFC) {
-          const double psi = g0c - 1.5;
-          rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap[2], fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][idx]));
-          rv[LY::IKA] = fma(ih2, lap[3], -g[LY::IKA][idx]);  // S_kappa = 0
-        }
-#pragma unroll
-        for (int q = 0; q < LY::NU; ++q) {
-          const double r = rv[q];
-          norm_add<T>(O.f0[q], r, acc[q], fa[q], idx);
-          if (O.e0[q]) static_cast<T*>(O.e0[q])[idx] = T(0);
-          if (O.r64[q]) O.r64[q][idx] = r;
-        }
-        if (O.cr32) {
-          O.cr32[idx] = narrow_rn(g0c);
-          O.cv32[0][idx] = narrow_rn(uc);
-          O.cv32[1][idx] = narrow_rn(vc);
-        }
-      }
-    }
   }
-  __syncthreads();
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, lb);
 }
 
 template <int KIND, typename T>
-__global__ void __launch_bounds__(TPB, 4) k_resid64_tile(Fields64 F, Resid64Out O, Geo G, Step64 K,
+__global__ void __launch_bounds__(TPB, 3) k_resid64_tile(Fields64 F, Resid64Out O, Geo G, Step64 K,
                                                       Phys<double> P, double* partials) {
   resid64_tile_body<KIND, T>(F, O, G, K, P, partials, blockIdx.x, gridDim.x);
 }
 
 // Per-point quantities every point shares with its neighbours in the
 // float64 residual (used in 3-D): X[0] = |u|^2, X[1 + d] = rho^k u_d, and for
-// CDFT X[4] = ln rho + 2 c_e rho.  mag: the largest magnitudes (high words) of
-// the whole grid's u, rho^k, mu (PFC: the unknown; CDFT: X[4]) and, PFC, kappa
-// and rho, which scale the residual's fixed-point sums; zero before the pass.
+// CDFT X[4] = ln rho + 2 c_e rho.
 struct Shared64 {
   double* x[5];
-  unsigned* mag;
 };
-constexpr int X64_NM = 5;
 
-// The shared quantities of one point with iterate gv, and its magnitudes.
+// The shared quantities of one point with iterate gv.
 template <int KIND, int DIM>
-__device__ __forceinline__ void shared64_point(const Shared64& X, const double* gv, double rk, double ce, int idx,
-                                               unsigned (&m)[X64_NM]) {
-  using LY = Layout<KIND, DIM>;
+__device__ __forceinline__ void shared64_point(const Shared64& X, const double* gv, double rk, double ce, int idx) {
   double q = 0;
 #pragma unroll
   for (int d = 0; d < DIM; ++d) {
     q += gv[1 + d] * gv[1 + d];
     X.x[1 + d][idx] = rk * gv[1 + d];
-    m[0] = max(m[0], fix_mag(gv[1 + d]));
   }
   X.x[0][idx] = q;
-  m[1] = fix_mag(rk);
-  if constexpr (KIND == KPFC) {
-    m[2] = fix_mag(gv[LY::IMU]);
-    m[3] = fix_mag(gv[LY::IKA]);
-    m[4] = fix_mag(gv[0]);
-  } else {
-    const double mu = log(gv[0]) + 2.0 * ce * gv[0];
-    X.x[4][idx] = mu;
-    m[2] = fix_mag(mu);
-  }
+  if constexpr (KIND == KCDFT) X.x[4][idx] = log(gv[0]) + 2.0 * ce * gv[0];
 }
 
 template <int KIND, int DIM>
 __global__ void __launch_bounds__(TPB) k_shared64(Fields64 F, Shared64 X, int N, double ce) {
-  using LY = Layout<KIND, DIM>;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned m[X64_NM] = {0u, 0u, 0u, 0u, 0u};
-  if (idx < N) {
-    double gv[LY::NU];
+  if (idx >= N) return;
+  double gv[1 + DIM];
 #pragma unroll
-    for (int q = 0; q < LY::NU; ++q) gv[q] = F.g[q][idx];
-    shared64_point<KIND, DIM>(X, gv, F.rho[idx], ce, idx, m);
-  }
-  grid_max(m, X.mag);
+  for (int q = 0; q < 1 + DIM; ++q) gv[q] = F.g[q][idx];
+  shared64_point<KIND, DIM>(X, gv, F.rho[idx], ce, idx);
 }
 
 // After a cycle (3-D): the float64 update g += e of update64_point (with its
@@ -2731,34 +2553,31 @@ __global__ void __launch_bounds__(TPB) k_update_shared64(Fields64 F, Resid64Out 
                                                          double delta) {
   using LY = Layout<KIND, DIM>;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned m[X64_NM] = {0u, 0u, 0u, 0u, 0u};
-  if (idx < N) {
-    double gv[LY::NU];
-    T ev[LY::NU];  // all loads before the first store
+  if (idx >= N) return;
+  double gv[LY::NU];
+  T ev[LY::NU];  // all loads before the first store
 #pragma unroll
-    for (int q = 0; q < LY::NU; ++q) {
-      gv[q] = F.g[q][idx];
-      ev[q] = static_cast<const T*>(O.e0[q])[idx];
-    }
-    const double rk = F.rho[idx];
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) gv[q] += from_t<T>(ev[q]);
-    gv[0] = (delta > 0.0) ? proj_rho(gv[0], delta) : fabs(gv[0]);
-    if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) F.g[q][idx] = gv[q];
-    shared64_point<KIND, DIM>(X, gv, rk, ce, idx, m);
+  for (int q = 0; q < LY::NU; ++q) {
+    gv[q] = F.g[q][idx];
+    ev[q] = static_cast<const T*>(O.e0[q])[idx];
   }
-  grid_max(m, X.mag);
+  const double rk = F.rho[idx];
+#pragma unroll
+  for (int q = 0; q < LY::NU; ++q) gv[q] += from_t<T>(ev[q]);
+  gv[0] = (delta > 0.0) ? proj_rho(gv[0], delta) : fabs(gv[0]);
+  if (F.nonpos && gv[0] <= 0.0) atomicOr(F.nonpos, 1);  // CDFT, delta = 0: ln 0 next
+#pragma unroll
+  for (int q = 0; q < LY::NU; ++q) F.g[q][idx] = gv[q];
+  shared64_point<KIND, DIM>(X, gv, rk, ce, idx);
 }
 
-// Float64 residual reading the shared quantities of k_shared64.  Bound by the
-// float64 pipe: ~28 instructions a point in 3-D with the neighbour sums in
-// fixed point (scaled by the grid's magnitudes), 81 without.
-template <int KIND, int DIM, typename T, bool FIX>
-__device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64& X, const Resid64Out& O, const Geo& G,
-                                               const Step64& K, const Phys<double>& P, double* partials,
-                                               const int (&em)[X64_NM]) {
+// Float64 residual reading the shared quantities of k_shared64, its Laplacians in
+// fixed point: 45 float64 instructions a point in 3-D, 81 with them in float64.
+// The rows are formed and stored one after the other (all at once they spill 120
+// registers): 200 us at 128^3, 335 with float64 sums.
+template <int KIND, int DIM, typename T>
+__global__ void __launch_bounds__(TPB, 4) k_resid64_x(Fields64 F, Shared64 X, Resid64Out O, Geo G, Step64 K,
+                                                   Phys<double> P, double* partials) {
   using LY = Layout<KIND, DIM>;
   constexpr bool PFC = KIND == KPFC;
   double acc[LY::NU];
@@ -2767,77 +2586,47 @@ __device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64
   float fa[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) fa[q] = 0.0f;
-  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_v = K.c_v;
+  const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_m = K.c_m, c_v = K.c_v;
   const double third = 1.0 / 3.0;
   const double* const* g = F.g;
   const double* M = PFC ? g[LY::IMU] : X.x[4];
-  const int e_b = max(2 * em[0] - 1023 + 3, em[2] + 1) + 1;  // |u|^2 + 2 mu
-  const int e_ru = max(em[0] + em[1] - 1023 + 1, FIX_EMIN);  // rho^k u
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < G.N; idx += gridDim.x * blockDim.x) {
     int i, j, k;
     coords(idx, G, i, j, k);
     const Nb n = neighbours(i, j, k, G);
-    auto lap = [&](const double* a, double c, int e) {  // h^2 Lap
-      if constexpr (FIX) {
-        long long s = 0;
+    const double rkc = __ldg(F.rho + idx), g0c = g[0][idx];
+    double uc[3], w[3];
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) s += to_fix(a[n.m[d]], e) + to_fix(a[n.p[d]], e);
-        return from_fix(s - 2 * DIM * to_fix(c, e), e);
-      } else {
-        return nbsum<double, DIM>(a, n) - 2.0 * DIM * c;
-      }
-    };
-    double dv, dq[DIM];  // 2h div(rho^k u), differences of |u|^2 + 2 mu
-    if constexpr (FIX) {
-      long long s = 0;
+    for (int d = 0; d < DIM; ++d) uc[d] = g[1 + d][idx];
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        s += to_fix(X.x[1 + d][n.p[d]], e_ru) - to_fix(X.x[1 + d][n.m[d]], e_ru);
-        dq[d] = from_fix((to_fix(X.x[0][n.p[d]], e_b) - to_fix(X.x[0][n.m[d]], e_b)) +
-                             2 * (to_fix(M[n.p[d]], e_b) - to_fix(M[n.m[d]], e_b)),
-                         e_b);
-      }
-      dv = from_fix(s, e_ru);
-    } else {
-      dv = 0;
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        dv += X.x[1 + d][n.p[d]] - X.x[1 + d][n.m[d]];
-        dq[d] = (X.x[0][n.p[d]] - X.x[0][n.m[d]]) + 2.0 * (M[n.p[d]] - M[n.m[d]]);
-      }
-    }
-    const double rkc = F.rho[n.c], g0c = g[0][n.c];
-    double uc[3], w[3], S[LY::NU], rv[LY::NU];  // all loads before the first store
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) uc[d] = g[1 + d][n.c];
-#pragma unroll
-    for (int d = 0; d < LY::NOM; ++d) w[d] = c_w * F.om[d][n.c];
-#pragma unroll
-    for (int q = 0; q < (PFC ? LY::IKA : LY::NU); ++q) S[q] = F.S[q][idx];
-    rv[0] = fma(-c_div, dv, S[0] - g0c);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      // u + c_w (omega x u) + c_q d(|u|^2 + 2 mu)
-      double br;
-      if constexpr (DIM == 2)
-        br = a == 0 ? fma(-w[0], uc[1], uc[0]) : fma(w[0], uc[0], uc[1]);
-      else
-        br = fma(w[(a + 1) % 3], uc[(a + 2) % 3], fma(-w[(a + 2) % 3], uc[(a + 1) % 3], uc[a]));
-      br = fma(c_q, dq[a], br);
-      rv[1 + a] = fma(c_v, lap(g[1 + a], uc[a], em[0]), fma(-rkc, br, S[1 + a]));
-    }
-    if constexpr (PFC) {
-      const double psi = g0c - 1.5, kc = g[LY::IKA][n.c];
-      rv[LY::IMU] = S[LY::IMU] - fma(-ih2, lap(g[LY::IKA], kc, em[3]),
-                                     fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][n.c]));
-      rv[LY::IKA] = fma(ih2, lap(g[0], g0c, em[4]), -kc);  // S_kappa = 0
-    }
-#pragma unroll
-    for (int q = 0; q < LY::NU; ++q) {
-      const double r = rv[q];
+    for (int d = 0; d < LY::NOM; ++d) w[d] = c_w * __ldg(F.om[d] + idx);
+    auto S = [&](int q) { return __ldg(F.S[q] + idx); };
+    auto dif = [&](const double* a, int d) { return __ldg(a + n.p[d]) - __ldg(a + n.m[d]); };
+    auto row = [&](int q, double r) {
       norm_add<T>(O.f0[q], r, acc[q], fa[q], idx);
       if (O.e0[q]) static_cast<T*>(O.e0[q])[idx] = T(0);
       if (O.r64[q]) O.r64[q][idx] = r;
+    };
+    double dv = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) dv += dif(X.x[1 + d], d);
+    row(0, fma(-c_div, dv, S(0) - g0c));
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      // S - rho^k u - rho^k (c_w (omega x u) + c_q d|u|^2 + c_m d mu) + c_v h^2 Lap u,
+      // u last: the sum in the brackets is not rounded at its size
+      double br = fma(c_m, dif(M, a), c_q * dif(X.x[0], a));
+      if constexpr (DIM == 2)
+        br = a == 0 ? fma(-w[0], uc[1], br) : fma(w[0], uc[0], br);
+      else
+        br = fma(w[(a + 1) % 3], uc[(a + 2) % 3], fma(-w[(a + 2) % 3], uc[(a + 1) % 3], br));
+      row(1 + a, fma(c_v, lap64<DIM>(g[1 + a], n), fma(-rkc, br, fma(-rkc, uc[a], S(1 + a)))));
+    }
+    if constexpr (PFC) {
+      const double psi = g0c - 1.5;
+      row(LY::IMU, S(LY::IMU) - fma(-ih2, lap64<DIM>(g[LY::IKA], n),
+                                    fma(-psi, fma(psi * psi, third, P.alpha), g[LY::IMU][idx])));
+      row(LY::IKA, fma(ih2, lap64<DIM>(g[0], n), -g[LY::IKA][idx]));  // S_kappa = 0
     }
     if (O.cr32) {
       O.cr32[idx] = narrow_rn(g0c);
@@ -2846,20 +2635,6 @@ __device__ __forceinline__ void resid64_x_body(const Fields64& F, const Shared64
     }
   }
   norm_partials<T, LY::NU>(O.f0[0], acc, fa, partials, blockIdx.x);
-}
-
-template <int KIND, int DIM, typename T>
-__global__ void __launch_bounds__(TPB, 4) k_resid64_x(Fields64 F, Shared64 X, Resid64Out O, Geo G, Step64 K,
-                                                   Phys<double> P, double* partials) {
-  int em[X64_NM];
-  bool fix = true;
-#pragma unroll
-  for (int a = 0; a < X64_NM; ++a) {
-    em[a] = max((int)(X.mag[a] >> 20), FIX_EMIN);
-    fix = fix && em[a] <= FIX_EMAX;
-  }
-  if (fix) resid64_x_body<KIND, DIM, T, true>(F, X, O, G, K, P, partials, em);
-  else resid64_x_body<KIND, DIM, T, false>(F, X, O, G, K, P, partials, em);
 }
 
 // g += e (float64), then the projection of Sec. 6 on rho.

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(TPB) k_gf_resid64(GF64 F, Resid64Out O, Geo G,
     acc[q] = 0.0;
     fa[q] = 0.0f;
   }
-  const double c = 2.0 * DIM * ih2;
+  const double c = 2.0 * DIM * ih2, sih2 = s * ih2, third = 1.0 / 3.0;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < G.N; idx += gridDim.x * blockDim.x) {
     int i, j, k;
     coords(idx, G, i, j, k);
@@ -310,14 +310,10 @@ __global__ void __launch_bounds__(TPB) k_gf_resid64(GF64 F, Resid64Out O, Geo G,
     double r[NU];
     const double g0 = F.g[0][idx];
     if constexpr (KIND == KPFC) {
-      const double g1 = F.g[1][idx], g2 = F.g[2][idx];
       const double psi = g0 - 1.5;
-      const double N0 = g0 + s * c * g1 - s * ih2 * nbsum<double, DIM>(F.g[1], n);
-      const double N1 = g1 - psi * (psi * psi * (1.0 / 3.0) + alpha) + c * g2 - ih2 * nbsum<double, DIM>(F.g[2], n);
-      const double N2 = g2 + c * g0 - ih2 * nbsum<double, DIM>(F.g[0], n);
-      r[0] = F.S[0][idx] - N0;
-      r[1] = F.S[1][idx] - N1;
-      r[2] = F.S[2][idx] - N2;
+      r[0] = F.S[0][idx] - fma(-sih2, lap64<DIM>(F.g[1], n), g0);
+      r[1] = F.S[1][idx] - fma(-ih2, lap64<DIM>(F.g[2], n), fma(-psi, fma(psi * psi, third, alpha), F.g[1][idx]));
+      r[2] = fma(ih2, lap64<DIM>(F.g[0], n), -F.g[2][idx]);  // S_kappa = 0
     } else {
       const double N0 = g0 + s * c * F.m[idx] - s * ih2 * nbsum<double, DIM>(F.m, n);
       r[0] = F.S[0][idx] - N0;
@@ -331,95 +327,6 @@ __global__ void __launch_bounds__(TPB) k_gf_resid64(GF64 F, Resid64Out O, Geo G,
     if (O.cr32) O.cr32[idx] = narrow_rn(g0);
   }
   norm_partials<T, NU>(O.f0[0], acc, fa, partials, blockIdx.x);
-}
-
-// The PFC residual in 2-D on 32 x 8 tiles with the neighbour sums in fixed
-// point (see resid64_tile_body): 15 float64 instructions a point instead of 24
-// on the pipe that bounds it, 17.4 -> 12.5 us a launch at 512^2.
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_gf_resid64_tile(GF64 F, Resid64Out O, Geo G, double ih2, double s, double alpha,
-                                                         double* partials) {
-  __shared__ long long sX[3][R64_SN];
-  __shared__ unsigned sMax[3];
-  double acc[3] = {0.0, 0.0, 0.0};
-  float fa[3] = {0.0f, 0.0f, 0.0f};
-  const int nx = G.nx, ny = G.ny;
-  const int ntx = (nx + R64_TX - 1) / R64_TX;
-  const int ntiles = ntx * ((ny + R64_TY - 1) / R64_TY);
-  const double third = 1.0 / 3.0, sih2 = s * ih2;
-  if (threadIdx.x < 3) sMax[threadIdx.x] = 0u;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int x0 = (tile % ntx) * R64_TX, y0 = (tile / ntx) * R64_TY;
-    auto cell = [&](int t) {
-      const int ly = t / R64_SW, lx = t - ly * R64_SW;
-      return wrapi(y0 + ly - 1, ny) * nx + wrapi(x0 + lx - 1, nx);
-    };
-    constexpr int PER = (R64_SN + TPB - 1) / TPB;
-    double X[PER][3];
-    unsigned mag[3] = {0u, 0u, 0u};
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int t = threadIdx.x + k * TPB;
-      if (t < R64_SN) {
-        const int gi = cell(t);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          X[k][q] = F.g[q][gi];
-          mag[q] = max(mag[q], fix_mag(X[k][q]));
-        }
-      }
-    }
-    block_max(mag, sMax);  // (sMax is zero; its first barrier: the tile before is finished)
-    int em[3];
-    bool fix = true;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      em[q] = max((int)(sMax[q] >> 20), FIX_EMIN);
-      fix = fix && em[q] <= FIX_EMAX;
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int t = threadIdx.x + k * TPB;
-      if (t < R64_SN)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) sX[q][t] = fix ? to_fix(X[k][q], em[q]) : __double_as_longlong(X[k][q]);
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) sMax[threadIdx.x] = 0u;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i = x0 + tx, j = y0 + ty;
-    if (i < nx && j < ny) {
-      const int idx = j * nx + i;
-      const int c = (ty + 1) * R64_SW + tx + 1;
-      double g[3], lap[3], S[2];  // h^2 Lap
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        g[q] = F.g[q][idx];
-        if (fix) {
-          lap[q] = from_fix((sX[q][c - 1] + sX[q][c + 1]) + (sX[q][c - R64_SW] + sX[q][c + R64_SW]) - (sX[q][c] << 2),
-                            em[q]);
-        } else {
-          auto x = [&](int k) { return __longlong_as_double(sX[q][k]); };
-          lap[q] = (x(c - 1) + x(c + 1) + x(c - R64_SW) + x(c + R64_SW)) - 4.0 * x(c);
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) S[q] = F.S[q][idx];
-      const double psi = g[0] - 1.5;
-      const double r[3] = {S[0] - fma(-sih2, lap[1], g[0]),
-                           S[1] - fma(-ih2, lap[2], fma(-psi, fma(psi * psi, third, alpha), g[1])),
-                           fma(ih2, lap[0], -g[2])};  // S_kappa = 0
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        norm_add<T>(O.f0[q], r[q], acc[q], fa[q], idx);
-        if (O.e0[q]) static_cast<T*>(O.e0[q])[idx] = T(0);
-        if (O.r64[q]) O.r64[q][idx] = r[q];
-      }
-      if (O.cr32) O.cr32[idx] = narrow_rn(g[0]);
-    }
-  }
-  __syncthreads();
-  norm_partials<T, 3>(O.f0[0], acc, fa, partials, blockIdx.x);
 }
 
 // rho^{k+1} = rho^k + s Lap_h mu with mu = g1 (PFC) or m + E (CDFT), projected;
@@ -513,10 +420,7 @@ struct GFSolver {
       k_gf_m64<<<nblocks(G.N), TPB, 0, s>>>(F, G.N, st->ce);
       FM_LAUNCHED();
     }
-    if constexpr (KIND == KPFC && DIM == 2)
-      k_gf_resid64_tile<T><<<st->nblk, TPB, 0, s>>>(F, O, G, ih2(st), st->dt, st->fn.alpha, st->partials);
-    else
-      k_gf_resid64<KIND, DIM, T><<<st->nblk, TPB, 0, s>>>(F, O, G, ih2(st), st->dt, st->fn.alpha, st->partials);
+    k_gf_resid64<KIND, DIM, T><<<st->nblk, TPB, 0, s>>>(F, O, G, ih2(st), st->dt, st->fn.alpha, st->partials);
     FM_LAUNCHED();
     return FM_OK;
   }

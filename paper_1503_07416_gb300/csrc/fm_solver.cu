@@ -707,10 +707,7 @@ struct Solver {
     Fields64 F = make_fields(st);
     const Step64 K = make_step64(P, 1.0 / h);
     if constexpr (DIM == 3) {
-      FM_CUDA(cudaMemsetAsync(st->mag, 0, 2 * sizeof(unsigned), s));
-      k_prepare_mag<DIM><<<st->nblk, TPB, 0, s>>>(F, G.N, st->mag);
-      FM_LAUNCHED();
-      k_prepare_fix<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P, st->mag);
+      k_prepare<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, G, K, P);
     } else {
       k_prepare_tile<KIND><<<prep_tiles(G.nx, G.ny), TPB, 0, s>>>(F, G, K, P);
     }
@@ -771,7 +768,6 @@ struct Solver {
   static Shared64 shared64(fm_state* st) {
     Shared64 X;
     for (int q = 0; q < 5; ++q) X.x[q] = st->x64[q];
-    X.mag = st->mag;
     return X;
   }
 
@@ -786,7 +782,6 @@ struct Solver {
       FM_LAUNCHED();
     } else {
       const Shared64 X = shared64(st);
-      FM_CUDA(cudaMemsetAsync(st->mag, 0, X64_NM * sizeof(unsigned), s));
       if (update)
         k_update_shared64<KIND, DIM, T><<<nblocks(G.N), TPB, 0, s>>>(F, O, X, G.N, P.ce, st->prm.delta);
       else
@@ -1358,7 +1353,6 @@ static size_t carve(fm_state* st, char* base) {
   st->partials = (double*)C.take((size_t)st->nblk * 8 * d8);
   st->dscal = (double*)C.take(64 * d8);
   st->ctl = C.take(64);
-  st->mag = (unsigned*)C.take(8 * sizeof(unsigned));
   for (int l = 0; l < st->nlev; ++l) {
     LevelBufs& B = st->lv[l];
     const size_t N = B.g.N;

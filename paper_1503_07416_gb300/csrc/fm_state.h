@@ -56,7 +56,6 @@ struct fm_state {
   double* tmp;                    // float64 scratch of N values
   double* r64[fm::MAXU];          // float64 residual scratch (row-level entry points)
   double* x64[5];                 // 3-D: per-point quantities shared by the residual
-  unsigned* mag;                  // 3-D: the largest magnitudes that scale the fixed-point sums
   double* partials;               // per-block partial sums (deterministic reductions)
   int nblk;                       // blocks of the reduction kernels
   int sms;                        // multiprocessors of the device
