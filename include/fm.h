@@ -372,6 +372,13 @@ int fm_batch_time_sweep_variant(fm_batch* b, int variant, int iters, double* ms_
  * repeats; batches take the first). */
 int fm_tuning(const fm_state* st, int level, int* variant, float* ms_per_variant);
 
+/* Blocks of the thread-block cluster that runs the float64 V-cycle of the
+ * state's coarsest levels (at most 1,024 points each): 16, or 8 (the portable
+ * size) where the device cannot schedule 16 or the environment variable
+ * FM_CLUSTER=8 is set at fm_create; 0 if the state has no such levels (or solves
+ * them in float32).  The result does not depend on it.  FM_EINVAL for null. */
+int fm_cluster_blocks(const fm_state* st);
+
 /* Enable (1) or disable (0) CUDA-event timing of every finest-level smoother
  * launch issued by fm_step, and reset the accumulated totals. */
 int fm_profile(fm_state* st, int enable);

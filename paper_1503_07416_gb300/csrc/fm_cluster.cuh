@@ -37,7 +37,7 @@ namespace fm {
 
 constexpr int CL_TPB = 384;  // twelve warps: two to four sets of the 3 to 5 roles of warps
 constexpr int CL_MAX = 16;   // blocks of a cluster
-constexpr size_t CL_SMEM_MAX = 128 * 1024;  // 3-D, 8 blocks: 8 coefficients x ~1,200 points + the slabs, under 110 KB
+constexpr size_t CL_SMEM_MAX = 128 * 1024;  // the largest plan: PFC 16 x 16 x 4 on 8 blocks, 115,456 bytes
 
 template <int KIND, int DIM>
 struct ClDim {

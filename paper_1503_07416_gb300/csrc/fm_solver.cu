@@ -27,7 +27,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <atomic>
 #include <cmath>
 #include <new>
 
@@ -995,44 +994,68 @@ struct Solver {
     return FM_OK;
   }
 
-  // The float64 V-cycle of the small levels from l down by one cluster
-  // (fm_cluster.cuh), on the levels of the state in their own precision T.
-  static int cluster_cycle(fm_state* st, int l) {
-    SmallLv<T> S;
+  // The small levels from l down in the state's own precision T, their spacings
+  // and the plan of a cluster of nb blocks; returns its shared memory.
+  static size_t cluster_plan(const fm_state* st, int l, int nb, const Phys<double>& P, SmallLv<T>& S, ClPlan& M) {
     double h[MAXSMALL];
     S.count = st->nlev - l;
     for (int q = 0; q < S.count; ++q) {
       S.lv[q] = make_lvl<T>(st, l + q);
       h[q] = st->lv[l + q].h;
     }
-    const Phys<double> P = make_phys<double>(st);
-    const auto kernel = k_vcycle_cluster<T, KIND, DIM>;
+    return cl_plan<T, KIND, DIM>(S, P, h, nb, M);
+  }
+
+  static cudaLaunchConfig_t cluster_config(int nb, size_t smem, cudaStream_t s, cudaLaunchAttribute* attr) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim = {(unsigned)nb, 1, 1};
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim = {(unsigned)CL_MAX, 1, 1};
+    cfg.gridDim = dim3(nb);
     cfg.blockDim = dim3(CL_TPB);
-    cfg.stream = st->stream;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    ClPlan M;
-    static std::atomic<int> size{0};  // blocks of the cluster: 16, or 8 (the portable size) where 16 do not fit
-    int nb = size.load();
-    if (!nb) {
-      FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX));
-      FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      cfg.gridDim = dim3(CL_MAX);
-      cfg.dynamicSmemBytes = CL_SMEM_MAX;
+    return cfg;
+  }
+
+  // At fm_create: the kernel's attributes, which belong to the device, and the
+  // blocks of the state's cluster: 16, or 8 (the portable size) where 16 cannot be
+  // scheduled with the state's shared memory.
+  static int cluster_setup(fm_state* st) {
+    const bool used = sizeof(T) == 8 || st->coarse64;
+    if (!used || st->coarse_fused) return FM_OK;
+    const auto kernel = k_vcycle_cluster<T, KIND, DIM>;
+    FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX));
+    FM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    const char* e = getenv("FM_CLUSTER");
+    for (int nb = e && atoi(e) == 8 ? 8 : CL_MAX; nb >= 8; nb /= 2) {
+      SmallLv<T> S;
+      ClPlan M;
+      const size_t smem = cluster_plan(st, st->small_from, nb, make_phys<double>(st), S, M);
+      cudaLaunchAttribute attr[1];
+      const cudaLaunchConfig_t cfg = cluster_config(nb, smem, st->stream, attr);
       int n = 0;
-      nb = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1 ? CL_MAX : 8;
+      if (smem <= CL_SMEM_MAX && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1) {
+        st->cl_blocks = nb;
+        return FM_OK;
+      }
       cudaGetLastError();
-      size.store(nb);
     }
-    cfg.gridDim = dim3(nb);
-    attr[0].val.clusterDim = {(unsigned)nb, 1, 1};
-    cfg.dynamicSmemBytes = cl_plan<T, KIND, DIM>(S, P, h, nb, M);
-    if (cfg.dynamicSmemBytes > CL_SMEM_MAX) return FM_EINVAL;
-    if (cudaLaunchKernelEx(&cfg, kernel, S, M, P, st->prm.nu1, st->prm.nu2, st->prm.ncoarse) != cudaSuccess) {
+    return FM_ECUDA;
+  }
+
+  // The float64 V-cycle of the small levels from l down by one cluster
+  // (fm_cluster.cuh), on the levels of the state in their own precision T.
+  static int cluster_cycle(fm_state* st, int l) {
+    SmallLv<T> S;
+    ClPlan M;
+    const Phys<double> P = make_phys<double>(st);
+    const size_t smem = cluster_plan(st, l, st->cl_blocks, P, S, M);
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = cluster_config(st->cl_blocks, smem, st->stream, attr);
+    if (cudaLaunchKernelEx(&cfg, k_vcycle_cluster<T, KIND, DIM>, S, M, P, st->prm.nu1, st->prm.nu2, st->prm.ncoarse) !=
+        cudaSuccess) {
       cudaGetLastError();
       return FM_ECUDA;
     }
@@ -1287,6 +1310,13 @@ static int dispatch_autotune(fm_state* st) {
   if (st->kind == FM_PFC)
     return st->dim == 2 ? Solver<T, KPFC, 2>::autotune(st) : Solver<T, KPFC, 3>::autotune(st);
   return st->dim == 2 ? Solver<T, KCDFT, 2>::autotune(st) : Solver<T, KCDFT, 3>::autotune(st);
+}
+
+template <typename T>
+static int dispatch_cluster_setup(fm_state* st) {
+  if (st->kind == FM_PFC)
+    return st->dim == 2 ? Solver<T, KPFC, 2>::cluster_setup(st) : Solver<T, KPFC, 3>::cluster_setup(st);
+  return st->dim == 2 ? Solver<T, KCDFT, 2>::cluster_setup(st) : Solver<T, KCDFT, 3>::cluster_setup(st);
 }
 
 template <typename T>
@@ -1619,7 +1649,8 @@ int fm_create(const fm_grid* grid, const fm_params* prm, const fm_functional* fn
     }
   }
   if (st->model == FM_HYDRO && prm->walls == FM_WALLS_NONE) {
-    const int rc = prm->precision == FM_MIXED ? dispatch_autotune<float>(st) : dispatch_autotune<double>(st);
+    int rc = prm->precision == FM_MIXED ? dispatch_cluster_setup<float>(st) : dispatch_cluster_setup<double>(st);
+    if (!rc) rc = prm->precision == FM_MIXED ? dispatch_autotune<float>(st) : dispatch_autotune<double>(st);
     if (rc) {
       fm_destroy(st);
       return rc;
@@ -1656,6 +1687,8 @@ int fm_set_stream(fm_state* st, void* stream) {
 }
 
 int fm_levels(const fm_state* st) { return st ? st->nlev : FM_EINVAL; }
+
+int fm_cluster_blocks(const fm_state* st) { return st ? st->cl_blocks : FM_EINVAL; }
 
 int fm_tuning(const fm_state* st, int level, int* variant, float* ms_per_variant) {
   if (!st || level < 0 || level >= st->nlev) return FM_EINVAL;

@@ -76,6 +76,7 @@ struct fm_state {
   int rbv[fm::MAXLEV];            // chosen variant of the fused sweep per level
   float rbt[fm::MAXLEV][FM_SWEEP_VARIANTS];  // autotuner timings (ms per sweep)
   int small_from;                 // first level of the one-launch V-cycle of the small levels
+  int cl_blocks;                  // blocks of its cluster in float64 (16 or 8; 0: not used)
   void* ctl;                      // device control block of the step
   cudaGraph_t graph;
   cudaGraphExec_t gexec;

@@ -112,6 +112,7 @@ _SIGS = {
     "fm_mass_noalloc": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int), C.c_double, C.c_void_p,
                                   C.c_void_p]),
     "fm_profile": (C.c_int, [C.c_void_p, C.c_int]),
+    "fm_cluster_blocks": (C.c_int, [C.c_void_p]),
     "fm_tuning": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_float)]),
     "fm_profile_read": (C.c_int, [C.c_void_p, C.POINTER(C.c_double), C.POINTER(C.c_longlong),
                                   C.POINTER(C.c_longlong)]),
@@ -416,6 +417,11 @@ def fm_mass_noalloc(rho, h, out, stream=0):
     code = lib().fm_mass_noalloc(C.c_void_p(rho.data_ptr()), len(dims), n, C.c_double(h),
                                  C.c_void_p(out.data_ptr()), C.c_void_p(stream))
     _check(code, "fm_mass_noalloc")
+
+
+def fm_cluster_blocks(st):
+    """Blocks of the cluster of the float64 coarse V-cycle (0: not used)."""
+    return lib().fm_cluster_blocks(st)
 
 
 def fm_tuning(st, level):
