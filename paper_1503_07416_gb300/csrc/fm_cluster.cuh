@@ -591,11 +591,15 @@ __global__ void __launch_bounds__(CL_TPB) k_vcycle_cluster(const __grid_constant
 // (PFC) and 15 us (CDFT) against 32 and 37 us for four colour launches between
 // two conversions.
 constexpr int CT_TX = 8, CT_TY = 4, CT_SETS = 3;
-// Largest level swept on tiles: two tiles a multiprocessor.  Beyond it the
-// recomputed halo (2.6 point updates for one) costs more than the launches: a
-// cycle of two sweeps takes 39.6 us on tiles and 48.1 us as colour launches at
-// 128 x 64, 53.8 and 48.5 us at 128^2 (CDFT 45.4 / 59.3, 61.3 / 59.6 us).
-constexpr int CT_MAXN = 8192;
+// Swept on tiles: levels of at most two tiles a multiprocessor.  One block more
+// starts a third round, and the recomputed halo (2.6 point updates for one; far
+// more on a level narrower than a tile) then costs more than the launches.  A
+// cycle of four sweeps of a level of its own, on tiles and as colour launches:
+// 128 x 64 (256 tiles) 50.0 / 59.9 us, 128 x 76 (304) 56.2 / 65.0, 110 x 90 (322) 69.1 /
+// 66.0, 2 x 1024 (256) 130 / 139, 2 x 4096 (1,024) 194 / 144; CDFT 4096 x 2 (512) 118 / 103.
+__host__ __device__ constexpr int ct_tiles(const Geo& g) {
+  return ((g.nx + CT_TX - 1) / CT_TX) * ((g.ny + CT_TY - 1) / CT_TY);
+}
 
 template <int KIND>
 __host__ __device__ constexpr int ct_threads() { return ClDim<KIND, 2>::R * CT_SETS * 32; }

@@ -1117,7 +1117,7 @@ struct Solver {
       const Lvl<float> L = make_lvl<float>(st, l);
       const Phys<double> P = make_phys<double>(st);
       const PtK<double> K = make_ptk<double, 2>(P, st->lv[l].h);
-      const int ntx = (L.g.nx + CT_TX - 1) / CT_TX, nblk = ntx * ((L.g.ny + CT_TY - 1) / CT_TY);
+      const int ntx = (L.g.nx + CT_TX - 1) / CT_TX, nblk = ct_tiles(L.g);
       CtPtr<const float> ef{};
       CtPtr<float> of{};
       CtPtr<double> b[2] = {};
@@ -1155,13 +1155,13 @@ struct Solver {
 
   // The coarsest-grid solve in float64 (mixed path): the V-cycle of the
   // levels from l down by one cluster; or a larger coarsest level's ncoarse
-  // sweeps, on tiles (2-D, at most CT_MAXN points) or as colour launches on
+  // sweeps, on tiles (2-D, at most two a multiprocessor) or as colour launches on
   // its float64 copy between two conversions.
   // *out_in_r: on return the correction of level l is in its r buffer.
   static int coarse_solve64(fm_state* st, int l, int* out_in_r) {
     if (!st->coarse_fused) return cluster_cycle(st, l);
     if constexpr (DIM == 2 && sizeof(T) == 4) {
-      if (st->lv[l].g.N <= CT_MAXN) return coarse_tiles64(st, l, out_in_r);
+      if (ct_tiles(st->lv[l].g) <= 2 * st->sms) return coarse_tiles64(st, l, out_in_r);
     }
     int rc = coarse_to64(st, l);
     if (rc) return rc;

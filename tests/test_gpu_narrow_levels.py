@@ -1,0 +1,54 @@
+"""Levels narrower than a tile: what sweeps them is chosen by the tiles they take,
+not by their points alone, and the sweeps are the same either way."""
+import numpy as np
+import pytest
+
+from paper_1503_07416_gb300 import fm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1503_07416_gb300 import build
+    build.build_library()
+    fm.lib()
+
+
+def _one_cycle(kind, n, coarse, ncoarse):
+    """(residual left by one damped cycle, kernels of the step)."""
+    rng = np.random.default_rng(9)
+    shape = tuple(reversed(n))
+    rho = (0.8 if kind == "pfc" else 0.3) + 0.03 * rng.uniform(-1, 1, shape)
+    vel = [0.05 * rng.standard_normal(shape) for _ in n]
+    kw = dict(alpha=0.6) if kind == "pfc" else dict(nu=2.362, delta=1e-10)
+    sol = fm.Solver(kind, n, 0.9 if kind == "pfc" else 0.25, precision=fm.FM_MIXED, coarse_precision=coarse, w_damp=0.5,
+                    ncoarse=ncoarse, coarsest=8192, tol=1e-300, max_cycles=1, **kw)
+    assert fm.fm_levels(sol.handle) == 1
+    sol.set_fields(rho, vel)
+    before = fm.fm_profile_read(sol.handle)[2]
+    code, info = fm.fm_step_raw(sol.handle, 0.02)
+    launches = fm.fm_profile_read(sol.handle)[2] - before
+    sol.close()
+    assert code == fm.FM_ENOCONV and info.cycles == 1
+    return info.res, launches
+
+
+# (tiles of 8 x 4 points, at most 304 of them on a GB300): narrow levels of fewer
+# points than 128 x 64 that take more tiles, and squarer ones that take as many or fewer
+@pytest.mark.parametrize("kind,n,tiled", [("pfc", (2, 2048), False), ("pfc", (4, 2000), False), ("cdft", (4096, 2), False),
+                                          ("pfc", (110, 90), False), ("pfc", (128, 76), True), ("pfc", (2, 1024), True),
+                                          ("cdft", (1024, 8), True), ("pfc", (92, 98), True)])
+def test_coarsest_level_route(kind, n, tiled):
+    """Two launches of two sweeps on tiles; or two conversions and eight colour
+    launches.  The residual after the cycle against the float32 solve, a separate
+    implementation: they differ by the float32 rounding of a few dozen updates, a
+    few 1e-6 of it; bound 1e-4."""
+    res, launches = _one_cycle(kind, n, fm.FM_FP64, 4)
+    ref, _ = _one_cycle(kind, n, fm.FM_MIXED, 4)
+    assert abs(res - ref) <= 1e-4 * ref
+    _, more = _one_cycle(kind, n, fm.FM_FP64, 6)
+    assert more - launches == (1 if tiled else 4)
