@@ -505,7 +505,7 @@ struct Batch {
       I.partials = st->partials;
       I.tmp = st->tmp;
       I.rho = st->rho;
-      I.nblk64 = st->nblk;
+      I.nblk64 = st->nres;
     }
   }
 
@@ -522,7 +522,7 @@ struct Batch {
     for (int i = 0; i < b->count; ++i) v.push_back({i, prep_tiles(b->inst[i]->lv[0].g.nx, b->inst[i]->lv[0].g.ny)});
     b->w_prep = add_list(b, v);
     v.clear();
-    for (int i = 0; i < b->count; ++i) v.push_back({i, b->inst[i]->nblk});
+    for (int i = 0; i < b->count; ++i) v.push_back({i, b->inst[i]->nres});
     b->w_resid64 = add_list(b, v);
     v.clear();
     for (int i = 0; i < b->count; ++i) {

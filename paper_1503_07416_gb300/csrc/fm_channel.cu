@@ -284,8 +284,9 @@ __device__ __forceinline__ double gv(const double* x, int i, int N, int type, co
 
 // omega^k, S, g^0 (kappa^0 = Lap_h rho^k) with the wall ghosts: 7.1 us at 256^2,
 // 10.7 point by point.
+template <int TX>
 __global__ void __launch_bounds__(TPB) k_ch_prepare(Fields64 F, Geo G, Step64 K, Phys<double> P, Walls64 W) {
-  prepare_tile<KPFC, true>(F, G, K, P, blockIdx.x, W);
+  prepare_tile<KPFC, true, TX>(F, G, K, P, blockIdx.x, W);
 }
 
 // mu^0 = psi^3/3 + alpha psi + Lap_h kappa^0 + S_mu; the blocks after the last
@@ -314,10 +315,10 @@ __global__ void __launch_bounds__(TPB) k_ch_prepare_mu(Fields64 F, Geo G, Step64
 // cycle and the block partial sums of r^2 (15.3 us a launch at 256^2 point by
 // point with the wall rows' ghosts chosen at every load, 11.2 on the periodic
 // solver's tiles, whose halo rows hold the ghosts).
-template <typename T>
+template <typename T, int TX>
 __global__ void __launch_bounds__(TPB, 4) k_ch_resid64(Fields64 F, Resid64Out O, Geo G, Step64 K, Phys<double> P,
                                                        Walls64 W, double* partials) {
-  resid64_tile_body<KPFC, T, true>(F, O, G, K, P, partials, blockIdx.x, gridDim.x, W);
+  resid64_tile_body<KPFC, T, true, TX>(F, O, G, K, P, partials, blockIdx.x, gridDim.x, W);
 }
 
 // rho^{k+1} = S1 - (s/4h) sum_d ([rho^k u_d]_{+d} - [rho^k u_d]_{-d}) with the
@@ -411,7 +412,12 @@ struct ChannelSolver {
   static int enqueue_prepare(fm_state* st) {
     const Geo G = st->lv[0].g;
     const Fields64 F = make_fields(st);
-    k_ch_prepare<<<prep_tiles(G.nx, G.ny), TPB, 0, st->stream>>>(F, G, step64(st), make_phys<double>(st), walls64(st));
+    if (narrow_tiles(G))
+      k_ch_prepare<R64_NARROW><<<prep_tiles<R64_NARROW>(G.nx, G.ny), TPB, 0, st->stream>>>(
+          F, G, step64(st), make_phys<double>(st), walls64(st));
+    else
+      k_ch_prepare<PT_TX><<<prep_tiles(G.nx, G.ny), TPB, 0, st->stream>>>(F, G, step64(st), make_phys<double>(st),
+                                                                        walls64(st));
     FM_LAUNCHED();
     const InjAll<T> A = injection(st, 0);
     k_ch_prepare_mu<T><<<nblocks(G.N) + nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(F, G, step64(st), st->fn.alpha,
@@ -421,8 +427,14 @@ struct ChannelSolver {
   }
 
   static int launch_resid64(fm_state* st, const Resid64Out& O) {
-    k_ch_resid64<T><<<st->nblk, TPB, 0, st->stream>>>(make_fields(st), O, st->lv[0].g, step64(st),
-                                                       make_phys<double>(st), walls64(st), st->partials);
+    const Geo G = st->lv[0].g;
+    const Phys<double> P = make_phys<double>(st);
+    if (narrow_tiles(G))
+      k_ch_resid64<T, R64_NARROW><<<st->nres, TPB, 0, st->stream>>>(make_fields(st), O, G, step64(st), P, walls64(st),
+                                                                    st->partials);
+    else
+      k_ch_resid64<T, R64_TX><<<st->nres, TPB, 0, st->stream>>>(make_fields(st), O, G, step64(st), P, walls64(st),
+                                                               st->partials);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -433,7 +445,7 @@ struct ChannelSolver {
     const double h = st->lv[0].h;
     const InjAll<T> A = injection(st, 1);
     k_norm_ctl<LY::NU, InjRows, T><<<1 + nblocks(A.off[st->nlev]), TPB, 0, st->stream>>>(
-        st->partials, st->nblk, h * h, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
+        st->partials, st->nres, h * h, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -508,7 +520,7 @@ struct ChannelSolver {
     int rc = launch_resid64(st, out0(st, false, r64));
     if (rc) return rc;
     const double h = st->lv[0].h;
-    k_norm_final<LY::NU><<<1, TPB, 0, st->stream>>>(st->partials, st->nblk, h * h, st->dscal);
+    k_norm_final<LY::NU><<<1, TPB, 0, st->stream>>>(st->partials, st->nres, h * h, st->dscal);
     FM_LAUNCHED();
     FM_CUDA(cudaMemcpyAsync(st->hscal, st->dscal, sizeof(double), cudaMemcpyDeviceToHost, st->stream));
     FM_CUDA(cudaStreamSynchronize(st->stream));

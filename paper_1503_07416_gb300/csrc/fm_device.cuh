@@ -2138,23 +2138,26 @@ __device__ __forceinline__ void ghost_velocity(double& u, double& v, int y, int 
 // rho^k u, rho^k v (PFC: rho^k) of the tile and its one-point halo in shared
 // memory, so that the products are formed once a cell, and the Laplacians in
 // fixed point: 13.9 us at 512^2 (float64 sums 20.0, 20.8 point by point).
-constexpr int PT_TX = 32, PT_TY = 8, PT_SW = PT_TX + 2, PT_SN = PT_SW * (PT_TY + 2);
+constexpr int PT_TX = 32;  // width; TX x TY = 256 points
+template <int TX = PT_TX>
 __host__ __device__ constexpr int prep_tiles(int nx, int ny) {
-  return ((nx + PT_TX - 1) / PT_TX) * ((ny + PT_TY - 1) / PT_TY);
+  constexpr int TY = TPB / TX;
+  return ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
 }
 
-template <int KIND, bool WALLS = false>
+template <int KIND, bool WALLS = false, int TX = PT_TX>
 __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, const Step64& K, const Phys<double>& P,
                                              int tile, const Walls64& W = Walls64{}) {
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
   constexpr int NA = PFC ? 5 : 4;
-  __shared__ double sX[NA][PT_SN];
+  constexpr int TY = TPB / TX, SW = TX + 2, SN = SW * (TY + 2);
+  __shared__ double sX[NA][SN];
   const int nx = G.nx, ny = G.ny;
-  const int ntx = (nx + PT_TX - 1) / PT_TX;
-  const int x0 = (tile % ntx) * PT_TX, y0 = (tile / ntx) * PT_TY;
-  for (int t = threadIdx.x; t < PT_SN; t += TPB) {
-    const int ly = t / PT_SW, lx = t - ly * PT_SW, y = y0 + ly - 1;
+  const int ntx = (nx + TX - 1) / TX;
+  const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+  for (int t = threadIdx.x; t < SN; t += TPB) {
+    const int ly = t / SW, lx = t - ly * SW, y = y0 + ly - 1;
     const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
     double u = F.vel[0][gi], v = F.vel[1][gi];
     const double r = F.rho[gi];
@@ -2166,11 +2169,11 @@ __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, co
     if constexpr (PFC) sX[4][t] = r;
   }
   __syncthreads();
-  const int i = x0 + (threadIdx.x & 31), j = y0 + (threadIdx.x >> 5);
+  const int i = x0 + (threadIdx.x % TX), j = y0 + (threadIdx.x / TX);
   if (i >= nx || j >= ny) return;
   const int idx = j * nx + i;
-  const int c = ((threadIdx.x >> 5) + 1) * PT_SW + (threadIdx.x & 31) + 1;
-  const int xm = c - 1, xp = c + 1, ym = c - PT_SW, yp = c + PT_SW;
+  const int c = ((threadIdx.x / TX) + 1) * SW + (threadIdx.x % TX) + 1;
+  const int xm = c - 1, xp = c + 1, ym = c - SW, yp = c + SW;
   const double w = K.hih * ((sX[1][xp] - sX[1][xm]) - (sX[0][yp] - sX[0][ym]));
   const double div = (sX[2][xp] - sX[2][xm]) + (sX[3][yp] - sX[3][ym]);
   const double rk = F.rho[idx], uc[2] = {sX[0][c], sX[1][c]};
@@ -2178,8 +2181,8 @@ __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, co
     if (F.nonpos && rk <= 0.0) atomicOr(F.nonpos, 1);  // ln rho^k undefined: FM_ENONPOS
   }
   const double cw = K.c_w * w;
-  double sv[2] = {fma(K.c_v, lap_tile<PT_SW>(sX[0] + c), rk * fma(cw, uc[1], uc[0])),
-                  fma(K.c_v, lap_tile<PT_SW>(sX[1] + c), rk * fma(-cw, uc[0], uc[1]))};
+  double sv[2] = {fma(K.c_v, lap_tile<SW>(sX[0] + c), rk * fma(cw, uc[1], uc[0])),
+                  fma(K.c_v, lap_tile<SW>(sX[1] + c), rk * fma(-cw, uc[0], uc[1]))};
   if constexpr (!PFC) {
     const Nb n = neighbours(i, j, 0, G);
 #pragma unroll
@@ -2189,7 +2192,7 @@ __device__ __forceinline__ void prepare_tile(const Fields64& F, const Geo& G, co
       sv[a] += K.c_m * rk * (Ep - Em);
     }
   }
-  const double lapr = PFC ? lap_tile<PT_SW>(sX[NA - 1] + c) * K.ih2 : 0.0;
+  const double lapr = PFC ? lap_tile<SW>(sX[NA - 1] + c) * K.ih2 : 0.0;
   const bool keep = F.hist && *F.hist > 0;  // g^0 extrapolated in time already (k_extrapolate)
   F.S[0][idx] = fma(-K.c_div, div, rk);
 #pragma unroll
@@ -2422,19 +2425,31 @@ struct Resid64Out {
 // 25.6 us a launch at 512^2 (float64 Laplacians 34.4; the form before 36.8), 83 us
 // at 1024^2 (122 before).  Bounded to three blocks a multiprocessor; to four
 // 26.3 and 82 us.
-constexpr int R64_TX = 32, R64_TY = 8;
-constexpr int R64_SW = R64_TX + 2, R64_SN = R64_SW * (R64_TY + 2);
+// TX: the tile's width (TX x TY = 256 points, 340 with the halo for 32 and 8).
+constexpr int R64_TX = 32;
+template <int TX = R64_TX>
+__host__ __device__ constexpr int r64_tiles(const Geo& g) {
+  constexpr int TY = TPB / TX;
+  return ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
+}
 
-template <int KIND, typename T, bool WALLS = false>
+// The channel's residual and source take tiles of 8 x 32 where 32 columns would be
+// mostly halo: a channel 2 points wide fills a quarter of them instead of a
+// sixteenth.
+constexpr int R64_NARROW = 8;
+static inline bool narrow_tiles(const Geo& g) { return g.nx <= 2 * R64_NARROW; }
+
+template <int KIND, typename T, bool WALLS = false, int TX = R64_TX>
 __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid64Out& O, const Geo& G,
                                                   const Step64& K,
                                                   const Phys<double>& P, double* partials, int lb, int nb,
                                                   const Walls64& W = Walls64{}) {
   using LY = Layout<KIND, 2>;
   constexpr bool PFC = KIND == KPFC;
+  constexpr int TY = TPB / TX, SW = TX + 2, SN = SW * (TY + 2);
   // staged: u, v (PFC: kappa, rho), whose Laplacians are taken; |u|^2, mu, rho^k u, rho^k v
   constexpr int NL = PFC ? 4 : 2, NS = NL + 4;
-  __shared__ double sX[NS][R64_SN];
+  __shared__ double sX[NS][SN];
   double acc[LY::NU];
 #pragma unroll
   for (int q = 0; q < LY::NU; ++q) acc[q] = 0.0;
@@ -2444,13 +2459,13 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
   const double ih2 = K.ih2, c_div = K.c_div, c_w = K.c_w, c_q = K.c_div, c_v = K.c_v;
   const double third = 1.0 / 3.0;
   const int nx = G.nx, ny = G.ny;
-  const int ntx = (nx + R64_TX - 1) / R64_TX;
-  const int ntiles = ntx * ((ny + R64_TY - 1) / R64_TY);
+  const int ntx = (nx + TX - 1) / TX;
+  const int ntiles = r64_tiles<TX>(G);
   const double* const* g = F.g;
   for (int tile = lb; tile < ntiles; tile += nb) {
-    const int x0 = (tile % ntx) * R64_TX, y0 = (tile / ntx) * R64_TY;
-    for (int t = threadIdx.x; t < R64_SN; t += TPB) {
-      const int ly = t / R64_SW, lx = t - ly * R64_SW, y = y0 + ly - 1;
+    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    for (int t = threadIdx.x; t < SN; t += TPB) {
+      const int ly = t / SW, lx = t - ly * SW, y = y0 + ly - 1;
       const int gi = tile_row<WALLS>(y, ny) * nx + wrapi(x0 + lx - 1, nx);
       double u = g[1][gi], v = g[2][gi], m;
       const double rk = F.rho[gi], r = g[0][gi];
@@ -2470,12 +2485,12 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
       sX[NL + 3][t] = rk * v;
     }
     __syncthreads();
-    const int ty = threadIdx.x / R64_TX, tx = threadIdx.x - ty * R64_TX;
+    const int ty = threadIdx.x / TX, tx = threadIdx.x - ty * TX;
     const int i = x0 + tx, j = y0 + ty;
     if (i < nx && j < ny) {
       const int idx = j * nx + i;
-      const int c = (ty + 1) * R64_SW + tx + 1;
-      const int xm = c - 1, xp = c + 1, ym = c - R64_SW, yp = c + R64_SW;
+      const int c = (ty + 1) * SW + tx + 1;
+      const int xm = c - 1, xp = c + 1, ym = c - SW, yp = c + SW;
       const double rkc = __ldg(F.rho + idx), w = __ldg(F.om[0] + idx);
       const double uc = sX[0][c], vc = sX[1][c], g0c = PFC ? sX[NL - 1][c] : g[0][idx];
       auto S = [&](int q) { return __ldg(F.S[q] + idx); };
@@ -2489,13 +2504,13 @@ __device__ __forceinline__ void resid64_tile_body(const Fields64& F, const Resid
       const double dqx = fma(2.0, dif(NL + 1, xp, xm), dif(NL, xp, xm));
       const double dqy = fma(2.0, dif(NL + 1, yp, ym), dif(NL, yp, ym));
       row(0, fma(-c_div, dif(NL + 2, xp, xm) + dif(NL + 3, yp, ym), S(0) - g0c));
-      row(1, fma(c_v, lap_tile<R64_SW>(sX[0] + c), fma(-rkc, fma(c_q, dqx, fma(-cw, vc, uc)), S(1))));
-      row(2, fma(c_v, lap_tile<R64_SW>(sX[1] + c), fma(-rkc, fma(c_q, dqy, fma(cw, uc, vc)), S(2))));
+      row(1, fma(c_v, lap_tile<SW>(sX[0] + c), fma(-rkc, fma(c_q, dqx, fma(-cw, vc, uc)), S(1))));
+      row(2, fma(c_v, lap_tile<SW>(sX[1] + c), fma(-rkc, fma(c_q, dqy, fma(cw, uc, vc)), S(2))));
       if constexpr (PFC) {
         const double psi = g0c - 1.5;
-        row(LY::IMU, S(LY::IMU) - fma(-ih2, lap_tile<R64_SW>(sX[2] + c),
+        row(LY::IMU, S(LY::IMU) - fma(-ih2, lap_tile<SW>(sX[2] + c),
                                       fma(-psi, fma(psi * psi, third, P.alpha), sX[NL + 1][c])));
-        row(LY::IKA, fma(ih2, lap_tile<R64_SW>(sX[3] + c), -sX[2][c]));  // S_kappa = 0
+        row(LY::IKA, fma(ih2, lap_tile<SW>(sX[3] + c), -sX[2][c]));  // S_kappa = 0
       }
       if (O.cr32) {
         O.cr32[idx] = narrow_rn(g0c);

@@ -777,7 +777,7 @@ struct Solver {
                             const Phys<double>& P, bool update = false) {
     cudaStream_t s = st->stream;
     if constexpr (DIM == 2) {
-      k_resid64_tile<KIND, T><<<st->nblk, TPB, 0, s>>>(F, O, G, make_step64(P, 1.0 / h), P, st->partials);
+      k_resid64_tile<KIND, T><<<st->nres, TPB, 0, s>>>(F, O, G, make_step64(P, 1.0 / h), P, st->partials);
       FM_LAUNCHED();
     } else {
       const Shared64 X = shared64(st);
@@ -786,7 +786,7 @@ struct Solver {
       else
         k_shared64<KIND, DIM><<<nblocks(G.N), TPB, 0, s>>>(F, X, G.N, P.ce);
       FM_LAUNCHED();
-      k_resid64_x<KIND, DIM, T><<<st->nblk, TPB, 0, s>>>(F, X, O, G, make_step64(P, 1.0 / h), P,
+      k_resid64_x<KIND, DIM, T><<<st->nres, TPB, 0, s>>>(F, X, O, G, make_step64(P, 1.0 / h), P,
                                                            st->partials);
       FM_LAUNCHED();
     }
@@ -808,7 +808,7 @@ struct Solver {
     const double w = (DIM == 3) ? h * h * h : h * h;
     const InjAll<T> A = injection(st, true);
     k_norm_ctl<LY::NU, InjSample, T><<<1 + nblocks(A.off[st->nlev]), TPB, 0, s>>>(
-        st->partials, st->nblk, w, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
+        st->partials, st->nres, w, (Ctl*)st->ctl, st->prm.tol, st->prm.max_cycles, in_body, hdl, use_handle, A);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -824,7 +824,7 @@ struct Solver {
     int rc = launch_resid64(st, F, O, G, h, P);
     if (rc) return rc;
     const double w = (DIM == 3) ? h * h * h : h * h;
-    k_norm_final<LY::NU><<<1, TPB, 0, s>>>(st->partials, st->nblk, w, st->dscal);
+    k_norm_final<LY::NU><<<1, TPB, 0, s>>>(st->partials, st->nres, w, st->dscal);
     FM_LAUNCHED();
     FM_CUDA(cudaMemcpyAsync(st->hscal, st->dscal, sizeof(double), cudaMemcpyDeviceToHost, s));
     FM_CUDA(cudaStreamSynchronize(s));
@@ -1380,7 +1380,7 @@ static size_t carve(fm_state* st, char* base) {
     st->x64[q] = (st->model == FM_HYDRO && st->dim == 3 && (q < 4 || st->kind == FM_CDFT))
                      ? (double*)C.take(N0 * d8)
                      : nullptr;
-  st->partials = (double*)C.take((size_t)st->nblk * 8 * d8);
+  st->partials = (double*)C.take((size_t)(st->nblk > st->nres ? st->nblk : st->nres) * 8 * d8);
   st->dscal = (double*)C.take(64 * d8);
   st->ctl = C.take(64);
   for (int l = 0; l < st->nlev; ++l) {
@@ -1613,6 +1613,15 @@ int fm_create(const fm_grid* grid, const fm_params* prm, const fm_functional* fn
   }
   const int need = (int)((st->lv[0].g.N + TPB - 1) / TPB);
   st->nblk = need < 4 * sms ? need : 4 * sms;
+  // a block a tile while four a multiprocessor hold them: counted in points, a grid
+  // 2 points wide gave each block 16 tiles one after the other (2 x 8192, us a cycle:
+  // channel 142, a block a tile 69, on narrow tiles 49; periodic 151 and 83)
+  st->nres = st->nblk;
+  if (st->dim == 2 && st->model == FM_HYDRO) {
+    const Geo& G = st->lv[0].g;
+    const int tiles = st->prm.walls == FM_WALLS_Y && narrow_tiles(G) ? r64_tiles<R64_NARROW>(G) : r64_tiles(G);
+    st->nres = tiles < 4 * sms ? tiles : 4 * sms;
+  }
   const size_t bytes = carve(st, nullptr);
   void* arena = nullptr;
   if (cudaMalloc(&arena, bytes) != cudaSuccess) {

@@ -58,6 +58,7 @@ struct fm_state {
   double* x64[5];                 // 3-D: per-point quantities shared by the residual
   double* partials;               // per-block partial sums (deterministic reductions)
   int nblk;                       // blocks of the reduction kernels
+  int nres;                       // blocks of the float64 residual (2-D hydrodynamic: of its tiles)
   int sms;                        // multiprocessors of the device
   int smem_optin;                 // shared memory per block (opt-in maximum)
   double* dscal;                  // device scalars

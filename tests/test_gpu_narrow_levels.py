@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from paper_1503_07416_gb300 import fm
+from tests.test_gpu_fixed_point import test_source_and_residual_rows as _rows
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +53,11 @@ def test_coarsest_level_route(kind, n, tiled):
     assert abs(res - ref) <= 1e-4 * ref
     _, more = _one_cycle(kind, n, fm.FM_FP64, 6)
     assert more - launches == (1 if tiled else 4)
+
+
+@pytest.mark.parametrize("vel_of", ["ordinary", "spike"])
+@pytest.mark.parametrize("n", [(2, 600), (8, 34), (10, 66), (16, 32), (16, 2), (18, 34)])
+def test_narrow_channel_rows(n, vel_of):
+    """The channel's source and residual on 8 x 32 tiles (up to 16 points wide) and
+    just beyond: rows, ghosts and ragged tiles as in test_gpu_fixed_point."""
+    _rows("pfc", n, "walls", vel_of)
