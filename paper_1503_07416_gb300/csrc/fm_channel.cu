@@ -243,6 +243,7 @@ struct ChPol {
   using W = WallsT<T>;
   static constexpr int NU = LY::NU, NC = 4;
   static constexpr bool WALLS = true;
+  static constexpr int TILED64 = 1 << 30;  // points a multiprocessor up to which float64 sweeps on tiles (fz_tile)
   __host__ __device__ static K constants(const Phys<T>& P, T h) { return make_ptk<T, 2>(P, h); }
   __device__ static const T* coef(const Lvl<T>& L, int c) {
     return c == 0 ? L.cr : (c == 1 ? L.rk : L.cv[c - 2]);
@@ -465,19 +466,19 @@ struct ChannelSolver {
     }
     const Lvl<T> L = make_lvl<T>(st, l);
     if (l == st->nlev - 1) {
-      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, s));
+      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, st->sms, s));
       return FM_OK;
     }
     const Lvl<T> C = make_lvl<T>(st, l + 1);
     int c_in_r = 0;
-    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, s));
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, st->sms, s));
     const Lvl<T> F = fz_view(L, *out_in_r);
     FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
     const int rc = vcycle(st, l + 1, P, &c_in_r);
     if (rc) return rc;
     k_ch_prolong<T><<<nblocks(F.g.N), TPB, 0, s>>>(F, fz_view(C, c_in_r));
     FM_LAUNCHED();
-    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, st->sms, s));
     return FM_OK;
   }
 

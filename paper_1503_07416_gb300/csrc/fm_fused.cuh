@@ -136,6 +136,14 @@ __global__ void __launch_bounds__(rb_threads(TX, TY), rb_minb<typename M::T>(TX,
   }
 }
 
+// One colour of a sweep, in place, a point a thread (see fz_tiled).
+template <class M>
+__global__ void __launch_bounds__(TPB) kf_colour(const __grid_constant__ Lvl<typename M::T> L, Phys<typename M::T> P,
+                                                 typename M::K K, typename M::W W, int color) {
+  int i, j, k;
+  if (colour_point(blockIdx.x * blockDim.x + threadIdx.x, color, L.g, i, j, k)) M::update_lvl(L, P, K, W, i, j);
+}
+
 // f_C = R(f - M(e)) + M_C(e_C), e_C = eh_C = the injection of e, on RR_TX x
 // RR_TY coarse points a block (see k_resid_restrict2; between walls the
 // restriction and injection average rows 2J and 2J + 1).  The correction is
@@ -262,19 +270,66 @@ static cudaError_t fz_launch_smooth(const Lvl<typename M::T>& L, const Phys<type
   return cudaPeekAtLastError();
 }
 
-// `iters` sweeps of a level (the correction in r if *in_r), two a launch while
-// two are left.  Tiles of 32 x 16 on levels of at least 256^2 points, 16 x 8
-// below, where 32 x 16 leaves multiprocessors without a tile: a cycle of 20
-// sweeps takes 59.9 / 55.6 us (flow), 84.1 / 75.2 us (channel) with the large
-// and the small tiles at 256 x 128, 63.5 / 63.6 and 92.4 / 96.1 us at 256^2,
-// 78.8 / 81.7 and 127 / 140 us at 512 x 256; float64 alike.
-// float64 takes one sweep a launch: the two-sweep tile's wider halo is 1.3 to
-// 1.7 times the point updates, which are what bounds it.
+// The view of a level whose correction is in r.
+template <typename T>
+static Lvl<T> fz_view(Lvl<T> L, int in_r) {
+  if (in_r)
+    for (int q = 0; q < MAXU; ++q) {
+      T* t = L.e[q];
+      L.e[q] = L.r[q];
+      L.r[q] = t;
+    }
+  return L;
+}
+
+// What sweeps a level: 0 a launch per colour, 1 tiles of 16 x 8, 2 of 32 x 16.
+// A level of four sweeps, us a cycle, colour / 16 x 8 / 32 x 16:
+//  * float32, tiles run two sweeps a launch: channel 128^2 46 / 33 / 35, 512^2 88 / 84 /
+//    78, flow 31 / 26 / 27 and 50 / 49 / 46; large tiles from 256^2 points on.  Levels
+//    narrower than a tile compute its columns for nothing: they stay on tiles while
+//    a few tiles a multiprocessor hold them (channel 8192 x 2, 512 tiles, 48 / 34 / 34;
+//    2 x 16384, 2,048 tiles, 56 / 78 / 94) or less than half is added (65536 x 4 92 / 95 / 102).
+//  * float64 is bound by the busiest multiprocessor's point updates, a tile's ring
+//    among them (562 a sweep for 32 x 16, 154 for 16 x 8): tiles of at most two a
+//    multiprocessor (128^2 76 / 59 / 94), or where these are below 1.35 a point
+//    (channel 512^2 299 / 300 / 303, in the step 301 against 332; 300 x 500 186 / 185 / 229;
+//    150 x 250 79 / 87 / 98).  The flow's update reads too little for the tile to
+//    pay once the pipe is full (M::TILED64): 128^2 44 / 39 / 55, 512^2 129 / 155 / 150.
+template <class M>
+static int fz_tile(const Geo& g, int sms) {
+  auto tiles = [&](int tx, int ty) { return (long long)((g.nx + tx - 1) / tx) * ((g.ny + ty - 1) / ty); };
+  const long long big = tiles(32, 16), small = tiles(16, 8);
+  if (sizeof(typename M::T) == 4) {
+    if (g.N >= 256 * 256 && 4 * 512 * big <= 5LL * g.N) return 2;
+    return small <= 4 * sms || 2 * 128 * small <= 3LL * g.N ? 1 : 0;
+  }
+  if (g.N > (long long)M::TILED64 * sms) return 0;
+  // point updates of a sweep on the busiest multiprocessors, times their number
+  auto cost = [&](long long t, int updates) { return (t + sms - 1) / sms * sms * updates; };
+  if (g.N >= 256 * 256 && 100 * cost(big, 562) <= 135LL * g.N) return 2;
+  return small <= 2 * sms || 100 * cost(small, 154) <= 135LL * g.N ? 1 : 0;
+}
+
+// `iters` sweeps of a level (the correction in r if *in_r), on tiles two a launch
+// while two are left.  float64 takes one sweep a launch: the two-sweep tile's wider
+// halo is 1.3 to 1.7 times the point updates, which are what bounds it.
 template <class M>
 static cudaError_t fz_smooth(const Lvl<typename M::T>& L, const Phys<typename M::T>& P, const typename M::W& W,
-                             int iters, int* in_r, long long* launches, cudaStream_t s) {
+                             int iters, int* in_r, long long* launches, int sms, cudaStream_t s) {
   const typename M::K K = M::constants(P, L.h);
-  const bool big = L.g.N >= 256 * 256;
+  const int tile = fz_tile<M>(L.g, sms);
+  if (!tile) {
+    const Lvl<typename M::T> V = fz_view(L, *in_r);
+    const int tpb = point_tpb<typename M::T>(L.g.N / 2, sms);
+    for (int c = 0; c < 2 * iters; ++c) {
+      kf_colour<M><<<blocks_of(L.g.N / 2, tpb), tpb, 0, s>>>(V, P, K, W, c & 1);
+      const cudaError_t e = cudaPeekAtLastError();
+      if (e != cudaSuccess) return e;
+      ++*launches;
+    }
+    return cudaSuccess;
+  }
+  const bool big = tile == 2;
   for (int it = 0; it < iters;) {
     cudaError_t e;
     if (sizeof(typename M::T) == 4 && it + 2 <= iters) {
@@ -291,18 +346,6 @@ static cudaError_t fz_smooth(const Lvl<typename M::T>& L, const Phys<typename M:
     ++*launches;
   }
   return cudaSuccess;
-}
-
-// The view of a level whose correction is in r.
-template <typename T>
-static Lvl<T> fz_view(Lvl<T> L, int in_r) {
-  if (in_r)
-    for (int q = 0; q < MAXU; ++q) {
-      T* t = L.e[q];
-      L.e[q] = L.r[q];
-      L.r[q] = t;
-    }
-  return L;
 }
 
 template <class M>

@@ -145,6 +145,7 @@ struct GfPol {
   using W = GfW;
   static constexpr int NU = GL<KIND>::NU, NC = 1;
   static constexpr bool WALLS = false;
+  static constexpr int TILED64 = 256;  // points a multiprocessor up to which float64 sweeps on tiles (fz_tile)
   __host__ __device__ static K constants(const Phys<T>& P, T h) { return make_gk<T, 2>(P, h); }
   __device__ static const T* coef(const Lvl<T>& L, int) { return L.cr; }
   template <class A>
@@ -478,12 +479,12 @@ struct GFSolver {
     }
     const Lvl<T> L = make_lvl<T>(st, l);
     if (l == st->nlev - 1) {
-      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, s));
+      FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.ncoarse, out_in_r, &st->launches, st->sms, s));
       return FM_OK;
     }
     const Lvl<T> C = make_lvl<T>(st, l + 1);
     int c_in_r = 0;
-    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, s));
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu1, out_in_r, &st->launches, st->sms, s));
     const Lvl<T> F = fz_view(L, *out_in_r);
     FM_CUDA(fz_down<Pol>(F, C, P, W, &st->launches, s));
     const int rc = vcycle2(st, l + 1, P, &c_in_r);
@@ -491,7 +492,7 @@ struct GFSolver {
     const int tp = point_tpb<T>(C.g.N, st->sms);
     k_prolong<T, NU, 2><<<blocks_of(C.g.N, tp), tp, 0, s>>>(F, fz_view(C, c_in_r), P);
     FM_LAUNCHED();
-    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, s));
+    FM_CUDA(fz_smooth<Pol>(L, P, W, st->prm.nu2, out_in_r, &st->launches, st->sms, s));
     return FM_OK;
   }
 

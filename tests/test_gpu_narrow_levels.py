@@ -3,8 +3,12 @@ not by their points alone, and the sweeps are the same either way."""
 import numpy as np
 import pytest
 
+from oracle import channel as Ch
+from oracle import gradflow as GF
+from oracle import scheme as S
 from paper_1503_07416_gb300 import fm
 from tests.test_gpu_fixed_point import test_source_and_residual_rows as _rows
+from tests.test_gpu_fused import _lagged_ghost_update
 
 pytestmark = pytest.mark.gpu
 
@@ -61,3 +65,53 @@ def test_narrow_channel_rows(n, vel_of):
     """The channel's source and residual on 8 x 32 tiles (up to 16 points wide) and
     just beyond: rows, ghosts and ragged tiles as in test_gpu_fixed_point."""
     _rows("pfc", n, "walls", vel_of)
+
+
+# a level of its own: narrow ones swept by colour launches and on tiles, the float64
+# flow on either side of its line, a level of 2.1 tiles a multiprocessor
+SWEEPS = [("gradflow", (2, 8192), fm.FM_MIXED, "colour"), ("gradflow", (8192, 2), fm.FM_MIXED, "tiles"),
+          ("gradflow", (2, 4096), fm.FM_FP64, "colour"), ("gradflow", (128, 128), fm.FM_FP64, "tiles"),
+          ("gradflow", (256, 160), fm.FM_FP64, "colour"), ("gradflow", (66, 1000), fm.FM_MIXED, "tiles"),
+          ("walls", (2, 8192), fm.FM_MIXED, "colour"), ("walls", (8, 1024), fm.FM_MIXED, "tiles"),
+          ("walls", (2, 4096), fm.FM_FP64, "colour"), ("walls", (150, 250), fm.FM_FP64, "colour"),
+          ("walls", (136, 144), fm.FM_FP64, "tiles"), ("walls", (256, 256), fm.FM_FP64, "tiles")]
+
+
+@pytest.mark.parametrize("model,n,precision,route", SWEEPS)
+def test_fused_solvers_route(model, n, precision, route, monkeypatch):
+    """Launches of two more sweeps: four per colour, one of two sweeps on float32
+    tiles, two on float64 tiles.  The residual after a cycle of six sweeps against the
+    oracle's, with the bounds of test_gpu_fused."""
+    rng = np.random.default_rng(5)
+    shape, h, s = tuple(reversed(n)), 0.9, 0.02
+    rho = 0.8 + 0.05 * rng.uniform(-1, 1, shape)
+    P = S.Params(kind=S.PFC, dim=2, h=h, s=s, alpha=0.6, w_damp=0.5)
+    opts = S.SolverOpts(coarsest=8192, ncoarse=6)
+    if model == "gradflow":
+        kw, vel, W = dict(model=fm.FM_GRADFLOW), None, None
+        f, g = GF.source(rho, P), GF.initial_iterate(rho, P)
+        GF.vcycle(g, f, P, opts)
+        want = S.res_norm(GF.residual(g, f, P), h)
+    else:
+        monkeypatch.setattr(Ch, "point_update", _lagged_ghost_update)
+        W = Ch.Walls(-2e-3, 1e-3)
+        kw, vel = dict(walls=fm.FM_WALLS_Y, u_wall=(W.u_bot, W.u_top)), [1e-3 * rng.standard_normal(shape) for _ in n]
+        c = Ch.Coeffs(rho, Ch.vorticity(vel, h, W))
+        f, g = Ch.source(rho, vel, c.om, P, W), Ch.initial_iterate(rho, vel, P, W)
+        Ch.vcycle(g, f, c, P, W, opts)
+        want = S.res_norm(Ch.residual(g, f, c, P, W), h)
+    count, res = [], 0.0
+    for sweeps in (4, 6):
+        sol = fm.Solver("pfc", n, h, alpha=0.6, precision=precision, w_damp=0.5, ncoarse=sweeps, coarsest=8192, tol=1e-300,
+                        max_cycles=1, **kw)
+        assert fm.fm_levels(sol.handle) == 1
+        sol.set_fields(rho, vel)
+        before = fm.fm_profile_read(sol.handle)[2]
+        code, info = fm.fm_step_raw(sol.handle, s)
+        count.append(fm.fm_profile_read(sol.handle)[2] - before)
+        res = info.res
+        sol.close()
+        assert code == fm.FM_ENOCONV and info.cycles == 1
+    assert count[1] - count[0] == (4 if route == "colour" else (2 if precision == fm.FM_FP64 else 1))
+    bound = 1e-3 if model == "walls" else (1e-7 if precision == fm.FM_FP64 else 1e-4)
+    assert abs(res - want) <= bound * want, (res, want)
