@@ -416,25 +416,21 @@ static void fixed_variants(fm_state* st, const char* spec, int nvar) {
   }
 }
 
-// Element-wise conversions of up to CONV_MAX arrays in one launch: array a
-// (n[a] values) from src[a] to dst[a], block row blockIdx.y taking array a.
-constexpr int CONV_MAX = 96;
-// the coarse solve's conversions: the entry level's f and e, and rk, cr, omega
-// (3) and the coefficient velocity (3) of up to MAXSMALL levels
-static_assert(CONV_MAX >= 2 * MAXU + MAXSMALL * 8, "room for every array the coarse-solve conversions copy");
+// Element-wise conversions of arrays of n values in one launch: array a from
+// src[a] to dst[a], block row blockIdx.y taking array a.
+constexpr int CONV_MAX = 2 * MAXU + 2 + 3 + 3;  // a level's f and e, rk and cr, omega, the coefficient velocity
 template <typename A, typename B>
 struct ConvSet {
   const A* src[CONV_MAX];
   B* dst[CONV_MAX];
-  int n[CONV_MAX];
+  int n;
   int count;
-  int maxn;
 };
 template <typename A, typename B>
 __global__ void __launch_bounds__(TPB) k_convert_set(const __grid_constant__ ConvSet<A, B> C) {
   const int a = blockIdx.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < C.n[a]) C.dst[a][i] = static_cast<B>(C.src[a][i]);
+  if (i < C.n) C.dst[a][i] = static_cast<B>(C.src[a][i]);
 }
 
 // e = r on every point of a level (the correction back in e).
@@ -1063,48 +1059,38 @@ struct Solver {
     return FM_OK;
   }
 
-  // Conversions between the coarse levels and their float64 copies (lv64):
-  // to64 copies the entry level l's right-hand side and correction and the
-  // coefficients of levels l .. nlev - 1; from64 copies the entry level's
-  // float64 correction (in r when in_r) back.  One launch each.
+  // Conversions between the coarsest level l and its float64 copy (lv64): to64
+  // copies its right-hand side, correction and coefficients, from64 the float64
+  // correction back.  One launch each.
   static int coarse_to64(fm_state* st, int l) {
     ConvSet<T, double> C{};
-    auto add = [&](const void* src, void* dst, int n) {
-      if (src && dst && C.count < CONV_MAX) {
-        C.src[C.count] = static_cast<const T*>(src);
-        C.dst[C.count] = static_cast<double*>(dst);
-        C.n[C.count] = n;
-        C.count++;
-        if (n > C.maxn) C.maxn = n;
-      }
+    C.n = st->lv[l].g.N;
+    auto add = [&](const void* src, void* dst) {
+      C.src[C.count] = static_cast<const T*>(src);
+      C.dst[C.count++] = static_cast<double*>(dst);
     };
-    const int n0 = st->lv[l].g.N;
+    const LevelBufs &F = st->lv[l], &D = st->lv64;
     for (int q = 0; q < LY::NU; ++q) {
-      add(st->lv[l].f[q], st->lv64[l].f[q], n0);
-      add(st->lv[l].e[q], st->lv64[l].e[q], n0);
+      add(F.f[q], D.f[q]);
+      add(F.e[q], D.e[q]);
     }
-    for (int k = l; k < st->nlev; ++k) {
-      const int n = st->lv[k].g.N;
-      add(st->lv[k].rk, st->lv64[k].rk, n);
-      add(st->lv[k].cr, st->lv64[k].cr, n);
-      for (int d = 0; d < LY::NOM; ++d) add(st->lv[k].om[d], st->lv64[k].om[d], n);
-      for (int d = 0; d < DIM; ++d) add(st->lv[k].cv[d], st->lv64[k].cv[d], n);
-    }
-    k_convert_set<T, double><<<dim3((C.maxn + TPB - 1) / TPB, C.count), TPB, 0, st->stream>>>(C);
+    add(F.rk, D.rk);
+    add(F.cr, D.cr);
+    for (int d = 0; d < LY::NOM; ++d) add(F.om[d], D.om[d]);
+    for (int d = 0; d < DIM; ++d) add(F.cv[d], D.cv[d]);
+    k_convert_set<T, double><<<dim3((C.n + TPB - 1) / TPB, C.count), TPB, 0, st->stream>>>(C);
     FM_LAUNCHED();
     return FM_OK;
   }
-  static int coarse_from64(fm_state* st, int l, int in_r) {
+  static int coarse_from64(fm_state* st, int l) {
     ConvSet<double, T> C{};
-    const int n0 = st->lv[l].g.N;
-    for (int q = 0; q < LY::NU; ++q) {
-      C.src[q] = static_cast<const double*>(in_r ? st->lv64[l].r[q] : st->lv64[l].e[q]);
-      C.dst[q] = static_cast<T*>(st->lv[l].e[q]);
-      C.n[q] = n0;
-    }
+    C.n = st->lv[l].g.N;
     C.count = LY::NU;
-    C.maxn = n0;
-    k_convert_set<double, T><<<dim3((n0 + TPB - 1) / TPB, C.count), TPB, 0, st->stream>>>(C);
+    for (int q = 0; q < LY::NU; ++q) {
+      C.src[q] = static_cast<const double*>(st->lv64.e[q]);
+      C.dst[q] = static_cast<T*>(st->lv[l].e[q]);
+    }
+    k_convert_set<double, T><<<dim3((C.n + TPB - 1) / TPB, C.count), TPB, 0, st->stream>>>(C);
     FM_LAUNCHED();
     return FM_OK;
   }
@@ -1125,8 +1111,8 @@ struct Solver {
       for (int q = 0; q < LY::NU; ++q) {
         ef.p[q] = L.e[q];
         of.p[q] = n > 2 ? L.e[q] : L.r[q];  // (one launch: not over the values its tiles still read)
-        b[0].p[q] = (double*)st->lv64[l].e[q];
-        b[1].p[q] = (double*)st->lv64[l].r[q];
+        b[0].p[q] = (double*)st->lv64.e[q];
+        b[1].p[q] = (double*)st->lv64.r[q];
       }
       *out_in_r = n > 2 ? 0 : 1;
       for (int it = 0, k = 0; it < n; it += 2, ++k) {
@@ -1170,7 +1156,7 @@ struct Solver {
       // colour launches of 32-thread blocks: the float64 point updates of a
       // small level spread over all multiprocessors (GB300 issues few float64
       // operations per multiprocessor and clock)
-      const Lvl<double> L64 = make_lvl_bufs<double>(st->lv64[l]);
+      const Lvl<double> L64 = make_lvl_bufs<double>(st->lv64);
       const int half = L64.g.N / 2;
       const PtK<double> K64 = make_ptk<double, DIM>(P64, L64.h);
       // (r is unused by these sweeps: what a launch's points keep for the next)
@@ -1186,7 +1172,7 @@ struct Solver {
           FM_LAUNCHED();
         }
     }
-    return coarse_from64(st, l, 0);
+    return coarse_from64(st, l);
   }
 
   static int vcycle(fm_state* st, int l, const Phys<T>& P, int* out_in_r) {
@@ -1413,31 +1399,24 @@ static size_t carve(fm_state* st, char* base) {
       }
     }
   }
-  // float64 copies of the coarse levels (mixed path, coarsest solve in
-  // float64): e, f, r, eh and the coefficients of levels small_from ..
-  // nlev - 1 (the entry level's eh stays in the float32 level: the
-  // prolongation reads it; a multi-block coarsest level's r[0] holds the
-  // CDFT chemical-potential parts of its colour launches)
-  for (int l = 0; l < MAXLEV; ++l) st->lv64[l] = LevelBufs{};
+  // Float64 copy of a coarsest level swept by itself in the mixed path: its colour
+  // launches use all of it, r[0] and r[1] for what their points keep (|u|^2's
+  // change; CDFT the chemical-potential part); its tiles e and r in turn.
+  st->lv64 = LevelBufs{};
   if (st->coarse64 && st->coarse_fused) {
-    for (int l = st->small_from; l < st->nlev; ++l) {
-      LevelBufs& B = st->lv64[l];
-      B.g = st->lv[l].g;
-      B.h = st->lv[l].h;
-      const size_t N = B.g.N;
-      for (int q = 0; q < MAXU; ++q) {
-        B.e[q] = q < st->nu ? C.take(N * d8) : nullptr;
-        B.f[q] = q < st->nu ? C.take(N * d8) : nullptr;
-        B.r[q] = q < st->nu ? C.take(N * d8) : nullptr;
-        B.eh[q] = (q < st->nu && l > st->small_from) ? C.take(N * d8) : nullptr;
-      }
-      B.rk = C.take(N * d8);
-      B.cr = C.take(N * d8);
-      for (int d = 0; d < 3; ++d) {
-        B.om[d] = d < st->nom ? C.take(N * d8) : nullptr;
-        B.cv[d] = d < st->dim ? C.take(N * d8) : nullptr;
-      }
+    LevelBufs& B = st->lv64;
+    B.g = st->lv[st->nlev - 1].g;
+    B.h = st->lv[st->nlev - 1].h;
+    const size_t N = B.g.N;
+    for (int q = 0; q < st->nu; ++q) {
+      B.e[q] = C.take(N * d8);
+      B.f[q] = C.take(N * d8);
+      B.r[q] = C.take(N * d8);
     }
+    B.rk = C.take(N * d8);
+    B.cr = C.take(N * d8);
+    for (int d = 0; d < st->nom; ++d) B.om[d] = C.take(N * d8);
+    for (int d = 0; d < st->dim; ++d) B.cv[d] = C.take(N * d8);
   }
   if (st->kind == FM_CDFT) {
     st->fft.Jhat = (double2*)C.take(N0 * sizeof(double2));
