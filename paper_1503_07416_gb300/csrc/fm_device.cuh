@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(TPB) k_inverse(const __grid_constant__ IvAll A
 
 // --------------------------------------------------------------------------
 // Point operations of one level (shared by the per-level kernels and the
-// single-block small-level V-cycle)
+// one-block float32 V-cycle of the small levels)
 // --------------------------------------------------------------------------
 template <typename T, int KIND, int DIM>
 __device__ __forceinline__ void resid_point(const Lvl<T>& L, const Phys<T>& P, const PtK<T>& K, int idx) {
@@ -677,7 +677,8 @@ __global__ void __launch_bounds__(TPB, OCC ? 3 : 1) k_smooth_keep(Lvl<double> L,
 // The same colour sweep compiled for six resident blocks per SM (at most 40
 // registers a thread instead of 64): the 3-D point update waits on its many
 // cached loads, and more warps in flight hide that latency.  The 3-D
-// autotuner times it against k_smooth per level (it spills in float64).
+// autotuner times it against k_smooth per level (float32; in float64 the choice
+// selects k_smooth_keep bounded to three blocks).
 template <typename T, int KIND, int DIM>
 __global__ void __launch_bounds__(TPB, 6) k_smooth_occ(Lvl<T> L, Phys<T> P, PtK<T> K, int color) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2422,9 +2423,9 @@ struct Resid64Out {
 // worth fixed point: a difference is one float64 instruction (19 clocks of a
 // multiprocessor), or two conversions and a rounding (~28).  The rows are formed
 // and stored one after the other: all of them at once spilled 44 registers.
-// 25.6 us a launch at 512^2 (float64 Laplacians 34.4; the form before 36.8), 83 us
-// at 1024^2 (122 before).  Bounded to three blocks a multiprocessor; to four
-// 26.3 and 82 us.
+// 24.6 us a launch at 512^2 (36.8 in float64), 85 us at 1024^2 (122); with float64
+// Laplacians alone 34.4 against 26.4 at 512^2 on the same number of blocks.  Bounded to three blocks
+// a multiprocessor.
 // TX: the tile's width (TX x TY = 256 points, 340 with the halo for 32 and 8).
 constexpr int R64_TX = 32;
 template <int TX = R64_TX>
@@ -2589,7 +2590,7 @@ __global__ void __launch_bounds__(TPB) k_update_shared64(Fields64 F, Resid64Out 
 // Float64 residual reading the shared quantities of k_shared64, its Laplacians in
 // fixed point: 45 float64 instructions a point in 3-D, 81 with them in float64.
 // The rows are formed and stored one after the other (all at once they spill 120
-// registers): 200 us at 128^3, 335 with float64 sums.
+// registers): 206 us at 128^3, 335 with float64 sums.
 template <int KIND, int DIM, typename T>
 __global__ void __launch_bounds__(TPB, 4) k_resid64_x(Fields64 F, Shared64 X, Resid64Out O, Geo G, Step64 K,
                                                    Phys<double> P, double* partials) {

@@ -1366,7 +1366,7 @@ static size_t carve(fm_state* st, char* base) {
     st->x64[q] = (st->model == FM_HYDRO && st->dim == 3 && (q < 4 || st->kind == FM_CDFT))
                      ? (double*)C.take(N0 * d8)
                      : nullptr;
-  st->partials = (double*)C.take((size_t)(st->nblk > st->nres ? st->nblk : st->nres) * 8 * d8);
+  st->partials = (double*)C.take((size_t)4 * st->sms * 8 * d8);  // (no reduction has more blocks)
   st->dscal = (double*)C.take(64 * d8);
   st->ctl = C.take(64);
   for (int l = 0; l < st->nlev; ++l) {
@@ -1592,14 +1592,15 @@ int fm_create(const fm_grid* grid, const fm_params* prm, const fm_functional* fn
   }
   const int need = (int)((st->lv[0].g.N + TPB - 1) / TPB);
   st->nblk = need < 4 * sms ? need : 4 * sms;
-  // a block a tile while four a multiprocessor hold them: counted in points, a grid
-  // 2 points wide gave each block 16 tiles one after the other (2 x 8192, us a cycle:
-  // channel 142, a block a tile 69, on narrow tiles 49; periodic 151 and 83)
+  // a block a tile while three a multiprocessor hold them, as many as are resident
+  // (512^2: 24.6 us a launch, with four 26.4; 1024^2 85.0 and 82.6).  Counted in points, a
+  // grid 2 points wide gave each block 16 tiles one after the other (2 x 8192, us a
+  // cycle: channel 142, a block a tile 69, on narrow tiles 49; periodic 151 and 83).
   st->nres = st->nblk;
   if (st->dim == 2 && st->model == FM_HYDRO) {
     const Geo& G = st->lv[0].g;
     const int tiles = st->prm.walls == FM_WALLS_Y && narrow_tiles(G) ? r64_tiles<R64_NARROW>(G) : r64_tiles(G);
-    st->nres = tiles < 4 * sms ? tiles : 4 * sms;
+    st->nres = tiles < 3 * sms ? tiles : 3 * sms;
   }
   const size_t bytes = carve(st, nullptr);
   void* arena = nullptr;
