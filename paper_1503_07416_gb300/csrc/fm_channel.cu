@@ -283,7 +283,7 @@ __device__ __forceinline__ double gv(const double* x, int i, int N, int type, co
   return i >= 0 ? v : ghost_of(v, type, i < -N ? W.ut : W.ub);
 }
 
-// omega^k, S, g^0 (kappa^0 = Lap_h rho^k) with the wall ghosts: 7.1 us at 256^2,
+// omega^k, S, g^0 (kappa^0 = Lap_h rho^k) with the wall ghosts: 6.9 us at 256^2,
 // 10.7 point by point.
 template <int TX>
 __global__ void __launch_bounds__(TPB) k_ch_prepare(Fields64 F, Geo G, Step64 K, Phys<double> P, Walls64 W) {
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(TPB) k_ch_prepare_mu(Fields64 F, Geo G, Step64
 
 // r = S - N(g) in float64 with the wall ghosts; the level-0 set-up of a
 // cycle and the block partial sums of r^2 (15.3 us a launch at 256^2 point by
-// point with the wall rows' ghosts chosen at every load, 11.2 on the periodic
+// point with the wall rows' ghosts chosen at every load, 11.0 on the periodic
 // solver's tiles, whose halo rows hold the ghosts).
 template <typename T, int TX>
 __global__ void __launch_bounds__(TPB, 4) k_ch_resid64(Fields64 F, Resid64Out O, Geo G, Step64 K, Phys<double> P,

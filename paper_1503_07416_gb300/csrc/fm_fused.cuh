@@ -1,16 +1,17 @@
 // Fused 2-D level kernels of the gradient-flow and channel solvers: one or
-// two red-black sweeps per launch on tiles in shared memory, the residual,
-// restriction and coarse right-hand side in one launch, and the V-cycle of the
-// smallest levels in one block.
+// two red-black sweeps per launch on tiles in shared memory (or a launch per
+// colour where that is the better form, see fz_tile), the residual, restriction and
+// coarse right-hand side in one launch, and the V-cycle of the smallest levels in
+// one block.
 //
 // Both solvers' levels lie in L2 and their point updates are short, so a
 // cycle's time is its number of launches: ~2.6 us each inside the step's
 // graph, 44 a cycle for the 512^2 flow (four levels) and 66 for the 256^2
-// channel (five levels) with a launch per colour, and with these kernels 17
-// and 19.  Measured, four steps: 512^2 flow 4,675 -> 3,617 us, 256^2 channel
-// 2,570 -> 1,714 us.  A policy M gives the model:
+// channel (five levels) with a launch per colour, and 16 with these kernels and the
+// injection on the norm launch.  Measured, four steps: 512^2 flow 4,672 -> 2,997 us,
+// 256^2 channel 2,463 -> 1,524 us.  A policy M gives the model:
 //   T, NU unknowns, NC coefficients read at neighbours, K level constants,
-//   W wall speeds, WALLS; coef(L, c) the c-th of them;
+//   W wall speeds, WALLS, TILED64 (see fz_tile); coef(L, c) the c-th of the coefficients;
 //   update(a, P, K, n, fc): the point update through an accessor a;
 //   apply(F, P, K, W, x, y, M): M(e) at a point of a level in global memory;
 //   apply_coarse(F, C, P, KC, W, I, J, M): M_C of the injected correction.

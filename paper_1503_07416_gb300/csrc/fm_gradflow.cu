@@ -291,7 +291,8 @@ __global__ void __launch_bounds__(TPB) k_gf_m64(GF64 F, int N, double ce) {
 
 // r = S - N(g) in float64, the level-0 set-up of a cycle (f0 = r in T, e0 =
 // 0, the coefficient density in float for the mixed path) and the block
-// partial sums of r^2 (grid-stride loop, fixed order).
+// partial sums of r^2 (grid-stride loop, fixed order).  PFC: the Laplacians in fixed
+// point, 12.9 us a launch at 512^2, 17.7 in float64.
 template <int KIND, int DIM, typename T>
 __global__ void __launch_bounds__(TPB) k_gf_resid64(GF64 F, Resid64Out O, Geo G, double ih2, double s, double alpha,
                                                     double* partials) {
