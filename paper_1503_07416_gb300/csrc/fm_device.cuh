@@ -1977,11 +1977,12 @@ struct Fields64 {
 // values of one sum, whose largest magnitude has the biased exponent emax, are
 // held as trunc(x 2^k), k chosen so that the largest has bit 58 set: those down to
 // 2^-6 of it exactly, smaller ones to 2^-58 of it.  Up to 16 of them add without
-// an error and the result is rounded once, so a sum is at least as accurate as
-// the float64 one.  The scale is each sum's own: one shared by a tile or a grid
-// saves conversions, but keeps fewer bits than float64 wherever the values are far
-// below the largest of the set (a quiet region beside a fast one, a weak velocity
-// component beside a strong one).
+// an error and the result is rounded once: it is off by half of its last place and at
+// most 2^-54 of the largest value, a float64 sum by up to half a last place at each
+// of its four or six additions.  The scale is each sum's own: one shared by a tile
+// or a grid saves conversions, but keeps fewer bits than float64 wherever the
+// values are far below the largest of the set (a quiet region beside a fast one, a
+// weak velocity component beside a strong one).
 constexpr int FIX_EMIN = 64;                   // clamp below (2^-959): bits below 2^-1017 are dropped
 constexpr unsigned FIX_TOP = 2031u << 20;      // high words from here (2^1008, or non-finite): plain float64
 
@@ -2424,8 +2425,8 @@ struct Resid64Out {
 // multiprocessor), or two conversions and a rounding (~28).  The rows are formed
 // and stored one after the other: all of them at once spilled 44 registers.
 // 24.6 us a launch at 512^2 (36.8 in float64), 85 us at 1024^2 (122); with float64
-// Laplacians alone 34.4 against 26.4 at 512^2 on the same number of blocks.  Bounded to three blocks
-// a multiprocessor.
+// Laplacians alone 34.4 against 26.4 at 512^2 on the same number of blocks.  Bounded
+// to three blocks a multiprocessor.
 // TX: the tile's width (TX x TY = 256 points, 340 with the halo for 32 and 8).
 constexpr int R64_TX = 32;
 template <int TX = R64_TX>

@@ -293,8 +293,8 @@ static Lvl<T> fz_view(Lvl<T> L, int in_r) {
 //  * float64 is bound by the busiest multiprocessor's point updates, a tile's ring
 //    among them (562 a sweep for 32 x 16, 154 for 16 x 8): tiles of at most two a
 //    multiprocessor (128^2 76 / 59 / 94), or where these are below 1.35 a point
-//    (channel 512^2 299 / 300 / 303, in the step 301 against 332; 300 x 500 186 / 185 / 229;
-//    150 x 250 79 / 87 / 98).  The flow's update reads too little for the tile to
+//    (channel 256^2 106 / 104 / 99, 512^2 299 / 300 / 303, 300 x 500 186 / 185 / 229, 150 x 250
+//    79 / 87 / 98).  The flow's update reads too little for the tile to
 //    pay once the pipe is full (M::TILED64): 128^2 44 / 39 / 55, 512^2 129 / 155 / 150.
 template <class M>
 static int fz_tile(const Geo& g, int sms) {
